@@ -129,6 +129,11 @@ class ClockSampler:
             self.proc = subprocess.Popen(["nvidia-smi", "-i", str(self.gpu), "--query-gpu=" + self.FIELDS,
                                           "--format=csv,noheader,nounits", "-lms", "200"],
                                          stdout=self.tmp, stderr=subprocess.DEVNULL)
+            # nvidia-smi takes longer to start than a small box to step: wait
+            # (at most 5 s) for its first row, so it samples from the warm-up on
+            t0 = time.monotonic()
+            while os.path.getsize(self.tmp.name) == 0 and self.proc.poll() is None and time.monotonic() - t0 < 5.0:
+                time.sleep(0.02)
         except Exception:
             self.proc = None
 
