@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(128, FISH_COL_MINB)
         if (groups == 0) return;
         const int first = I.first;
         for (int g = 0; g < groups; ++g)
-            fluid_columns<P2, false, false, LIM, true, CFLF, false, int, false>(Ab, (long long)first + 128ll * g + threadIdx.x);
+            fluid_columns<P2, false, false, LIM, true, CFLF, false, int, false>(Ab, (long long)first + 128ll * g + threadIdx.x, 0, Ab.n);
     }
 }
 
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(32 * ROWS, FISH_CT_MINB * 4 / ROWS)
         for (int g = 0; g < groups; ++g) {
             const long long q = (long long)first / ROWS + g;
             const long long ob = (q / nseg) * ROWS + (threadIdx.x >> 5);
-            ct_columns<float, LIM, true>(Ab, ob * nseg + q % nseg, threadIdx.x & 31);
+            ct_columns<float, LIM, true>(Ab, ob * nseg + q % nseg, threadIdx.x & 31, 0, Ab.n);
         }
     }
 }

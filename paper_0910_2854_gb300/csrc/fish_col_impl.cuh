@@ -26,10 +26,60 @@ template <class A_> static bool fits_int(const A_ &A)
 #endif
 }
 
-// blocks of fluid_col_kernel: one thread per column group
-template <class V> static unsigned fluid_blocks(const ColFluidArgs<typename VT<V>::S> &A)
+// Length of the segments a sweep of n cells is cut into, for `blocks` column
+// blocks of a kernel that keeps `slots` blocks on the GPU, `lone` of which
+// already run without sharing a scheduler (FP32) or an FP64 pipe.  A segment
+// of len cells costs len + `extra` march steps (its windows fill over the
+// cells before it), so the number of segments S minimises
+//   waves(blocks S) (ceil(n / S) + extra),
+// a last wave of at most `lone` blocks counting `lone_cost` of a full one.
+// Measured against every S from 1 to 64 on boxes from 32^3 to 1024^2 x 512:
+// within 3 % of the best S, e.g. L_d 95 -> 45 us at 128^3 (FP32, 4
+// segments), 666 -> 110 us at 32^3 (FP64, 16), 19.7 -> 17.6 ms at 256^3
+// (FP64, 2: less of the last wave idle), 2.95 -> 2.85 ms at 640^3 (FP32, 3).
+static inline int col_segments(int n, long long blocks, int slots, int lone, double lone_cost, int extra)
 {
-    return col_grid((long long)(A.nf / VT<V>::W) * A.no, 128);
+    double best = 1e300;
+    int len = n;
+    for (int S = 1; S <= n; ++S) {
+        const int l = (n + S - 1) / S;
+        if ((n + l - 1) / l != S) continue;  // the same length as a smaller S
+        const long long B = blocks * S;
+        const long long full = B / slots, rem = B % slots;
+        const double waves = (double)full + (rem == 0 ? 0.0 : (rem <= lone ? lone_cost : 1.0));
+        const double cost = waves * (l + extra);
+        if (cost < best * 0.999) {
+            best = cost;
+            len = l;
+        }
+        if (B > 64ll * slots) break;  // many waves: finer cuts only add steps
+    }
+    return len;
+}
+
+static inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return 152;
+    return sms;
+}
+
+// Launch fluid_col_kernel over all columns: one thread per column group, the
+// sweep in segments.
+template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF, bool NU, class IX>
+static cudaError_t fluid_run(const ColFluidArgs<typename VT<V>::S> &A, cudaStream_t s)
+{
+    constexpr int T = fluid_threads<V>();
+    const unsigned blocks = col_grid((long long)(A.nf / VT<V>::W) * A.no, T);
+    const int sms = sm_count();
+    constexpr int resident = fluid_resident<V, HSE>();
+    const int len = VT<V>::F64 ? col_segments(A.n, blocks, resident * sms, 4 * sms, 0.6, 4)
+                               : col_segments(A.n, blocks, resident * sms, sms, 0.7, 5);
+    const dim3 grid(blocks, (unsigned)((A.n + len - 1) / len));
+    fluid_col_kernel<V, HSE, GRAV, LIM, FT1, CFLF, NU, IX><<<grid, T, 0, s>>>(A, len);
+    return cudaGetLastError();
 }
 
 // (external linkage: the packed instantiations are spread over several
@@ -39,28 +89,22 @@ cudaError_t col_fluid_launch(const ColFluidArgs<typename VT<V>::S> &A, cudaStrea
 {
     if constexpr (NU) {
         if (A.cfl_min) return cudaErrorInvalidValue;
-        fluid_col_kernel<V, HSE, GRAV, LIM, FT1, false, true><<<fluid_blocks<V>(A), 128, 0, s>>>(A);
-        return cudaGetLastError();
-    }
-    // the packed FP32 kernels index with int where the box allows it
-    constexpr bool I32 = std::is_same<V, P2>::value;
-    const bool small = I32 && fits_int(A);
-    if constexpr (std::is_same<V, P2>::value && !HSE) {
-        if (A.cfl_min) {
-            if (small) fluid_col_kernel<V, HSE, GRAV, LIM, FT1, true, false, int><<<fluid_blocks<V>(A), 128, 0, s>>>(A);
-            else fluid_col_kernel<V, HSE, GRAV, LIM, FT1, true><<<fluid_blocks<V>(A), 128, 0, s>>>(A);
-            return cudaGetLastError();
+        return fluid_run<V, HSE, GRAV, LIM, FT1, false, true, long long>(A, s);
+    } else {
+        // the packed FP32 kernels index with int where the box allows it
+        constexpr bool I32 = std::is_same<V, P2>::value;
+        const bool small = I32 && fits_int(A);
+        if constexpr (I32 && !HSE) {
+            if (A.cfl_min)
+                return small ? fluid_run<V, HSE, GRAV, LIM, FT1, true, false, int>(A, s)
+                             : fluid_run<V, HSE, GRAV, LIM, FT1, true, false, long long>(A, s);
         }
-    }
-    if (A.cfl_min) return cudaErrorInvalidValue;  // only the two-column kernels carry the CFL epilogue
-    if constexpr (I32) {
-        if (small) {
-            fluid_col_kernel<V, HSE, GRAV, LIM, FT1, false, false, int><<<fluid_blocks<V>(A), 128, 0, s>>>(A);
-            return cudaGetLastError();
+        if (A.cfl_min) return cudaErrorInvalidValue;  // only the two-column kernels carry the CFL epilogue
+        if constexpr (I32) {
+            if (small) return fluid_run<V, HSE, GRAV, LIM, FT1, false, false, int>(A, s);
         }
+        return fluid_run<V, HSE, GRAV, LIM, FT1, false, false, long long>(A, s);
     }
-    fluid_col_kernel<V, HSE, GRAV, LIM, FT1><<<fluid_blocks<V>(A), 128, 0, s>>>(A);
-    return cudaGetLastError();
 }
 
 #ifndef FISH_F64_VL
@@ -141,11 +185,16 @@ template <class V, int LIM, bool FT1, bool NU = false>
 cudaError_t col_ct_launch(const ColCTArgs<typename VT<V>::S> &A, cudaStream_t s)
 {
     // one warp per 31 W columns of a row (plus a halo lane); a block takes
-    // one segment of FISH_CT_ROWS consecutive rows
+    // one segment of ct_rows() consecutive rows
     const int segc = 31 * VT<V>::W;
-    const long long blocks = (long long)((A.nf + segc - 1) / segc) * ((A.no + FISH_CT_ROWS - 1) / FISH_CT_ROWS);
+    const long long blocks = (long long)((A.nf + segc - 1) / segc) * ((A.no + ct_rows<V>() - 1) / ct_rows<V>());
+    const int sms = sm_count();
+    constexpr int resident = ct_resident<V>();
+    const int len = VT<V>::F64 ? col_segments(A.n, blocks, resident * sms, 4 * sms, 0.6, 6)
+                               : col_segments(A.n, blocks, resident * sms, sms, 0.7, 8);
+    const dim3 grid((unsigned)blocks, (unsigned)((A.n + len - 1) / len));
     // (64-bit indices: int indices measured slower for this march)
-    ct_col_kernel<V, LIM, FT1, NU><<<(unsigned)blocks, 32 * FISH_CT_ROWS, 0, s>>>(A);
+    ct_col_kernel<V, LIM, FT1, NU><<<grid, 32 * ct_rows<V>(), 0, s>>>(A, len);
     return cudaGetLastError();
 }
 

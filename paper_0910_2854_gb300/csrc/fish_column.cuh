@@ -13,9 +13,17 @@
 // The march is the paper's pipelined loop (Sec. 3) held in registers: raw
 // cell r enters, predicted cell r-1 is formed, corrected cell r-3 leaves.
 // Windows are indexed by r mod 4 (unrolled by four) so they rotate without
-// moves; the steady-state loop over interior cells carries no boundary tests,
-// ghost cells (periodic wrap or zeroth-order extrapolation, no ghost storage)
-// are handled by a short prologue and a guarded tail.
+// moves.  Ghost cells (periodic wrap or zeroth-order extrapolation, no ghost
+// storage) are an index map of the loads.
+//
+// A thread marches a segment [a, b) of its columns: the raw cells a-3 .. b+2
+// enter and the updated cells a .. b-1 leave.  One loop serves the start of a
+// segment, its interior and its end: a step evaluates every stage, and only
+// the old state's loads and the result's stores wait for the windows to fill.
+// So the code of a kernel is four copies of the step (it was 23 with separate
+// prologue, interior and tail), which a short march would otherwise fetch
+// from L2 once per step, and a box with few columns is cut into segments until
+// it fills the GPU (col_segments in fish_col_impl.cuh).
 //
 // Both operators read the current buffers and write the other ones.
 #pragma once
@@ -487,14 +495,31 @@ __device__ __forceinline__ void fload_mapped(const ColFluidArgs<typename VT<V>::
     if (A.wd) R.w = A.wd[cc];
 }
 
-// load interior cell at element offset i (no map; its lower b_d face is the
-// upper face of the previous cell, set by the caller)
-template <class V, bool GRAV, bool FT1, class IX = long long>
-__device__ __forceinline__ void fload_direct(const ColFluidArgs<typename VT<V>::S> &A,
-                                             const FCtx<typename VT<V>::S, IX> &X, IX i, FRaw<V> &R)
+// Cell of the box that raw cell c stands for (c up to four cells outside the
+// box, which may be thinner than that).
+__device__ __forceinline__ int wrap_cell(int c, int n, int bc)
+{
+    if ((unsigned)c < (unsigned)n) return c;
+    if (bc == BC_PERIODIC) {
+        while (c < 0) c += n;
+        while (c >= n) c -= n;
+        return c;
+    }
+    return c < 0 ? 0 : n - 1;
+}
+
+// Load raw cell c, the one after the cell whose raw data R holds: its lower
+// b_d face is that cell's upper one, and for the ghosts above an outflow box,
+// which copy cell n-1 as a whole, that of cell n-1.
+template <class V, bool PHI, bool FT1, bool NU, class IX = long long>
+__device__ __forceinline__ void fload_next(const ColFluidArgs<typename VT<V>::S> &A,
+                                           const FCtx<typename VT<V>::S, IX> &X, int c, FRaw<V> &R)
 {
     const auto *bfp = FT1 ? A.bt1 : A.bt2;
     const auto *bop = FT1 ? A.bt2 : A.bt1;
+    const int cc = wrap_cell(c, A.n, A.bc);
+    const IX i = X.base + (IX)cc * (IX)A.sd;
+    if (!(c >= A.n && A.bc == BC_OUTFLOW)) R.bdm = R.bd;
 #pragma unroll
     for (int k = 0; k < 5; ++k) R.u[k] = vload<V>(A.u[k], i);
     R.bd = vload<V>(A.bd, i);
@@ -502,7 +527,12 @@ __device__ __forceinline__ void fload_direct(const ColFluidArgs<typename VT<V>::
     R.bfm = __ldg(bfp + i + X.ofm);
     R.bo = vload<V>(bop, i);
     R.bom = vload<V>(bop, i + X.oom);
-    if (GRAV) R.phi = vload<V>(A.phi, i);
+    if constexpr (PHI) {
+        R.phi = vload<V>(A.phi, i);
+        if constexpr (!VT<V>::F64)
+            if (c != cc && A.bc == BC_OUTFLOW) R.phi = vb<V>(0.0f);
+    }
+    if constexpr (NU) R.w = A.wd[cc];
 }
 
 // L2 prefetch distance of the steady-state loops (cells ahead of the load)
@@ -531,16 +561,12 @@ __device__ __forceinline__ void fprefetch(const ColFluidArgs<typename VT<V>::S> 
     if (GRAV) pf_l2(A.phi + i);
 }
 
-// Stage flags of one march step.
+// Stages of a march step: the evaluation of the raw cell alone, with the
+// predictor flux behind it, or everything.
+enum : int { ST_RAW = 0, ST_FLUX = 1, ST_ALL = 2 };
+// (stage flags of the ring march)
 enum : int { ST_F1 = 1, ST_PRED = 2, ST_F2 = 4, ST_OUT = 8 };
-// Load kinds: none, interior (direct), mapped.
-enum : int { LD_NONE = 0, LD_DIRECT = 1, LD_MAPPED = 2, LD_DIRECT_PF = 3 };
 
-// One step of the march for raw cell r (K = r mod 4).  The raw data of cell
-// r is in M.R on entry (loaded by the previous step); the step loads raw
-// cell r+1 (kind LD) into M.R.  FT1: the fast axis is t1 (else t2).  NU:
-// irregular mesh along d (eq037): the cells' own widths replace h (the
-// widths of raw cells r .. r-4 ride along in M.w0 .. M.w4).
 // Operator-split gravity kick G_d(tau) of one cell (eq02512, reading C-22):
 // m_d -= tau rho dphi, E changes by the kinetic energy change; FP64 in the
 // oracle's operation order.
@@ -583,19 +609,22 @@ __device__ __forceinline__ V sg_image_dk(const ColFluidArgs<typename VT<V>::S> &
 // operator-split kicks G_d(dt/2) folded into the march (eq025111): the raw
 // cell is kicked as it is consumed, the output cell's old state before its
 // update and the result after it (reading C-22 for the kick).
-#ifndef FISH_CFL_SMEM
-#define FISH_CFL_SMEM 1   // CFL epilogue: cell-centred field from a shared-memory ring
-#endif
 // The ring of the packed kernels with the CFL epilogue (blocks of 128
 // threads): the cell-centred fields of a thread's raw cells r .. r-3, slot
 // r mod 4, component k at [(slot * 3 + k) * 128 + thread]; only the kernels
 // that use it allocate it.
 static __shared__ float2 cfl_bb_ring[4 * 3 * 128];
 
-template <class V, bool HSE, int GM, int LIM, bool FT1, bool CFLF, bool NU, int K, int ST, int LD, class IX = long long,
+// One step of the march for raw cell r (K = slot of cell r in the windows).
+// The raw data of cell r is in M.R on entry (loaded by the previous step); the
+// step loads raw cell r+1 into M.R.  a: first output cell of the segment, so
+// that cell r-3 is an output cell from r = a+3 on.  FT1: the fast axis is t1
+// (else t2).  NU: irregular mesh along d (eq037): the cells' own widths
+// replace h (the widths of raw cells r .. r-4 ride along in M.w0 .. M.w4).
+template <class V, bool HSE, int GM, int LIM, bool FT1, bool CFLF, bool NU, int K, int ST, class IX = long long,
           bool PFW = FISH_FL_PF_WARP != 0>
 __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, const FCtx<typename VT<V>::S, IX> &X,
-                                      FMarch<V> &M, int r, V lam, V lamh, V hdt, V dt, V rtwoh,
+                                      FMarch<V> &M, int r, int a, V lam, V lamh, V hdt, V dt, V rtwoh,
                                       const FPf<typename VT<V>::S, IX> &PF)
 {
     constexpr bool GRAV = GM == 1, SG = GM == 2, PHI = GM != 0;
@@ -607,7 +636,6 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
 #pragma unroll
     for (int k = 0; k < 5; ++k) ur[k] = M.R.u[k];
     bbr[0] = half * (M.R.bdm + M.R.bd);
-    const V bd_r = M.R.bd;
     const V bfc = half * (vshift_lo(M.R.bfm, M.R.bf) + M.R.bf);
     const V boc = half * (M.R.bom + M.R.bo);
     if constexpr (FT1) {
@@ -618,7 +646,7 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         bbr[2] = bfc;
     }
     const V phr = PHI ? M.R.phi : vb<V>(0.0f);  // no potential: phi = 0
-    if constexpr (CFLF && FISH_CFL_SMEM) {
+    if constexpr (CFLF) {
         // keep the cell-centred field of raw cell r for the CFL rate of its
         // update three steps later (b is unchanged by L_d)
         static_assert(VT<V>::W == 2, "the CFL epilogue is built for the packed kernels");
@@ -633,32 +661,31 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         M.w1 = M.w0;
         M.w0 = M.R.w;
     }
-    // prefetch raw cell r+1
-    if constexpr (LD == LD_DIRECT || LD == LD_DIRECT_PF) {
-        fload_direct<V, PHI, FT1, IX>(A, X, X.base + (IX)(r + 1) * (IX)A.sd, M.R);
-        if constexpr (NU) M.R.w = A.wd[r + 1];
-        M.R.bdm = bd_r;
-        if constexpr (LD == LD_DIRECT_PF) {
-            const int pf = min(r + 1 + FISH_PF_DIST, A.n - 1);
-            if constexpr (PFW) fpf_step(A, PF, pf);
-            else fprefetch<V, PHI, FT1, IX>(A, X, X.base + (IX)pf * (IX)A.sd);
-        }
-    } else if constexpr (LD == LD_MAPPED) {
-        fload_mapped<V, PHI, FT1, IX>(A, X, r + 1, M.R);
+    // load raw cell r+1
+    fload_next<V, PHI, FT1, NU, IX>(A, X, r + 1, M.R);
+    if constexpr (ST == ST_ALL) {
+        const int pf = min(r + 1 + FISH_PF_DIST, A.n - 1);
+        if constexpr (PFW) fpf_step(A, PF, pf);
+        else fprefetch<V, PHI, FT1, IX>(A, X, X.base + (IX)pf * (IX)A.sd);
     }
     // old state of the output cell o = r-3
     const int o = r - 3;
+    const bool out = ST == ST_ALL && o >= a;
     const IX io = X.base + (IX)o * (IX)A.sd;
     V un[5];
-    if constexpr ((ST & ST_OUT) != 0) {
+    if constexpr (ST == ST_ALL) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) un[k] = vload<V>(A.u[k], io);
+        for (int k = 0; k < 5; ++k) un[k] = ur[k];
+        if (out) {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) un[k] = vload<V>(A.u[k], io);
+        }
     }
     if constexpr (SG) {
         // kick of raw cell r with its centred potential difference (a ghost
         // takes its image cell's), and of the output cell's old state
         V dk;
-        if (r < 0 || r >= A.n) {
+        if (A.bc == BC_OUTFLOW && (r < 0 || r >= A.n)) {
             dk = sg_image_dk<V, IX>(A, X, r, rtwoh);
         } else if constexpr (VT<V>::F64) {
             dk = (M.R.phi - M.dprev) / (2.0 * A.h);  // phi_{r+1} - phi_{r-1}
@@ -668,17 +695,17 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         M.dprev = phr;
         sg_kick<V>(ur, dk, hdt);
         M.ph[k2] = dk;
-        if constexpr ((ST & ST_OUT) != 0) sg_kick<V>(un, M.q[(K + 1) & 3], hdt);
+        if constexpr (ST == ST_ALL) sg_kick<V>(un, M.q[(K + 1) & 3], hdt);
     }
     ceval<V>(ur, bbr, vb<V>(A.gamma), vb<V>(A.gm1), M.C[k2], M.chk);
 #pragma unroll
     for (int k = 0; k < 3; ++k) M.bb[k2][k] = bbr[k];
     if (!SG && (GRAV || HSE)) M.ph[k2] = phr;
-    if constexpr ((ST & ST_F1) != 0) {
+    if constexpr (ST >= ST_FLUX) {
         // predictor flux at (r-1, r) (eq0140 / eq0324)
         cflux1<V, HSE>(M.C[p2], M.C[k2], M.ph[p2], phr, vb<V>(A.alpha), M.F1[k2]);
     }
-    if constexpr ((ST & ST_PRED) != 0) {
+    if constexpr (ST == ST_ALL) {
         // predicted half step of cell r-1 (eq0253; source eq0254, reading C-6)
         const CCell<V> &cp = M.C[p2];
         V up[5];
@@ -711,63 +738,50 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         constexpr int s3 = (K + 3) & 3;  // slot of cell r-1
         ceval<V>(up, M.bb[p2], vb<V>(A.gamma), vb<V>(A.gm1), M.P[s3], M.chk);
         if (PHI || HSE) M.q[s3] = M.ph[p2];
-        if constexpr ((ST & ST_F2) != 0) {
-            // corrector flux at (r-3, r-2) from predicted cells r-4 .. r-1 (eq0230)
-            constexpr int s0 = K & 3, s1 = (K + 1) & 3, s2 = (K + 2) & 3;
-            cflux2<V, HSE, LIM, NU>(M.P[s0], M.P[s1], M.P[s2], M.P[s3], M.q[s0], M.q[s1], M.q[s2], M.q[s3],
-                                    M.F2[k2], A.lim, vb<V>(M.w4), vb<V>(M.w3), vb<V>(M.w2), vb<V>(M.w1));
-            if constexpr ((ST & ST_OUT) != 0) {
-                V lo = lam;
-                if constexpr (NU) {
-                    if constexpr (VT<V>::F64) lo = dt / M.w3;
-                    else lo = vdiv(dt, vb<V>(M.w3));
-                }
+        // corrector flux at (r-3, r-2) from predicted cells r-4 .. r-1 (eq0230)
+        constexpr int s0 = K & 3, s1 = (K + 1) & 3, s2 = (K + 2) & 3;
+        if (!VT<V>::F64 || r >= a + 2)  // (FP64, bound by its pipe, skips the fluxes no output cell uses)
+        cflux2<V, HSE, LIM, NU>(M.P[s0], M.P[s1], M.P[s2], M.P[s3], M.q[s0], M.q[s1], M.q[s2], M.q[s3], M.F2[k2],
+                                A.lim, vb<V>(M.w4), vb<V>(M.w3), vb<V>(M.w2), vb<V>(M.w1));
+        V lo = lam;
+        if constexpr (NU) {
+            if constexpr (VT<V>::F64) lo = dt / M.w3;
+            else lo = vdiv(dt, vb<V>(M.w3));
+        }
 #pragma unroll
-                for (int k = 0; k < 5; ++k) {
-                    if constexpr (VT<V>::F64) un[k] = un[k] - lo * (M.F2[k2][k] - M.F2[p2][k]);
-                    else un[k] = vfma(-lo, M.F2[k2][k] - M.F2[p2][k], un[k]);
-                }
-                if (GRAV) {
-                    // corrector source from the predicted state (eq0255)
-                    V dphi;
-                    if constexpr (NU) {
-                        const V span = vb<V>(0.5f) * vb<V>(M.w4) + vb<V>(M.w3) + vb<V>(0.5f) * vb<V>(M.w2);
-                        if constexpr (VT<V>::F64) dphi = (M.q[s2] - M.q[s0]) / span;
-                        else dphi = vdiv(M.q[s0] + M.q[s1], span);
-                    } else if constexpr (VT<V>::F64) {
-                        dphi = (M.q[s2] - M.q[s0]) / (2.0 * A.h);
-                    } else {
-                        dphi = (M.q[s0] + M.q[s1]) * rtwoh;
-                    }
-                    un[1] = un[1] - dt * M.P[s1].u[0] * dphi;
-                    un[4] = un[4] - dt * M.P[s1].u[1] * dphi;
-                }
-                if constexpr (SG) sg_kick<V>(un, M.q[s1], hdt);  // output cell: second half kick
+        for (int k = 0; k < 5; ++k) {
+            if constexpr (VT<V>::F64) un[k] = un[k] - lo * (M.F2[k2][k] - M.F2[p2][k]);
+            else un[k] = vfma(-lo, M.F2[k2][k] - M.F2[p2][k], un[k]);
+        }
+        if (GRAV) {
+            // corrector source from the predicted state (eq0255)
+            V dphi;
+            if constexpr (NU) {
+                const V span = vb<V>(0.5f) * vb<V>(M.w4) + vb<V>(M.w3) + vb<V>(0.5f) * vb<V>(M.w2);
+                if constexpr (VT<V>::F64) dphi = (M.q[s2] - M.q[s0]) / span;
+                else dphi = vdiv(M.q[s0] + M.q[s1], span);
+            } else if constexpr (VT<V>::F64) {
+                dphi = (M.q[s2] - M.q[s0]) / (2.0 * A.h);
+            } else {
+                dphi = (M.q[s0] + M.q[s1]) * rtwoh;
+            }
+            un[1] = un[1] - dt * M.P[s1].u[0] * dphi;
+            un[4] = un[4] - dt * M.P[s1].u[1] * dphi;
+        }
+        if constexpr (SG) sg_kick<V>(un, M.q[s1], hdt);  // output cell: second half kick
+        if (out) {
 #pragma unroll
-                for (int k = 0; k < 5; ++k) vstore(A.uo[k], io, un[k]);
-                if constexpr (CFLF) {
-                    // CFL rate of the updated cell with its cell-centred field,
-                    // formed when the cell entered as raw cell o = r-3 (slot
-                    // (r-3) mod 4 of the ring)
-                    V bc[3];
-                    if constexpr (FISH_CFL_SMEM) {
-                        const int t = threadIdx.x & 127;
+            for (int k = 0; k < 5; ++k) vstore(A.uo[k], io, un[k]);
+            if constexpr (CFLF) {
+                // CFL rate of the updated cell with its cell-centred field,
+                // formed when the cell entered as raw cell o = r-3 (slot
+                // (r-3) mod 4 of the ring)
+                V bc[3];
+                const int t = threadIdx.x & 127;
 #pragma unroll
-                        for (int k = 0; k < 3; ++k) bc[k].v = cfl_bb_ring[(((K + 1) & 3) * 3 + k) * 128 + t];
-                    } else {
-                        const auto *bfp = FT1 ? A.bt1 : A.bt2;
-                        const auto *bop = FT1 ? A.bt2 : A.bt1;
-                        const IX iom = X.base + (IX)(o > 0 ? o - 1 : gmap(-1, A.n, A.bc)) * (IX)A.sd;
-                        bc[0] = half * (vload<V>(A.bd, iom) + vload<V>(A.bd, io));
-                        const V bfv = vload<V>(bfp, io);
-                        const V bfc = half * (vshift_lo(__ldg(bfp + io + X.ofm), bfv) + bfv);
-                        const V boc = half * (vload<V>(bop, io + X.oom) + vload<V>(bop, io));
-                        bc[FT1 ? 1 : 2] = bfc;
-                        bc[FT1 ? 2 : 1] = boc;
-                    }
-                    const V rh[3] = {vb<V>(A.rh[0]), vb<V>(A.rh[1]), vb<V>(A.rh[2])};
-                    M.cflr = vmax(M.cflr, cfl_rate3<V>(un, bc, vb<V>(A.gamma), vb<V>(A.gm1), rh));
-                }
+                for (int k = 0; k < 3; ++k) bc[k].v = cfl_bb_ring[(((K + 1) & 3) * 3 + k) * 128 + t];
+                const V rh[3] = {vb<V>(A.rh[0]), vb<V>(A.rh[1]), vb<V>(A.rh[2])};
+                M.cflr = vmax(M.cflr, cfl_rate3<V>(un, bc, vb<V>(A.gamma), vb<V>(A.gm1), rh));
             }
         }
     }
@@ -781,37 +795,15 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
 #define FISH_COL_MINB1 3   // one-column FP32 kernels
 #endif
 
-// L_d over all columns.  The prologue runs raw cells -3 .. 2 (K = 1, 2, 3,
-// 0, 1, 2); boxes with n < 8 load everything through the map.
-template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF, bool NU, int PLD, class IX = long long,
-          bool PFW = FISH_FL_PF_WARP != 0>
-__device__ __forceinline__ void fprologue(const ColFluidArgs<typename VT<V>::S> &A,
-                                          const FCtx<typename VT<V>::S, IX> &X, FMarch<V> &M, V lam, V lamh, V hdt,
-                                          V dt, V rtwoh, const FPf<typename VT<V>::S, IX> &PF)
-{
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, 0, LD_MAPPED, IX, PFW>(A, X, M, -3, lam, lamh, hdt, dt, rtwoh, PF);
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_F1, LD_MAPPED, IX, PFW>(A, X, M, -2, lam, lamh, hdt, dt, rtwoh, PF);
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ST_F1 | ST_PRED, PLD, IX, PFW>(A, X, M, -1, lam, lamh, hdt, dt, rtwoh, PF);
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ST_F1 | ST_PRED, PLD, IX, PFW>(A, X, M, 0, lam, lamh, hdt, dt, rtwoh, PF);
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_F1 | ST_PRED, PLD, IX, PFW>(A, X, M, 1, lam, lamh, hdt, dt, rtwoh, PF);
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_F1 | ST_PRED | ST_F2, PLD, IX, PFW>(A, X, M, 2, lam, lamh, hdt, dt, rtwoh, PF);
-}
-
-#ifndef FISH_COL_MINB
-#define FISH_COL_MINB 2
-#endif
-#ifndef FISH_COL_MINB1
-#define FISH_COL_MINB1 3   // one-column FP32 kernels
-#endif
-
-// The march of thread cid (column group cid of the box described by A).
+// The march of thread cid (column group cid of the box described by A) over
+// the output cells a .. b-1.
 // PFW: L2 prefetch of the next cells by one instruction per warp over the
 // warp's span of its first row (the single-box sweeps, whose rows hold a
 // multiple of 32 column groups), or per lane and field (the batch, whose
 // short rows leave warps that straddle two rows)
 template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF, bool NU = false, class IX = long long,
           bool PFW = FISH_FL_PF_WARP != 0>
-__device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>::S> &A, long long cid)
+__device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>::S> &A, long long cid, int a, int b)
 {
     using S = typename VT<V>::S;
     constexpr int W = VT<V>::W;
@@ -841,40 +833,47 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     const V lamh = vb<V>(S(dtd / (2.0 * A.h)));
     const V hdt = vb<V>(S(0.5 * dtd));
     const V rtwoh = vb<V>(S(1.0 / (2.0 * A.h)));
-    const int n = A.n;
 
     FMarch<V> M;
     checks_init(M.chk);
-    M.cflr = vb<V>(0.0f);
-    M.phm2 = vb<V>(0.0f);
-    M.ph[0] = M.ph[1] = vb<V>(0.0f);
+    const V zero = vb<V>(0.0f);
+    M.cflr = M.phm2 = M.dprev = M.ph[0] = M.ph[1] = zero;
     M.w0 = M.w1 = M.w2 = M.w3 = M.w4 = typename VT<V>::S(1);
-    M.dprev = vb<V>(0.0f);
-    fload_mapped<V, GRAV != 0, FT1, IX>(A, X, -3, M.R);
-    constexpr int ALL = ST_F1 | ST_PRED | ST_F2 | ST_OUT;
-    int r = 3;
-    if (n >= 8) {
-        fprologue<V, HSE, GRAV, LIM, FT1, CFLF, NU, LD_DIRECT, IX, PFW>(A, X, M, lam, lamh, hdt, dt, rtwoh, PF);
-        // steady state: the four steps r .. r+3 prefetch interior cells
-#pragma unroll 1
-        for (; r + 4 <= n - 1; r += 4) {
-            fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ALL, LD_DIRECT_PF, IX, PFW>(A, X, M, r, lam, lamh, hdt, dt, rtwoh, PF);
-            fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ALL, LD_DIRECT_PF, IX, PFW>(A, X, M, r + 1, lam, lamh, hdt, dt, rtwoh, PF);
-            fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ALL, LD_DIRECT_PF, IX, PFW>(A, X, M, r + 2, lam, lamh, hdt, dt, rtwoh, PF);
-            fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ALL, LD_DIRECT_PF, IX, PFW>(A, X, M, r + 3, lam, lamh, hdt, dt, rtwoh, PF);
-        }
-    } else {
-        fprologue<V, HSE, GRAV, LIM, FT1, CFLF, NU, LD_MAPPED, IX, PFW>(A, X, M, lam, lamh, hdt, dt, rtwoh, PF);
+    // the windows behind the first output cell are zero until they fill: the
+    // fluxes formed from them are not used
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        M.q[i] = zero;
+        M.P[i].d = M.P[i].p = M.P[i].cs = M.P[i].cf = M.P[i].vn = zero;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) M.P[i].u[k] = M.P[i].F[k] = M.F2[i & 1][k] = zero;
     }
-    // tail: raw cells r .. n+2 (r = 3 mod 4, at most seven), loads through
-    // the map (harmless beyond n+2)
-    if (r <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ALL, LD_MAPPED, IX, PFW>(A, X, M, r, lam, lamh, hdt, dt, rtwoh, PF);
-    if (r + 1 <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ALL, LD_MAPPED, IX, PFW>(A, X, M, r + 1, lam, lamh, hdt, dt, rtwoh, PF);
-    if (r + 2 <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ALL, LD_MAPPED, IX, PFW>(A, X, M, r + 2, lam, lamh, hdt, dt, rtwoh, PF);
-    if (r + 3 <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ALL, LD_MAPPED, IX, PFW>(A, X, M, r + 3, lam, lamh, hdt, dt, rtwoh, PF);
-    if (r + 4 <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ALL, LD_MAPPED, IX, PFW>(A, X, M, r + 4, lam, lamh, hdt, dt, rtwoh, PF);
-    if (r + 5 <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ALL, LD_MAPPED, IX, PFW>(A, X, M, r + 5, lam, lamh, hdt, dt, rtwoh, PF);
-    if (r + 6 <= n + 2) fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ALL, LD_NONE, IX, PFW>(A, X, M, r + 6, lam, lamh, hdt, dt, rtwoh, PF);
+    fload_mapped<V, GRAV != 0, FT1, IX>(A, X, a - 3, M.R);
+    if constexpr (GRAV == 2) {
+        // potential data of the cell before the first (its centred difference)
+        FRaw<V> R0;
+        fload_mapped<V, true, FT1, IX>(A, X, a - 4, R0);
+        M.dprev = R0.phi;
+    }
+    if constexpr (PFW) {
+        // the first cells, so that their loads do not each wait for memory
+#pragma unroll
+        for (int c = -2; c < FISH_PF_DIST; ++c) fpf_step(A, PF, max(min(a + c, A.n - 1), 0));
+    }
+    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_RAW, IX, PFW>(A, X, M, a - 3, a, lam, lamh, hdt, dt, rtwoh, PF);
+    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_FLUX, IX, PFW>(A, X, M, a - 2, a, lam, lamh, hdt, dt, rtwoh, PF);
+    const int last = b + 2;
+#pragma unroll 1
+    for (int r = a - 1;; r += 4) {
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ST_ALL, IX, PFW>(A, X, M, r, a, lam, lamh, hdt, dt, rtwoh, PF);
+        if (r >= last) break;
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ST_ALL, IX, PFW>(A, X, M, r + 1, a, lam, lamh, hdt, dt, rtwoh, PF);
+        if (r + 1 >= last) break;
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_ALL, IX, PFW>(A, X, M, r + 2, a, lam, lamh, hdt, dt, rtwoh, PF);
+        if (r + 2 >= last) break;
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_ALL, IX, PFW>(A, X, M, r + 3, a, lam, lamh, hdt, dt, rtwoh, PF);
+        if (r + 3 >= last) break;
+    }
     const unsigned fl = checks_flags(M.chk);
     if (fl) atomicOr(A.flags, fl);
     if constexpr (CFLF) {
@@ -896,11 +895,25 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     }
 }
 
-template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF = false, bool NU = false, class IX = long long>
-__global__ void __launch_bounds__(128, VT<V>::F64 ? 1 : (VT<V>::W == 2 || HSE ? FISH_COL_MINB : FISH_COL_MINB1))
-    fluid_col_kernel(const ColFluidArgs<typename VT<V>::S> A)
+// Threads of a block.  FP64 is bound by the FP64 pipe of each SM quarter,
+// which one warp nearly fills, so its blocks are single warps that spread
+// evenly (32^3, 256 warps: 136 us per L_d with one-warp blocks, 151 us with
+// four-warp blocks, 719 us with the columns uncut).
+template <class V> constexpr int fluid_threads() { return VT<V>::F64 ? 32 : 128; }
+// Blocks per SM the kernels are compiled for.
+template <class V, bool HSE> constexpr int fluid_resident()
 {
-    fluid_columns<V, HSE, GRAV, LIM, FT1, CFLF, NU, IX>(A, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+    return VT<V>::F64 ? 8 : (VT<V>::W == 2 || HSE ? FISH_COL_MINB : FISH_COL_MINB1);
+}
+
+// Grid: column blocks x segments of `len` cells.
+template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF = false, bool NU = false, class IX = long long>
+__global__ void __launch_bounds__(fluid_threads<V>(), fluid_resident<V, HSE>())
+    fluid_col_kernel(const ColFluidArgs<typename VT<V>::S> A, int len)
+{
+    const int a = blockIdx.y * len;
+    fluid_columns<V, HSE, GRAV, LIM, FT1, CFLF, NU, IX>(A, (long long)blockIdx.x * blockDim.x + threadIdx.x, a,
+                                                        min(A.n, a + len));
 }
 
 // ---------------------------------------------------------------------------
@@ -935,8 +948,8 @@ template <class V, bool NU> __device__ __forceinline__ V cedge(V va, V vb_, V wa
 // field bf.  With OUT, bnew receives the updated face field of cell s-4 and
 // f[K & 1] holds the corrector flux at (s-4)'.  NU: irregular mesh along d
 // (widths in cw, eq037 and reading C-25/C-27; dt for the per-cell factors).
-template <class V, int LIM, int K, bool PRE1, bool PRE2, bool CORR, bool OUT, bool NU = false>
-__device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V &bnew, int lim,
+template <class V, int LIM, int K, bool OUT, bool NU = false>
+__device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V &bnew, int lim, bool live,
                                       const CWid<V> &cw = CWid<V>(), V dt = V())
 {
     constexpr int k1 = (K + 3) & 3, k2 = (K + 2) & 3, kp = (K + 1) & 3;
@@ -946,14 +959,14 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
     if constexpr (VT<V>::F64) vh = 0.25 * (vt + 2.0 * P.vt[k1] + P.vt[k2]);
     else vh = vb<V>(0.25f) * (vfma(vb<V>(2.0f), P.vt[k1], vt) + P.vt[k2]);
     P.vh[k1] = vh;
-    P.w[o] = vh * P.bf[k1];
-    if constexpr (PRE1) {
+    P.w[o] = vmul(vh, P.bf[k1]);
+    {
         // first-order upwind flux at (s-2)' (eq0363, edge velocity eq0364;
         // tie v = 0 takes the right cell, reading C-7)
         const V vbar = cedge<V, NU>(P.vh[k2], vh, cw.w2, cw.w1);
         P.f1[e] = vsel_pos(vbar, P.w[e], P.w[o]);
     }
-    if constexpr (PRE2) {
+    {
         // predictor half step of the face field at s-2
         V bp;
         V lh = lamh;
@@ -963,9 +976,9 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         }
         if constexpr (VT<V>::F64) bp = P.bf[k2] - lh * (P.f1[e] - P.f1[o]);
         else bp = vfma(-lh, P.f1[e] - P.f1[o], P.bf[k2]);
-        P.wp[k2] = P.vh[k2] * bp;
+        P.wp[k2] = vmul(P.vh[k2], bp);
     }
-    if constexpr (CORR) {
+    if (!VT<V>::F64 || live) {
         // corrector flux at q' = (s-4)': piecewise-linear TVD about the
         // upwind cell (reading C-10)
         const V vbar = cedge<V, NU>(P.vh[K], P.vh[kp], cw.w4, cw.w3);
@@ -1047,13 +1060,15 @@ template <class V> __device__ __forceinline__ void fixy_(V &a, bool f)
     }
 }
 
-// load the raw inputs of cell s (MAPPED: s through the boundary map; OUTLD:
-// also b_d of the output cell s-4, which is interior)
-template <class V, bool MAPPED, bool OUTLD, bool NU, class IX = long long>
+// Load the raw inputs of cell s (any s up to four cells outside the box) and
+// b_d of the cell s-4 that leaves when s enters (clamped to the box: before
+// the segment's first output cell, and in the load behind its last step, it is
+// not used).
+template <class V, bool NU, class IX = long long>
 __device__ __forceinline__ void ctload(const ColCTArgs<typename VT<V>::S> &A, const CTCtx<typename VT<V>::S, IX> &X,
                                        int s, CTRaw<V> &R)
 {
-    const int sm = MAPPED ? gmap(s, A.n, A.bc) : s;
+    const int sm = wrap_cell(s, A.n, A.bc);
     const IX i = X.base + (IX)sm * (IX)A.sd;
     if constexpr (NU) R.w = A.wd[sm];  // a ghost has the width of its image (reading C-23)
     R.rc = vload<V>(A.rho, i);
@@ -1073,8 +1088,7 @@ __device__ __forceinline__ void ctload(const ColCTArgs<typename VT<V>::S> &A, co
             fixy_(R.rm, true); fixy_(R.mm, true); fixy_(R.bF, true); fixy_(R.bO, true); fixy_(R.bOm, true);
         }
     }
-    // (the tail's last step loads one cell past the march: keep its index in range)
-    if constexpr (OUTLD) R.bdo = vload<V>(A.bd, X.base + (IX)(MAPPED ? min(s - 4, A.n - 1) : s - 4) * (IX)A.sd);
+    R.bdo = vload<V>(A.bd, X.base + (IX)max(min(s - 4, A.n - 1), 0) * (IX)A.sd);
 }
 
 // prefetch into L2 the fields of interior cell i (the neighbour rows too
@@ -1120,39 +1134,6 @@ template <class V> struct CTMarch {
     CWid<V> cw;             // irregular mesh: widths along d of cells s-1 .. s-5
 };
 
-// L2 prefetch of one cell of a warp's march with a single instruction: lane
-// l < 30 takes field row l / 3 of the ten the march reads (rho, m_d of this
-// row and the rows below / above, b_o of the row below, b_f, b_o, b_d of this
-// row) and the (l % 3)-th 128-byte line of the warp's span of that row.
-#ifndef FISH_CT_PF_WARP
-#define FISH_CT_PF_WARP 0   // measured slower than the per-field prefetch for this march
-#endif
-template <class S, class IX> struct CTPf {
-    const S *p;   // the lane's line in cell 0 (nullptr: lane idle); cell c: p + c * sd
-};
-
-template <class S, class IX>
-__device__ __forceinline__ void ctpf_setup(const ColCTArgs<S> &A, const CTCtx<S, IX> &X0, int c0, int c1, int lane,
-                                           CTPf<S, IX> &P)
-{
-    P.p = nullptr;
-    if (lane >= 30) return;
-    const int r = lane / 3;
-    // rows 0..5: rho, m_d of this row, the row below, the row above; 6: b_o
-    // below; 7, 8, 9: b_f, b_o, b_d of this row (selects, no local array)
-    const S *f = r == 6 || r == 8 ? A.bo : (r == 7 ? A.bf : (r == 9 ? A.bd : ((r & 1) ? A.md : A.rho)));
-    const IX ro = (r == 2 || r == 3 || r == 6) ? X0.oom : ((r == 4 || r == 5) ? X0.oop : (IX)0);
-    const IX r0 = X0.base + ro + (IX)c0;
-    const IX line = (r0 & ~(IX)31) + (IX)(32 * (lane % 3));
-    if (line <= X0.base + ro + (IX)c1) P.p = f + line;
-}
-
-template <class S, class IX>
-__device__ __forceinline__ void ctpf_step(const ColCTArgs<S> &A, const CTPf<S, IX> &P, int s)
-{
-    if (P.p) pf_l2(P.p + (IX)s * (IX)A.sd);
-}
-
 template <class V> __device__ __forceinline__ V shfl_up1(V a)
 {
     if constexpr (VT<V>::W == 2) return {make_float2(__shfl_up_sync(0xffffffffu, a.v.x, 1),
@@ -1160,17 +1141,13 @@ template <class V> __device__ __forceinline__ V shfl_up1(V a)
     else return __shfl_up_sync(0xffffffffu, a, 1);
 }
 
-// Load kinds of a CT step (for cell s+1): none, interior, interior with L2
-// prefetch, through the map.
-enum : int { CL_NONE = 0, CL_DIRECT = 1, CL_DIRECT_PF = 2, CL_MAPPED = 3 };
-
-// One cell s of the CT march (K = s mod 4); the raw inputs of s are in M.R.
-// Next loads cell s+1 (kind LD; NOUT: with b_d of cell s-3 for its output).
-template <class V, int LIM, bool FT1, bool NU, int K, bool PRE1, bool PRE2, bool CORR, bool OUT, int LD, bool NOUT,
-          class IX = long long>
+// One cell s of the CT march (K = slot of cell s in the windows); the raw
+// inputs of s are in M.R, the step loads those of s+1.  a: first output cell of
+// the segment, so that cell s-4 is an output cell from s = a+4 on (the stages
+// before work on windows that are still zero and their results are not used).
+template <class V, int LIM, bool FT1, bool NU, int K, class IX = long long>
 __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, const CTCtx<typename VT<V>::S, IX> &X,
-                                       CTMarch<V> &M, int s, V lamh, V lam, V lamf, V lamo, V dt,
-                                       const CTPf<typename VT<V>::S, IX> &PF)
+                                       CTMarch<V> &M, int s, int a, V lamh, V lam, V lamf, V lamo, V dt)
 {
     // widths of cells s .. s-5 for this step (the width of cell s arrived
     // with its raw inputs)
@@ -1192,16 +1169,8 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
     const V bF = M.R.bF, bO = M.R.bO, bOm = M.R.bOm;
     const V bdo = M.R.bdo;
     // load cell s+1
-    if constexpr (LD == CL_DIRECT || LD == CL_DIRECT_PF) {
-        ctload<V, false, NOUT, NU, IX>(A, X, s + 1, M.R);
-        if constexpr (LD == CL_DIRECT_PF) {
-            const int pfc = min(s + 1 + FISH_CT_PF_DIST, A.n - 1);
-            if constexpr (FISH_CT_PF_WARP) ctpf_step(A, PF, pfc);
-            else ctprefetch<V, IX>(A, X, X.base + (IX)pfc * (IX)A.sd);
-        }
-    } else if constexpr (LD == CL_MAPPED) {
-        ctload<V, true, NOUT, NU, IX>(A, X, s + 1, M.R);
-    }
+    ctload<V, NU, IX>(A, X, s + 1, M.R);
+    ctprefetch<V, IX>(A, X, X.base + (IX)max(min(s + 1 + FISH_CT_PF_DIST, A.n - 1), 0) * (IX)A.sd);
     const V half = vb<V>(0.5f);
     // face velocities (eq0361): the mean of the two cells across the face,
     // or on an irregular mesh their linear interpolation to it (reading C-27)
@@ -1220,19 +1189,21 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
         vtOm = vdiv(vfma(V(X.woa), vom, V(X.wom) * vc), V(X.wom + X.woa));
     }
     V nF, nO, dummy;
+    // (FP64, bound by its pipe, skips the corrector until its fluxes are used)
+    const bool live = s >= a + 3;
     constexpr bool PK = ct_packs<V, NU>();
     if constexpr (PK) {
         P2 n2;
-        cface<P2, LIM, K, PRE1, PRE2, CORR, OUT, false>(M.PFO, P2{make_float2(vtF, vtO)}, P2{make_float2(bF, bO)},
-                                                        vb<P2>(lamh), vb<P2>(lam), n2, A.lim);
+        cface<P2, LIM, K, true, false>(M.PFO, P2{make_float2(vtF, vtO)}, P2{make_float2(bF, bO)}, vb<P2>(lamh),
+                                       vb<P2>(lam), n2, A.lim, live);
         nF = n2.v.x;
         nO = n2.v.y;
     } else {
-        cface<V, LIM, K, PRE1, PRE2, CORR, OUT, NU>(M.PF, vtF, bF, lamh, lam, nF, A.lim, M.cw, dt);
-        cface<V, LIM, K, PRE1, PRE2, CORR, OUT, NU>(M.PO, vtO, bO, lamh, lam, nO, A.lim, M.cw, dt);
+        cface<V, LIM, K, true, NU>(M.PF, vtF, bF, lamh, lam, nF, A.lim, live, M.cw, dt);
+        cface<V, LIM, K, true, NU>(M.PO, vtO, bO, lamh, lam, nO, A.lim, live, M.cw, dt);
     }
-    cface<V, LIM, K, PRE1, PRE2, CORR, false, NU>(M.POm, vtOm, bOm, lamh, lam, dummy, A.lim, M.cw, dt);
-    if constexpr (OUT) {
+    cface<V, LIM, K, false, NU>(M.POm, vtOm, bOm, lamh, lam, dummy, A.lim, live, M.cw, dt);
+    {
         constexpr int e = K & 1;
         // edge flux of the fast-axis face below: the upper pencil of the lane beneath
         V fup, fpo;
@@ -1247,7 +1218,7 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
         V fdn;
         if constexpr (VT<V>::W == 2) fdn = vshift_lo(sh.v.y, fup);
         else fdn = sh;
-        if (X.active) {
+        if (X.active && s - 4 >= a) {
             const IX io = X.base + (IX)(s - 4) * (IX)A.sd;
             vstore(A.bfo, io, nF);
             vstore(A.boo, io, nO);
@@ -1267,17 +1238,15 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
 #ifndef FISH_CT_MINB
 #define FISH_CT_MINB 4
 #endif
-#ifndef FISH_CT_MINB2
-#define FISH_CT_MINB2 1   // FP64 and two-column CT blocks per SM (register bound)
-#endif
 
 // B_d over all columns (eq0350 advection of the transverse components,
 // eq0360 constraint update of b_d from the same edge fluxes).  Every lane of
 // a warp takes the same steps (shuffles); lanes without columns of their
 // own repeat a valid column and store nothing.
-// The march of warp gw (31 W columns of one row) of the box described by A.
+// The march of warp gw (31 W columns of one row) of the box described by A
+// over the output cells a .. b-1.
 template <class V, int LIM, bool FT1, bool NU = false, class IX = long long>
-__device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A, long long gw, int lane)
+__device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A, long long gw, int lane, int a, int b)
 {
     using S = typename VT<V>::S;
     constexpr int W = VT<V>::W;
@@ -1304,16 +1273,6 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
     X.ofp = (IX)(cfp - cb);
     X.oom = (IX)(gmap(ob - 1, A.no, A.bc) - ob) * (IX)A.so;
     X.oop = (IX)(gmap(ob + 1, A.no, A.bc) - ob) * (IX)A.so;
-    // per-warp L2 prefetch: the span of physical columns the warp reads
-    // (halo column to the column above the last lane's), clipped to the row
-    CTPf<S, IX> PFw;
-    {
-        CTCtx<S, IX> X0 = X;
-        X0.base = (IX)A.off + (IX)ob * (IX)A.so;
-        const int c0 = max(seg * SEGC - W, 0);
-        const int c1 = min(seg * SEGC + SEGC, A.nf - 1);
-        ctpf_setup(A, X0, c0, c1, lane, PFw);
-    }
     const double dtd = *A.dt;
     const V dtv = vb<V>(S(dtd));
     const V lamh = vb<V>(S(dtd / (2.0 * A.h)));
@@ -1332,7 +1291,6 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
         lamf = vb<V>(S(dtd / (double)X.wfa));
         lamo = vb<V>(S(dtd / (double)X.woa));
     }
-    const int n = A.n;
     CTMarch<V> M;
     {
         CFace<V> z;
@@ -1346,64 +1304,41 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
         z2.w[0] = z2.w[1] = z2.f1[0] = z2.f1[1] = z2.f[0] = z2.f[1] = vb<P2>(0.0f);
         M.PFO = z2;
     }
-    M.R.bdo = vb<V>(0.0f);
     M.cw.w0 = M.cw.w1 = M.cw.w2 = M.cw.w3 = M.cw.w4 = M.cw.w5 = vb<V>(1.0f);
-    ctload<V, true, false, NU, IX>(A, X, -4, M.R);
-    // prologue s = -4 .. 3 (stages switch on at -1, 0, 3); cells 0 .. 3 are
-    // loaded directly when n >= 4
-    ctstep<V, LIM, FT1, NU, 0, false, false, false, false, CL_MAPPED, false, IX>(A, X, M, -4, lamh, lam, lamf, lamo, dtv, PFw);
-    ctstep<V, LIM, FT1, NU, 1, false, false, false, false, CL_MAPPED, false, IX>(A, X, M, -3, lamh, lam, lamf, lamo, dtv, PFw);
-    ctstep<V, LIM, FT1, NU, 2, false, false, false, false, CL_MAPPED, false, IX>(A, X, M, -2, lamh, lam, lamf, lamo, dtv, PFw);
-    int s = 4;
-    if (n >= 8) {
-        ctstep<V, LIM, FT1, NU, 3, true, false, false, false, CL_DIRECT, false, IX>(A, X, M, -1, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 0, true, true, false, false, CL_DIRECT, false, IX>(A, X, M, 0, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 1, true, true, false, false, CL_DIRECT, false, IX>(A, X, M, 1, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 2, true, true, false, false, CL_DIRECT, false, IX>(A, X, M, 2, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 3, true, true, true, false, CL_DIRECT, true, IX>(A, X, M, 3, lamh, lam, lamf, lamo, dtv, PFw);
-        // steady state: the four steps s .. s+3 load interior cells s+1 .. s+4
+    ctload<V, NU, IX>(A, X, a - 4, M.R);
+    const int last = b + 3;
 #pragma unroll 1
-        for (; s + 4 <= n - 1; s += 4) {
-            ctstep<V, LIM, FT1, NU, 0, true, true, true, true, CL_DIRECT_PF, true, IX>(A, X, M, s, lamh, lam, lamf, lamo, dtv, PFw);
-            ctstep<V, LIM, FT1, NU, 1, true, true, true, true, CL_DIRECT_PF, true, IX>(A, X, M, s + 1, lamh, lam, lamf, lamo, dtv, PFw);
-            ctstep<V, LIM, FT1, NU, 2, true, true, true, true, CL_DIRECT_PF, true, IX>(A, X, M, s + 2, lamh, lam, lamf, lamo, dtv, PFw);
-            ctstep<V, LIM, FT1, NU, 3, true, true, true, true, CL_DIRECT_PF, true, IX>(A, X, M, s + 3, lamh, lam, lamf, lamo, dtv, PFw);
-        }
-    } else {
-        ctstep<V, LIM, FT1, NU, 3, true, false, false, false, CL_MAPPED, false, IX>(A, X, M, -1, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 0, true, true, false, false, CL_MAPPED, false, IX>(A, X, M, 0, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 1, true, true, false, false, CL_MAPPED, false, IX>(A, X, M, 1, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 2, true, true, false, false, CL_MAPPED, false, IX>(A, X, M, 2, lamh, lam, lamf, lamo, dtv, PFw);
-        ctstep<V, LIM, FT1, NU, 3, true, true, true, false, CL_MAPPED, true, IX>(A, X, M, 3, lamh, lam, lamf, lamo, dtv, PFw);
+    for (int s = a - 4;; s += 4) {
+        ctstep<V, LIM, FT1, NU, 0, IX>(A, X, M, s, a, lamh, lam, lamf, lamo, dtv);
+        if (s >= last) break;
+        ctstep<V, LIM, FT1, NU, 1, IX>(A, X, M, s + 1, a, lamh, lam, lamf, lamo, dtv);
+        if (s + 1 >= last) break;
+        ctstep<V, LIM, FT1, NU, 2, IX>(A, X, M, s + 2, a, lamh, lam, lamf, lamo, dtv);
+        if (s + 2 >= last) break;
+        ctstep<V, LIM, FT1, NU, 3, IX>(A, X, M, s + 3, a, lamh, lam, lamf, lamo, dtv);
+        if (s + 3 >= last) break;
     }
-    // tail: cells s .. n+3 through the map (n-4 <= s <= n-1 after the loop,
-    // s = 0 mod 4: at most eight cells)
-    if (s <= n + 3) ctstep<V, LIM, FT1, NU, 0, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 1 <= n + 3) ctstep<V, LIM, FT1, NU, 1, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s + 1, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 2 <= n + 3) ctstep<V, LIM, FT1, NU, 2, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s + 2, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 3 <= n + 3) ctstep<V, LIM, FT1, NU, 3, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s + 3, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 4 <= n + 3) ctstep<V, LIM, FT1, NU, 0, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s + 4, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 5 <= n + 3) ctstep<V, LIM, FT1, NU, 1, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s + 5, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 6 <= n + 3) ctstep<V, LIM, FT1, NU, 2, true, true, true, true, CL_MAPPED, true, IX>(A, X, M, s + 6, lamh, lam, lamf, lamo, dtv, PFw);
-    if (s + 7 <= n + 3) ctstep<V, LIM, FT1, NU, 3, true, true, true, true, CL_NONE, false, IX>(A, X, M, s + 7, lamh, lam, lamf, lamo, dtv, PFw);
 }
 
-// The warps of a block take the same segment of FISH_CT_ROWS consecutive
+// The warps of a block take the same segment of ct_rows() consecutive
 // rows of the other axis, so the neighbour-row loads of each warp (rho, m_d
 // of rows o-1 and o+1, the other-axis face of row o-1) are mostly the
-// own-row loads of its sibling warps, served from L1.  Grid: segments x
-// ceil(no/FISH_CT_ROWS).
-#ifndef FISH_CT_ROWS
-#define FISH_CT_ROWS 8   // rows (warps) per CT block
-#endif
+// own-row loads of its sibling warps, served from L1; FP64, bound by its pipe
+// and not by loads, takes one warp per block.  Grid: (column segments x
+// ceil(no / ct_rows())) x segments of `len` cells along the sweep.
+template <class V> constexpr int ct_rows() { return VT<V>::F64 ? 1 : 8; }
+// Blocks per SM the kernels are compiled for.
+template <class V> constexpr int ct_resident() { return (VT<V>::F64 ? 8 : FISH_CT_MINB * 4) / ct_rows<V>(); }
+
 template <class V, int LIM, bool FT1, bool NU = false, class IX = long long>
-__global__ void __launch_bounds__(32 * FISH_CT_ROWS, (VT<V>::F64 || VT<V>::W == 2) ? FISH_CT_MINB2 : FISH_CT_MINB * 4 / FISH_CT_ROWS)
-    ct_col_kernel(const ColCTArgs<typename VT<V>::S> A)
+__global__ void __launch_bounds__(32 * ct_rows<V>(), ct_resident<V>())
+    ct_col_kernel(const ColCTArgs<typename VT<V>::S> A, int len)
 {
     constexpr int SEGC = 31 * VT<V>::W;
     const long long nseg = (A.nf + SEGC - 1) / SEGC;
-    const long long seg = blockIdx.x % nseg, ob = (blockIdx.x / nseg) * FISH_CT_ROWS + (threadIdx.x >> 5);
-    ct_columns<V, LIM, FT1, NU, IX>(A, ob * nseg + seg, threadIdx.x & 31);
+    const long long seg = blockIdx.x % nseg, ob = (blockIdx.x / nseg) * ct_rows<V>() + (threadIdx.x >> 5);
+    const int a = blockIdx.y * len;
+    ct_columns<V, LIM, FT1, NU, IX>(A, ob * nseg + seg, threadIdx.x & 31, a, min(A.n, a + len));
 }
 
 // ---------------------------------------------------------------------------

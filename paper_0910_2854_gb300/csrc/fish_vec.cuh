@@ -58,6 +58,13 @@ __device__ __forceinline__ double vfma(double a, double b, double c) { return a 
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ P2 vfma(P2 a, P2 b, P2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
 
+// a*b, rounded: never contracted into a following addition in FP32, so that
+// one pencil advanced as float (the lower face of a row, the batch, the single
+// box) and as a component of a P2 gets the same bits
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ P2 vmul(P2 a, P2 b) { return a * b; }
+
 // ---- component-wise functions ---------------------------------------------
 __device__ __forceinline__ double vsqrt(double a) { return sqrt(a); }
 __device__ __forceinline__ float vsqrt(float a) { return sqrtf(a); }
@@ -82,7 +89,7 @@ __device__ __forceinline__ P2 vrcp(P2 a) { return {make_float2(__fdividef(1.0f, 
 
 // quotient: IEEE in FP64, a * rcp(b) in FP32
 __device__ __forceinline__ double vdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float vdiv(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ float vdiv(float a, float b) { return __fmul_rn(a, __fdividef(1.0f, b)); }
 __device__ __forceinline__ P2 vdiv(P2 a, P2 b) { return a * vrcp(b); }
 
 // select: c > 0 ? a : b, per component
@@ -123,8 +130,8 @@ __device__ __forceinline__ double vvanleer(double a, double b)
 }
 __device__ __forceinline__ float vvanleer(float a, float b)
 {
-    const float ab = a * b;
-    return ab > 0.0f ? __fdividef(ab + ab, a + b) : 0.0f;
+    const float ab = __fmul_rn(a, b);
+    return ab > 0.0f ? __fmul_rn(ab + ab, __fdividef(1.0f, a + b)) : 0.0f;
 }
 __device__ __forceinline__ P2 vvanleer(P2 a, P2 b)
 {

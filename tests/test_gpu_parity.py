@@ -591,3 +591,42 @@ def test_turbulence_twin_128():
     assert l1 <= 1e-5, l1
     for b in boxes.values():
         b.close()
+
+
+# ---------------------------------------------------------------------------
+# segments of the column marches
+# ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("bc", [W.BC_PERIODIC, W.BC_OUTFLOW])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 9, 16, 33])
+def test_sweep_segments(F, n, bc, precision):
+    """A sweep over few columns is cut into segments of one or two cells,
+    whose windows reach over the boundary and over neighbouring segments:
+    every operator along the axis of n cells (thinner than the stencil, odd,
+    and longer than several segments), plain and with each potential form."""
+    for d in range(3):
+        dims = [6, 5, 4]
+        dims[d] = n
+        w = W.random_smooth(*dims, seed=80 + n, bc=bc)
+        w.phi = 0.1 * np.cos(np.arange(n * 6 * 5 * 4, dtype=np.float64)[: dims[0] * dims[1] * dims[2]]
+                             ).reshape(dims[2], dims[1], dims[0])
+        for kw in ({}, {"phi": True}, {"phi": True, "hse": True}, {"phi": True, "gravity_split": True}):
+            kw = dict(kw)
+            phi = w.phi if kw.pop("phi", False) else None
+            ob = oracle.OracleBox(*w.dims, w.gamma, bc=w.bc, h=w.h, phi=phi, **kw)
+            ob.set_state(w.state)
+            gkw = dict(kw)
+            if gkw.pop("gravity_split", False):
+                gkw["gravity"] = "split"
+            gb = F.Box(*w.dims, w.gamma, bc=w.bc, precision=precision, h=w.h, **gkw)
+            gb.set_state(w.state)
+            if phi is not None:
+                gb.set_potential(phi)
+            dt = 0.4 * ob.cfl(1.0)
+            ob.fluid(d, dt)
+            gb.fluid(d, dt)
+            ob.ct(d, dt)
+            gb.ct(d, dt)
+            assert rel_err(gb.get_state(), ob.state) <= (1e-12 if precision == "fp64" else 1e-5), (d, kw)
+            gb.close()
