@@ -92,6 +92,7 @@ template <class V> struct CCell {
 // turns NaN if any evaluated cell produced one
 template <class V> struct Checks {
     V mn_rho, mn_p, nsum;
+    int hi;   // FP64: FLAG_* seen, by the bits of rho, p and c_F
 };
 
 template <class V> __device__ __forceinline__ void checks_init(Checks<V> &k)
@@ -99,11 +100,13 @@ template <class V> __device__ __forceinline__ void checks_init(Checks<V> &k)
     k.mn_rho = vb<V>(3.0e38f);
     k.mn_p = vb<V>(3.0e38f);
     k.nsum = vb<V>(0.0f);
+    k.hi = 0;
 }
 
 template <class V> __device__ __forceinline__ unsigned checks_flags(const Checks<V> &k)
 {
     unsigned f = 0;
+    if constexpr (VT<V>::F64) return (unsigned)k.hi;
 #pragma unroll
     for (int i = 0; i < VT<V>::W; ++i) {
         const auto r = vget(k.mn_rho, i), p = vget(k.mn_p, i), s = vget(k.nsum, i);
@@ -142,15 +145,18 @@ __device__ __forceinline__ void ceval(const V u[5], const V bb[3], V gamma, V gm
     for (int i = 0; i < 5; ++i) c.u[i] = u[i];
     V v0, v1, v2, p, a2, bn2, bt2, mag;
     if constexpr (VT<V>::F64) {
-        v0 = u[1] / rho;
-        v1 = u[2] / rho;
-        v2 = u[3] / rho;
-        const V kin = 0.5 * (u[1] * v0 + u[2] * v1 + u[3] * v2);
-        mag = 0.5 * (bb[0] * bb[0] + bb[1] * bb[1] + bb[2] * bb[2]);
-        p = gm1 * (u[4] - kin - mag);
-        a2 = gamma * p / rho;
-        bn2 = bb[0] * bb[0] / rho;
-        bt2 = (bb[1] * bb[1] + bb[2] * bb[2]) / rho;
+        const V ri = rcp64(rho);
+        v0 = quot64(u[1], rho, ri);
+        v1 = quot64(u[2], rho, ri);
+        v2 = quot64(u[3], rho, ri);
+        // kin = k2 / 2 and mag (here b^2, the factor 1/2 in the operations
+        // that use it, whose products with it are exact)
+        const V k2 = u[1] * v0 + u[2] * v1 + u[3] * v2;
+        mag = bb[0] * bb[0] + bb[1] * bb[1] + bb[2] * bb[2];
+        p = gm1 * __fma_rn(-0.5, mag, __fma_rn(-0.5, k2, u[4]));
+        a2 = quot64(gamma * p, rho, ri);
+        bn2 = quot64(bb[0] * bb[0], rho, ri);
+        bt2 = quot64(bb[1] * bb[1] + bb[2] * bb[2], rho, ri);
     } else {
         const V half = vb<V>(0.5f);
         const V ri = vrcp(rho);
@@ -167,10 +173,12 @@ __device__ __forceinline__ void ceval(const V u[5], const V bb[3], V gamma, V gm
         bn2 = bn * ri;
         bt2 = bt * ri;
     }
-    const V ptot = p + mag;
+    V ptot;
+    if constexpr (VT<V>::F64) ptot = __fma_rn(0.5, mag, p);
+    else ptot = p + mag;
     const V B2 = bn2 + bt2;
     V disc;
-    if constexpr (VT<V>::F64) disc = (a2 - B2) * (a2 - B2) + 4.0 * a2 * bt2;
+    if constexpr (VT<V>::F64) disc = __fma_rn(4.0, a2 * bt2, (a2 - B2) * (a2 - B2));
     else disc = vfma(a2 - B2, a2 - B2, vb<V>(4.0f) * a2 * bt2);
     c.cf = vsqrt(vb<V>(0.5f) * (a2 + B2 + vsqrt(disc)));
     c.cs = vsqrt(a2);
@@ -193,9 +201,15 @@ __device__ __forceinline__ void ceval(const V u[5], const V bb[3], V gamma, V gm
         c.F[3] = vfma(nb0, bb[2], u[3] * v0);
         c.F[4] = vfma(nb0, bv, (u[4] + ptot) * v0);
     }
-    k.mn_rho = vmin(k.mn_rho, rho);
-    k.mn_p = vmin(k.mn_p, p);
-    k.nsum = k.nsum + c.cf;
+    if constexpr (VT<V>::F64) {
+        if (!pos64(rho)) k.hi |= FLAG_RHO;
+        if (!pos64(p)) k.hi |= FLAG_P;
+        if ((__double2hiint(c.cf) & 0x7fffffff) > 0x7ff00000) k.hi |= FLAG_NAN;
+    } else {
+        k.mn_rho = vmin(k.mn_rho, rho);
+        k.mn_p = vmin(k.mn_p, p);
+        k.nsum = k.nsum + c.cf;
+    }
 }
 
 // Potential difference phi_b - phi_a across the interface a|b.  FP64 takes
@@ -240,7 +254,9 @@ __device__ __forceinline__ void chse(const CCell<V> &a, const CCell<V> &b, V phi
 }
 
 // first-order interface flux: eq0140 with D = alpha max(d_a, d_b) (eq0150),
-// or the HSE-corrected form eq0324 (reading C-3)
+// or the HSE-corrected form eq0324 (reading C-3).  FP64 without the correction
+// gives twice the flux (flux_scale: the factor is exact and goes into dt/dx).
+template <class V, bool HSE> constexpr double flux_scale() { return VT<V>::F64 && !HSE ? 0.5 : 1.0; }
 template <class V, bool HSE>
 __device__ __forceinline__ void cflux1(const CCell<V> &a, const CCell<V> &b, V phia, V phib, V alpha, V F[5])
 {
@@ -248,7 +264,7 @@ __device__ __forceinline__ void cflux1(const CCell<V> &a, const CCell<V> &b, V p
         const V D = alpha * vmax(a.d, b.d);
         if constexpr (VT<V>::F64) {
 #pragma unroll
-            for (int i = 0; i < 5; ++i) F[i] = 0.5 * (a.F[i] + b.F[i]) - 0.5 * D * (b.u[i] - a.u[i]);
+            for (int i = 0; i < 5; ++i) F[i] = (a.F[i] + b.F[i]) - D * (b.u[i] - a.u[i]);
         } else {
             const V half = vb<V>(0.5f);
 #pragma unroll
@@ -324,21 +340,23 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
         const V D = vmax(c1.d, c2.d);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
-            const V fp0 = 0.5 * (c0.F[i] + D * c0.u[i]);
-            const V fp1 = 0.5 * (c1.F[i] + D * c1.u[i]);
-            const V fp2 = 0.5 * (c2.F[i] + D * c2.u[i]);
-            const V fm1 = 0.5 * (c1.F[i] - D * c1.u[i]);
-            const V fm2 = 0.5 * (c2.F[i] - D * c2.u[i]);
-            const V fm3 = 0.5 * (c3.F[i] - D * c3.u[i]);
-            V slp, slm;
+            // twice the split fluxes F+ and F- (eq0130)
+            const V d1 = D * c1.u[i], d2 = D * c2.u[i];
+            const V fp0 = c0.F[i] + D * c0.u[i];
+            const V fp1 = c1.F[i] + d1;
+            const V fp2 = c2.F[i] + d2;
+            const V fm1 = c1.F[i] - d1;
+            const V fm2 = c2.F[i] - d2;
+            const V fm3 = c3.F[i] - D * c3.u[i];
+            V slp, slm;  // half of twice the limited slopes
             if constexpr (NU) {
-                slp = w1 * vlimit<LIM>((fp1 - fp0) / gl, (fp2 - fp1) / gc, lim);
-                slm = w2 * vlimit<LIM>((fm2 - fm1) / gc, (fm3 - fm2) / gr, lim);
+                slp = w1 * vlimit_half<LIM>((fp1 - fp0) / gl, (fp2 - fp1) / gc, lim);
+                slm = w2 * vlimit_half<LIM>((fm2 - fm1) / gc, (fm3 - fm2) / gr, lim);
             } else {
-                slp = vlimit<LIM>(fp1 - fp0, fp2 - fp1, lim);
-                slm = vlimit<LIM>(fm2 - fm1, fm3 - fm2, lim);
+                slp = vlimit_half<LIM>(fp1 - fp0, fp2 - fp1, lim);
+                slm = vlimit_half<LIM>(fm2 - fm1, fm3 - fm2, lim);
             }
-            F[i] = fp1 + fm2 + 0.5 * (slp - slm);
+            F[i] = fp1 + fm2 + (slp - slm);
         }
     } else {
         const V half = vb<V>(0.5f);
@@ -358,7 +376,18 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
             const V fm_l = half * ((c2.F[i] - c1.F[i]) - q1);
             const V fm_r = half * ((c3.F[i] - c2.F[i]) - q2);
             V slp, slm;
-            if constexpr (NU) {
+            if constexpr (VT<V>::F64) {
+                // (half the limited slopes)
+                if constexpr (NU) {
+                    slp = w1 * vlimit_half<LIM>(fp_l / gl, fp_r / gc, lim);
+                    slm = w2 * vlimit_half<LIM>(fm_l / gc, fm_r / gr, lim);
+                } else {
+                    slp = vlimit_half<LIM>(fp_l, fp_r, lim);
+                    slm = vlimit_half<LIM>(fm_l, fm_r, lim);
+                }
+                F[i] = half * (c1.F[i] + c2.F[i]) - half * q1 + (slp - slm);
+                continue;
+            } else if constexpr (NU) {
                 slp = w1 * vlimit<LIM>(vdiv(fp_l, gl), vdiv(fp_r, gc), lim);
                 slm = w2 * vlimit<LIM>(vdiv(fm_l, gc), vdiv(fm_r, gr), lim);
             } else {
@@ -711,7 +740,7 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         V up[5];
         V lh = lamh;
         if constexpr (NU) {
-            if constexpr (VT<V>::F64) lh = dt / (2.0 * M.w1);
+            if constexpr (VT<V>::F64) lh = flux_scale<V, HSE>() * (dt / (2.0 * M.w1));
             else lh = vdiv(hdt, vb<V>(M.w1));
         }
 #pragma unroll
@@ -745,7 +774,7 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
                                 A.lim, vb<V>(M.w4), vb<V>(M.w3), vb<V>(M.w2), vb<V>(M.w1));
         V lo = lam;
         if constexpr (NU) {
-            if constexpr (VT<V>::F64) lo = dt / M.w3;
+            if constexpr (VT<V>::F64) lo = flux_scale<V, HSE>() * (dt / M.w3);
             else lo = vdiv(dt, vb<V>(M.w3));
         }
 #pragma unroll
@@ -829,8 +858,8 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     }
     const double dtd = *A.dt;
     const V dt = vb<V>(S(dtd));
-    const V lam = vb<V>(S(dtd / A.h));
-    const V lamh = vb<V>(S(dtd / (2.0 * A.h)));
+    const V lam = vb<V>(S(flux_scale<V, HSE>() * (dtd / A.h)));
+    const V lamh = vb<V>(S(flux_scale<V, HSE>() * (dtd / (2.0 * A.h))));
     const V hdt = vb<V>(S(0.5 * dtd));
     const V rtwoh = vb<V>(S(1.0 / (2.0 * A.h)));
 
@@ -925,6 +954,8 @@ template <class V> struct CFace {
     V vh[4];   // smoothed velocity (eq0362) at s-1
     V bf[4];   // face field at s
     V w[2];    // cell product v b at s-1
+    V dw[2];   // FP64: differences of the predicted products, w_{s-2} - w_{s-3} (slot s & 1)
+    unsigned up;  // FP64: bit k: edge velocity > 0 at interface (s-2-k)'
     V f1[2];   // predictor flux at interface (s-2)'
     V wp[4];   // predicted product at s-2
     V f[2];    // corrector flux at interface (s-4)'
@@ -940,9 +971,12 @@ template <class V> struct CWid {
 template <class V, bool NU> __device__ __forceinline__ V cedge(V va, V vb_, V wa, V wb)
 {
     if constexpr (!NU) return vb<V>(0.5f) * (va + vb_);
-    else if constexpr (VT<V>::F64) return (wb * va + wa * vb_) / (wa + wb);
     else return vdiv(vfma(wb, va, wa * vb_), wa + wb);
 }
+
+// FP64 B_d: the velocities a face pencil is advanced with are eight times the
+// smoothed ones, so the factors dt/dx of its fluxes carry an eighth.
+constexpr double CT_SCALE = 0.125;
 
 // Advance a face pencil by cell s (K = s mod 4) with face velocity vt and
 // field bf.  With OUT, bnew receives the updated face field of cell s-4 and
@@ -954,10 +988,50 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
 {
     constexpr int k1 = (K + 3) & 3, k2 = (K + 2) & 3, kp = (K + 1) & 3;
     constexpr int e = K & 1, o = (K + 1) & 1;
+    if constexpr (VT<V>::F64) {
+        // The formulas below with vt twice the face velocity and the factor
+        // 1/4 of the smoothing left out: velocities, products and fluxes are
+        // eight times theirs, exactly, and lamh, lam an eighth (CT_SCALE).  The
+        // upwind sides are kept as bits and the differences of the predicted
+        // products in registers; the upwind operands are selected before the
+        // one limiter.
+        const V vh = __fma_rn(2.0, P.vt[k1], vt) + P.vt[k2];
+        P.vh[k1] = vh;
+        P.w[o] = vh * P.bf[k1];
+        V vbar;
+        if constexpr (NU) vbar = cw.w1 * P.vh[k2] + cw.w2 * vh;  // (positive weights over their sum: the sign)
+        else vbar = P.vh[k2] + vh;
+        const bool pos = pos64(vbar);
+        P.up = P.up << 1 | (pos ? 1u : 0u);
+        P.f1[e] = pos ? P.w[e] : P.w[o];
+        V lh = lamh;
+        if constexpr (NU) lh = CT_SCALE * (dt / (2.0 * cw.w2));
+        const V bp = P.bf[k2] - lh * (P.f1[e] - P.f1[o]);
+        P.wp[k2] = P.vh[k2] * bp;
+        const V d2 = P.wp[k2] - P.wp[kp];
+        if (live) {
+            const bool u = (P.up & 4u) != 0;  // interface (s-4)'
+            V la = u ? P.dw[e] : P.dw[o], lb = u ? P.dw[o] : d2;
+            if constexpr (NU) {
+                la = la / (0.5 * (u ? cw.w5 + cw.w4 : cw.w4 + cw.w3));
+                lb = lb / (0.5 * (u ? cw.w4 + cw.w3 : cw.w3 + cw.w2));
+            }
+            V sl = vlimit_half<LIM>(la, lb, lim);
+            if constexpr (NU) sl = (u ? cw.w4 : cw.w3) * sl;
+            P.f[e] = (u ? P.wp[K] : P.wp[kp]) + (u ? sl : -sl);
+            if constexpr (OUT) {
+                V lo = lam;
+                if constexpr (NU) lo = CT_SCALE * (dt / cw.w4);
+                bnew = P.bf[K] - lo * (P.f[e] - P.f[o]);
+            }
+        }
+        P.dw[e] = d2;
+        P.bf[K] = bf;
+        P.vt[K] = vt;
+        return;
+    }
     // smoothed face velocity at s-1 (eq0362) and the cell product w_{s-1}
-    V vh;
-    if constexpr (VT<V>::F64) vh = 0.25 * (vt + 2.0 * P.vt[k1] + P.vt[k2]);
-    else vh = vb<V>(0.25f) * (vfma(vb<V>(2.0f), P.vt[k1], vt) + P.vt[k2]);
+    const V vh = vb<V>(0.25f) * (vfma(vb<V>(2.0f), P.vt[k1], vt) + P.vt[k2]);
     P.vh[k1] = vh;
     P.w[o] = vmul(vh, P.bf[k1]);
     {
@@ -970,15 +1044,11 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         // predictor half step of the face field at s-2
         V bp;
         V lh = lamh;
-        if constexpr (NU) {
-            if constexpr (VT<V>::F64) lh = dt / (2.0 * cw.w2);
-            else lh = vdiv(vb<V>(0.5f) * dt, cw.w2);
-        }
-        if constexpr (VT<V>::F64) bp = P.bf[k2] - lh * (P.f1[e] - P.f1[o]);
-        else bp = vfma(-lh, P.f1[e] - P.f1[o], P.bf[k2]);
+        if constexpr (NU) lh = vdiv(vb<V>(0.5f) * dt, cw.w2);
+        bp = vfma(-lh, P.f1[e] - P.f1[o], P.bf[k2]);
         P.wp[k2] = vmul(P.vh[k2], bp);
     }
-    if (!VT<V>::F64 || live) {
+    {
         // corrector flux at q' = (s-4)': piecewise-linear TVD about the
         // upwind cell (reading C-10)
         const V vbar = cedge<V, NU>(P.vh[K], P.vh[kp], cw.w4, cw.w3);
@@ -988,10 +1058,7 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
             // half the upwind cell (reading C-25)
             const V half = vb<V>(0.5f);
             const V gl = half * (cw.w5 + cw.w4), gc = half * (cw.w4 + cw.w3), gr = half * (cw.w3 + cw.w2);
-            if constexpr (VT<V>::F64) {
-                P.f[e] = vbar > 0.0 ? w0 + 0.5 * cw.w4 * vlimit<LIM>((w0 - wm) / gl, (w1 - w0) / gc, lim)
-                                    : w1 - 0.5 * cw.w3 * vlimit<LIM>((w1 - w0) / gc, (w2 - w1) / gr, lim);
-            } else {
+            {
                 const V d0 = vdiv(w0 - wm, gl), d1 = vdiv(w1 - w0, gc), d2 = vdiv(w2 - w1, gr);
                 const V la = vsel_pos(vbar, d0, d1);
                 const V lb = vsel_pos(vbar, d1, d2);
@@ -999,8 +1066,6 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
                 const V sg = vsel_pos(vbar, half * cw.w4, -half * cw.w3);
                 P.f[e] = vfma(sg, vlimit<LIM>(la, lb, lim), base);
             }
-        } else if constexpr (VT<V>::F64) {
-            P.f[e] = vbar > 0.0 ? w0 + 0.5 * vlimit<LIM>(w0 - wm, w1 - w0, lim) : w1 - 0.5 * vlimit<LIM>(w1 - w0, w2 - w1, lim);
         } else {
             // select the upwind operands, then limit once
             const V d0 = w0 - wm, d1 = w1 - w0, d2 = w2 - w1;
@@ -1012,12 +1077,8 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         }
         if constexpr (OUT) {
             V lo = lam;
-            if constexpr (NU) {
-                if constexpr (VT<V>::F64) lo = dt / cw.w4;
-                else lo = vdiv(dt, cw.w4);
-            }
-            if constexpr (VT<V>::F64) bnew = P.bf[K] - lo * (P.f[e] - P.f[o]);
-            else bnew = vfma(-lo, P.f[e] - P.f[o], P.bf[K]);
+            if constexpr (NU) lo = vdiv(dt, cw.w4);
+            bnew = vfma(-lo, P.f[e] - P.f[o], P.bf[K]);
         }
     }
     P.bf[K] = bf;
@@ -1160,11 +1221,12 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
         M.cw.w0 = M.R.w;
     }
     // consume the raw inputs of cell s
-    const V vc = vdiv(M.R.mc, M.R.rc);
-    const V vop = vdiv(M.R.mo, M.R.ro);
-    const V vom = vdiv(M.R.mm, M.R.rm);
+    const V vc = vquot(M.R.mc, M.R.rc);
+    const V vop = vquot(M.R.mo, M.R.ro);
+    const V vom = vquot(M.R.mm, M.R.rm);
     V vfp;
-    if constexpr (VT<V>::W == 2) vfp = vshift_hi(vc, __fdividef(M.R.mf, M.R.rf));
+    if constexpr (VT<V>::F64) vfp = vquot(M.R.mf, M.R.rf);
+    else if constexpr (VT<V>::W == 2) vfp = vshift_hi(vc, __fdividef(M.R.mf, M.R.rf));
     else vfp = vdiv(V(M.R.mf), V(M.R.rf));
     const V bF = M.R.bF, bO = M.R.bO, bOm = M.R.bOm;
     const V bdo = M.R.bdo;
@@ -1175,14 +1237,19 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
     // face velocities (eq0361): the mean of the two cells across the face,
     // or on an irregular mesh their linear interpolation to it (reading C-27)
     V vtF, vtO, vtOm;
-    if constexpr (!NU) {
+    if constexpr (!NU && VT<V>::F64) {
+        // (twice the mean, see cface)
+        vtF = vc + vfp;
+        vtO = vc + vop;
+        vtOm = vom + vc;
+    } else if constexpr (!NU) {
         vtF = half * (vc + vfp);
         vtO = half * (vc + vop);
         vtOm = half * (vom + vc);
     } else if constexpr (VT<V>::F64) {
-        vtF = (X.wfb * vc + X.wfa * vfp) / (X.wfa + X.wfb);
-        vtO = (X.wop * vc + X.woa * vop) / (X.woa + X.wop);
-        vtOm = (X.woa * vom + X.wom * vc) / (X.wom + X.woa);
+        vtF = 2.0 * ((X.wfb * vc + X.wfa * vfp) / (X.wfa + X.wfb));
+        vtO = 2.0 * ((X.wop * vc + X.woa * vop) / (X.woa + X.wop));
+        vtOm = 2.0 * ((X.woa * vom + X.wom * vc) / (X.wom + X.woa));
     } else {
         vtF = vdiv(vfma(V(X.wfb), vc, V(X.wfa) * vfp), V(X.wfa + X.wfb));
         vtO = vdiv(vfma(V(X.wop), vc, V(X.woa) * vop), V(X.woa + X.wop));
@@ -1275,10 +1342,11 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
     X.oop = (IX)(gmap(ob + 1, A.no, A.bc) - ob) * (IX)A.so;
     const double dtd = *A.dt;
     const V dtv = vb<V>(S(dtd));
-    const V lamh = vb<V>(S(dtd / (2.0 * A.h)));
-    const V lam = vb<V>(S(dtd / A.h));
-    V lamf = vb<V>(S(dtd / A.hf));
-    V lamo = vb<V>(S(dtd / A.ho));
+    constexpr double sc = VT<V>::F64 ? CT_SCALE : 1.0;
+    const V lamh = vb<V>(S(sc * (dtd / (2.0 * A.h))));
+    const V lam = vb<V>(S(sc * (dtd / A.h)));
+    V lamf = vb<V>(S(sc * (dtd / A.hf)));
+    V lamo = vb<V>(S(sc * (dtd / A.ho)));
     if constexpr (NU) {
         // irregular mesh: widths of the lane's column and its neighbours (a
         // halo or ghost column has the width of its image), and the
@@ -1288,15 +1356,16 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
         X.woa = A.wo[ob];
         X.wop = A.wo[gmap(ob + 1, A.no, A.bc)];
         X.wom = A.wo[gmap(ob - 1, A.no, A.bc)];
-        lamf = vb<V>(S(dtd / (double)X.wfa));
-        lamo = vb<V>(S(dtd / (double)X.woa));
+        lamf = vb<V>(S(sc * (dtd / (double)X.wfa)));
+        lamo = vb<V>(S(sc * (dtd / (double)X.woa)));
     }
     CTMarch<V> M;
     {
         CFace<V> z;
 #pragma unroll
         for (int k = 0; k < 4; ++k) z.vt[k] = z.vh[k] = z.bf[k] = z.wp[k] = vb<V>(0.0f);
-        z.w[0] = z.w[1] = z.f1[0] = z.f1[1] = z.f[0] = z.f[1] = vb<V>(0.0f);
+        z.w[0] = z.w[1] = z.f1[0] = z.f1[1] = z.f[0] = z.f[1] = z.dw[0] = z.dw[1] = vb<V>(0.0f);
+        z.up = 0;
         M.PF = M.PO = M.POm = z;
         CFace<P2> z2;
 #pragma unroll

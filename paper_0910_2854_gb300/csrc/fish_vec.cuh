@@ -11,7 +11,12 @@
 // The FP64 instantiation is compiled without FMA contraction and every
 // formula keeps the operation order of the plain IEEE evaluation, so that
 // the double path rounds like a straightforward implementation of the
-// paper's formulas.
+// paper's formulas.  GB300's FP64 pipe is its bound (about two operations a
+// clock per SM), so what does not change a rounding is kept off that pipe:
+// factors that are powers of two are left in the operands (they scale every
+// intermediate exactly) or folded into an explicit fused multiply-add whose
+// product is exact; signs, minima and zero tests act on the bits as integers;
+// a quotient costs three operations behind a reciprocal that several share.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -105,12 +110,43 @@ __device__ __forceinline__ double vget(double a, int) { return a; }
 __device__ __forceinline__ float vget(float a, int) { return a; }
 __device__ __forceinline__ float vget(P2 a, int i) { return i ? a.v.y : a.v.x; }
 
+// ---- FP64 quotients ---------------------------------------------------------
+// A reciprocal by one third-order Newton step on the hardware's approximation
+// (about 20 bits, then 60), and the quotient corrected by its exact residual
+// (P. W. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", IBM J. Res. Dev. 34, 1990): the correctly rounded
+// a / b but for about one pair in 2^30, for finite operands whose quotient
+// and residual neither overflow nor underflow.  Zero, infinite or NaN
+// divisors give NaN.
+__device__ __forceinline__ double rcp64(double b)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+    const double e = __fma_rn(-b, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+__device__ __forceinline__ double quot64(double a, double b, double rb)
+{
+    const double q = a * rb;
+    return __fma_rn(__fma_rn(-b, q, a), rb, q);
+}
+// velocity m / rho of a cell
+__device__ __forceinline__ double vquot(double a, double b) { return quot64(a, b, rcp64(b)); }
+__device__ __forceinline__ float vquot(float a, float b) { return vdiv(a, b); }
+__device__ __forceinline__ P2 vquot(P2 a, P2 b) { return vdiv(a, b); }
+// a > 0 by the bits (no FP64 pipe operation)
+__device__ __forceinline__ bool pos64(double a) { return __double_as_longlong(a) > 0; }
+
 // ---- limiters (eq0190 minmod, eq0200 Van Leer; sign(0) = 0, reading C-8) --
 template <class S> __device__ __forceinline__ S ssgn(S a) { return a > S(0) ? S(1) : (a < S(0) ? S(-1) : S(0)); }
 
 __device__ __forceinline__ double vminmod(double a, double b)
 {
-    return 0.5 * (ssgn(a) + ssgn(b)) * fmin(fabs(a), fabs(b));
+    // the operand of smaller magnitude where the signs agree, by the bits
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+    const long long top = 0x7fffffffffffffffll;
+    const long long m = min(ia & top, ib & top);
+    return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(m | (ia & ~top));
 }
 __device__ __forceinline__ float sminmod_f(float a, float b)
 {
@@ -123,10 +159,12 @@ __device__ __forceinline__ P2 vminmod(P2 a, P2 b)
     return {make_float2(sminmod_f(a.v.x, b.v.x), sminmod_f(a.v.y, b.v.y))};
 }
 
-__device__ __forceinline__ double vvanleer(double a, double b)
+// half of the Van Leer limiter, ab / (a + b) (the factor 2 is exact)
+__device__ __forceinline__ double vvanleer_half(double a, double b)
 {
-    if (a * b > 0.0) return 2.0 * a * b / (a + b);
-    return 0.0;
+    const double ab = a * b, c = a + b;
+    const double q = quot64(ab, c, rcp64(c));
+    return pos64(ab) ? q : 0.0;
 }
 __device__ __forceinline__ float vvanleer(float a, float b)
 {
@@ -148,6 +186,14 @@ template <int LIM, class V> __device__ __forceinline__ V vlimit(V a, V b, int li
     else if constexpr (LIM == 1) return vminmod(a, b);
     else if constexpr (LIM == 2) return vb<V>(0);
     else return lim == 0 ? vvanleer(a, b) : (lim == 1 ? vminmod(a, b) : vb<V>(0));
+}
+// half the limiter, FP64
+template <int LIM> __device__ __forceinline__ double vlimit_half(double a, double b, int lim)
+{
+    if constexpr (LIM == 0) return vvanleer_half(a, b);
+    else if constexpr (LIM == 1) return 0.5 * vminmod(a, b);
+    else if constexpr (LIM == 2) return 0.0;
+    else return lim == 0 ? vvanleer_half(a, b) : (lim == 1 ? 0.5 * vminmod(a, b) : 0.0);
 }
 
 // ---- memory access -----------------------------------------------------------
