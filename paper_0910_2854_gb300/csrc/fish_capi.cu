@@ -18,7 +18,7 @@ using fish::Launch;
 
 namespace {
 
-constexpr int kDiagBlocks = 1024;
+constexpr int kDiagBlocks = 456;  // three blocks on each of 152 SMs: one even wave
 constexpr long long kStageChunk = 1ll << 25;  // doubles per conversion chunk (256 MB)
 
 }  // namespace

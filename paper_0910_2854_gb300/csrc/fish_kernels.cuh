@@ -13,22 +13,13 @@
 
 #include "fish_math.cuh"
 #include "fish_types.h"
+#include "fish_vec.cuh"
 
 namespace fish {
 
 // ---------------------------------------------------------------------------
 // CFL (eq0083-eq0084): min over cells and axes of h_d / (|v_d| + c_F,d)
 // ---------------------------------------------------------------------------
-// Coordinates of the element at memory offset idx (axes in memory order).
-__device__ __forceinline__ void coords_of(const Geom &g, long long idx, int cc[3])
-{
-    const int f0 = g.ord[0], f1 = g.ord[1], f2 = g.ord[2];
-    cc[f0] = (int)(idx % g.n[f0]);
-    const long long r = idx / g.n[f0];
-    cc[f1] = (int)(r % g.n[f1]);
-    cc[f2] = (int)(r / g.n[f1]);
-}
-
 template <class T> struct CFLArgs {
     const T *in[8];
     Geom g;
@@ -69,62 +60,162 @@ __device__ __forceinline__ float cfl_rate_f32(const float u[5], const float b[3]
     return best;
 }
 
-// CFL minimum over the box: one block per group of rows along the fastest
-// memory axis (no per-cell index division); per-block minimum, then one
-// atomic on the order-preserving bits of the positive double.
-template <class T>
+// Conversions that keep off the FP64 pipe, where GB300 converts: zeros and
+// normal numbers by moving the exponent and mantissa.  `odd` collects whether
+// an operand was something else, whose result is then not its value.
+__device__ __forceinline__ double widen(double f, unsigned &) { return f; }
+__device__ __forceinline__ double widen(float f, unsigned &odd)
+{
+    const unsigned u = __float_as_uint(f), top = u & 0x80000000u, m = u & 0x7fffffffu;
+    odd |= m != 0u && m - 0x00800000u >= 0x7f000000u ? 1u : 0u;  // subnormal, infinite, NaN
+    return __hiloint2double((int)(m ? top | ((m >> 3) + 0x38000000u) : top), (int)(m << 29));
+}
+// towards zero (1.2e-7 relative)
+__device__ __forceinline__ float narrow(double d, unsigned &odd)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), m = hi & 0x7fffffffu;
+    odd |= m != 0u && m - 0x38100000u >= 0x0fe00000u ? 1u : 0u;  // outside the normal numbers of FP32
+    return m ? __uint_as_float((hi & 0x80000000u) | ((m - 0x38000000u) << 3) | (lo >> 29)) : 0.0f;
+}
+
+// Upper bound of the FP64 path's largest rate (|v_d| + c_F,d) / h_d of a cell,
+// in FP32 behind the FP64 pressure, with margins for the FP32 rounding: with
+// c^2 = a^2 + B^2, t = a^2 / c^2 and s = b_t^2 / (rho c^2),
+//   c_F^2 = c^2 (1 + sqrt((2 t - 1)^2 + 4 t s)) / 2.
+// Infinite where an operand is no normal FP32 number or zero, NaN included.
+__device__ __forceinline__ float cfl_bound_f64(const double u[5], const double b[3], double gamma, double gm1,
+                                               const float rh[3], unsigned &flags)
+{
+    const double ri = rcp64(u[0]);
+    const double v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
+    const double k2 = u[1] * v[0] + u[2] * v[1] + u[3] * v[2];
+    const double b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+    const double p = gm1 * __fma_rn(-0.5, b2, __fma_rn(-0.5, k2, u[4]));
+    if (!pos64(u[0])) flags |= FLAG_RHO;
+    if (!pos64(p)) flags |= FLAG_P;
+    const double g2 = gamma * p, s2 = g2 + b2;   // rho a^2, rho c^2
+    unsigned odd = 0;
+    const float s2f = narrow(s2, odd), f2 = narrow(b2, odd);
+    const float c2 = narrow(s2 * ri, odd), rs = __fdividef(1.0f, s2f), t = narrow(g2, odd) * rs;
+    float r = 0.0f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const float bn = narrow(b[d], odd);
+        const float s = fmaxf(f2 - bn * bn, 0.0f) * rs + 1e-6f;
+        const float x = 2.0f * t - 1.0f;
+        const float cf = sqrtf(0.5f * c2 * (1.0f + sqrtf(x * x + 4.0f * t * s)));
+        r = fmaxf(r, (fabsf(narrow(v[d], odd)) + cf) * rh[d]);
+    }
+    // (b_n^2 against b^2 must not under- or overflow either)
+    return odd || !(s2f > 1e-30f && s2f < 1e30f && c2 > 1e-30f && r < 1e30f) ? __int_as_float(0x7f800000) : r * 1.00001f;
+}
+
+// CFL minimum over the box: a warp per row along the fastest memory axis (no
+// per-cell index division; short rows leave no warp idle), per-block minimum,
+// then one atomic on the order-preserving bits of the positive double.  Bound
+// by HBM in FP32.  FP64 would be bound by its pipe (six square roots and 24
+// quotients per cell, 9.8 ms at 256^3): a cell is evaluated in FP64 only if its
+// bound above reaches the smallest step found so far, by the warp or, at the
+// start of a row, by the whole grid.
+// PAIR (FP32, even rows): a lane takes two adjacent cells with 8-byte loads.
+template <class T, bool PAIR>
 __global__ void __launch_bounds__(256) cfl_kernel(CFLArgs<T> A)
 {
     const Geom &g = A.g;
-    const int f0 = g.ord[0], f1 = g.ord[1], f2 = g.ord[2];
-    const int nf = g.n[f0], nm = g.n[f1], ns = g.n[f2];
+    const bool yf = g.ord[0] == 1;  // y fastest (else x); z is the slowest axis of both layouts
+    const int nf = yf ? g.n[1] : g.n[0], nm = yf ? g.n[0] : g.n[1], ns = g.n[2];
+    const T *bxp = A.in[5], *byp = A.in[6], *bzp = A.in[7];
+    const long long of0 = gmap(-1, nf, g.bc);  // to the lower neighbour of a row's first cell
     const int kb = A.nk < 0 ? 0 : A.k0;
     const long long rows = (long long)nm * (A.nk < 0 ? ns : A.nk);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     double best = 1e300;   // min of h_d / (|v_d| + c_F,d)
-    float fbest = 0.0f;    // FP32 path: max of (|v_d| + c_F,d) / h_d
+    double sent = 1e300;   // FP64: the smallest minimum this thread has put into *minbits
+    float fbest = 0.0f;    // FP32 path: max of (|v_d| + c_F,d) / h_d; FP64: a lower bound of 1 / best
     unsigned flags = 0;
     float rh[3];
+#pragma unroll
     for (int d = 0; d < 3; ++d) rh[d] = (float)(1.0 / A.h[d]);
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
+    for (long long row = (long long)blockIdx.x * 8 + wid; row < rows; row += (long long)gridDim.x * 8) {
         const int m = (int)(row % nm), k = kb + (int)(row / nm);
-        const long long rbase = (long long)m * g.st[f1] + (long long)k * g.st[f2];
-        const long long om = (long long)(gmap(m - 1, nm, g.bc) - m) * g.st[f1];
-        const long long ok = (long long)(gmap(k - 1, ns, g.bc) - k) * g.st[f2];
+        const long long rbase = ((long long)k * nm + m) * nf;
+        // offsets to the lower neighbours: along the row, across the rows, across the planes
+        const long long om = (long long)(gmap(m - 1, nm, g.bc) - m) * nf;
+        const long long oz = (long long)(gmap(k - 1, ns, g.bc) - k) * nm * nf;
         if (A.w[0]) {
             // irregular mesh: this row's widths along the two slower axes
-            rh[f1] = (float)(1.0 / (double)A.w[f1][m]);
-            rh[f2] = (float)(1.0 / (double)A.w[f2][k]);
+            if (yf) rh[0] = (float)(1.0 / (double)A.w[0][m]);
+            else rh[1] = (float)(1.0 / (double)A.w[1][m]);
+            rh[2] = (float)(1.0 / (double)A.w[2][k]);
         }
-        for (int f = threadIdx.x; f < nf; f += blockDim.x) {
-            const long long idx = rbase + f;
-            const long long ofm = (long long)(gmap(f - 1, nf, g.bc) - f);
-            int cc[3];
-            cc[f0] = f;
-            cc[f1] = m;
-            cc[f2] = k;
-            if (A.w[0]) rh[f0] = (float)(1.0 / (double)A.w[f0][f]);
-            T bc[3];
-            bc[f0] = T(0.5) * (__ldg(A.in[5 + f0] + idx + ofm) + __ldg(A.in[5 + f0] + idx));
-            bc[f1] = T(0.5) * (__ldg(A.in[5 + f1] + idx + om) + __ldg(A.in[5 + f1] + idx));
-            bc[f2] = T(0.5) * (__ldg(A.in[5 + f2] + idx + ok) + __ldg(A.in[5 + f2] + idx));
-            if constexpr (sizeof(T) == 8) {
-                // per axis in the paper's frame, the oracle's operation order
+        if constexpr (sizeof(T) == 8)
+            fbest = fmaxf(fbest, 0.999999f / (float)__longlong_as_double(*(volatile long long *)A.minbits));
+        if constexpr (PAIR) {
+            for (int f = 2 * lane; f < nf; f += 64) {
+                const long long idx = rbase + f;
+                const long long of = f > 0 ? -1 : of0;
+                const T *bfp = yf ? byp : bxp, *bmp = yf ? bxp : byp;
+                const P2 bf = vload<P2>(bfp, idx), bz = vload<P2>(bzp, idx) + vload<P2>(bzp, idx + oz);
+                const P2 bfc = vshift_lo(__ldg(bfp + idx + of), bf) + bf;
+                const P2 bmc = vload<P2>(bmp, idx) + vload<P2>(bmp, idx + om);
+                P2 u[5];
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
-                    T u[5] = {__ldg(A.in[0] + idx), __ldg(A.in[1 + d] + idx), __ldg(A.in[1 + t1] + idx),
-                              __ldg(A.in[1 + t2] + idx), __ldg(A.in[4] + idx)};
-                    T bb[3] = {bc[d], bc[t1], bc[t2]};
-                    const T sp = signal_speed<T>(u, bb, A.gamma, A.gm1, flags);
-                    const T hd = A.w[0] ? A.w[d][cc[d]] : T(A.h[d]);  // eq0420
-                    const double r = (double)(hd / sp);
-                    best = r < best ? r : best;
+                for (int i = 0; i < 5; ++i) u[i] = vload<P2>(A.in[i], idx);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (A.w[0]) {
+                        if (yf) rh[1] = (float)(1.0 / (double)A.w[1][f + c]);
+                        else rh[0] = (float)(1.0 / (double)A.w[0][f + c]);
+                    }
+                    const float uc[5] = {vget(u[0], c), vget(u[1], c), vget(u[2], c), vget(u[3], c), vget(u[4], c)};
+                    const float bc[3] = {0.5f * vget(yf ? bmc : bfc, c), 0.5f * vget(yf ? bfc : bmc, c),
+                                         0.5f * vget(bz, c)};
+                    fbest = fmaxf(fbest, cfl_rate_f32(uc, bc, (float)A.gamma, (float)A.gm1, rh, flags));
                 }
+            }
+            continue;
+        }
+        for (int fw = 0; fw < nf; fw += 32) {
+            // (FP64: the lanes share their bound; the lanes past the row's end repeat its last cell)
+            const int f = min(fw + lane, nf - 1);
+            const long long idx = rbase + f;
+            const long long of = f > 0 ? -1 : of0;
+            if (A.w[0]) {
+                if (yf) rh[1] = (float)(1.0 / (double)A.w[1][f]);
+                else rh[0] = (float)(1.0 / (double)A.w[0][f]);
+            }
+            const T bc[3] = {T(0.5) * (__ldg(bxp + idx + (yf ? om : of)) + __ldg(bxp + idx)),
+                             T(0.5) * (__ldg(byp + idx + (yf ? of : om)) + __ldg(byp + idx)),
+                             T(0.5) * (__ldg(bzp + idx + oz) + __ldg(bzp + idx))};
+            const T u0[5] = {__ldg(A.in[0] + idx), __ldg(A.in[1] + idx), __ldg(A.in[2] + idx), __ldg(A.in[3] + idx),
+                             __ldg(A.in[4] + idx)};
+            if constexpr (sizeof(T) == 8) {
+                const float bound = cfl_bound_f64(u0, bc, A.gamma, A.gm1, rh, flags);
+                if (!(fbest > 1e-30f && bound < fbest)) {
+                    // per axis in the paper's frame, the oracle's operation order
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        const int t1 = (d + 1) % 3, t2 = (d + 2) % 3;
+                        const T u[5] = {u0[0], u0[1 + d], u0[1 + t1], u0[1 + t2], u0[4]};
+                        const T bb[3] = {bc[d], bc[t1], bc[t2]};
+                        const T sp = signal_speed<T>(u, bb, A.gamma, A.gm1, flags);
+                        // eq0420
+                        const T hd = A.w[0] ? A.w[d][d == 2 ? k : ((d == 1) == yf ? f : m)] : T(A.h[d]);
+                        const double r = (double)(hd / sp);
+                        best = r < best ? r : best;
+                    }
+                    fbest = fmaxf(fbest, 0.999999f / (float)best);
+                }
+                fbest = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fbest)));
             } else {
-                const float u[5] = {__ldg(A.in[0] + idx), __ldg(A.in[1] + idx), __ldg(A.in[2] + idx),
-                                    __ldg(A.in[3] + idx), __ldg(A.in[4] + idx)};
-                const float b[3] = {(float)bc[0], (float)bc[1], (float)bc[2]};
-                fbest = fmaxf(fbest, cfl_rate_f32(u, b, (float)A.gamma, (float)A.gm1, rh, flags));
+                fbest = fmaxf(fbest, cfl_rate_f32(u0, bc, (float)A.gamma, (float)A.gm1, rh, flags));
+            }
+        }
+        if constexpr (sizeof(T) == 8) {
+            // the row's minimum, so that the other warps' bounds follow
+            if (best > 0.0 && best < sent) {
+                sent = best;
+                atomicMin(A.minbits, (unsigned long long)__double_as_longlong(best));
             }
         }
     }
@@ -135,7 +226,6 @@ __global__ void __launch_bounds__(256) cfl_kernel(CFLArgs<T> A)
         best = o < best ? o : best;
     }
     __shared__ double wmin[8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (lane == 0) wmin[wid] = best;
     __syncthreads();
     if (wid == 0) {
@@ -180,43 +270,74 @@ template <class T> struct DiagArgs {
     const T *w[3] = {nullptr, nullptr, nullptr};
 };
 
+// A warp takes rows of the fastest memory axis (fixed by the grid, so the
+// order of the sums is fixed).  Bound by the FP64 pipe: eight sums per cell and
+// the divergence with quotients behind shared reciprocals of the widths.
 template <class T>
-__global__ void __launch_bounds__(256) diag_kernel(DiagArgs<T> A)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) diag_kernel(DiagArgs<T> A)
 {
     const Geom &g = A.g;
-    const long long N = (long long)g.n[0] * g.n[1] * g.n[2];
+    const bool yf = g.ord[0] == 1;  // y fastest (else x)
+    const int nf = yf ? g.n[1] : g.n[0], nm = yf ? g.n[0] : g.n[1], ns = g.n[2];
+    const long long rows = (long long)nm * ns;
+    const bool open = g.bc == BC_OUTFLOW;
+    const long long of0 = gmap(-1, nf, g.bc);  // to the lower neighbour of a row's first cell
     double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    double dmax = 0.0;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        int cc[3];
-        coords_of(g, idx, cc);
+    long long dmax = 0;  // bits of the largest |div b|
+    double hx[3], ri[3];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        hx[ax] = A.h[ax];
+        ri[ax] = rcp64(hx[ax]);
+    }
+    for (long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += (long long)gridDim.x * 8) {
+        const int m = (int)(row % nm), k = (int)(row / nm);
+        const long long base = row * nf;
+        const long long om = (long long)(gmap(m - 1, nm, g.bc) - m) * nf;
+        const long long oz = (long long)(gmap(k - 1, ns, g.bc) - k) * nm * nf;
         if (A.w[0]) {
-            const double vol = (double)A.w[0][cc[0]] * (double)A.w[1][cc[1]] * (double)A.w[2][cc[2]];
-#pragma unroll
-            for (int f = 0; f < 8; ++f) s[f] += (double)A.in[f][idx] * vol;
-        } else {
-#pragma unroll
-            for (int f = 0; f < 8; ++f) s[f] += (double)A.in[f][idx];
+            if (yf) ri[0] = rcp64(hx[0] = (double)A.w[0][m]);
+            else ri[1] = rcp64(hx[1] = (double)A.w[1][m]);
+            ri[2] = rcp64(hx[2] = (double)A.w[2][k]);
         }
-        bool skip = false;
-        if (g.bc == BC_OUTFLOW)
-            for (int ax = 0; ax < 3; ++ax)
-                if (g.n[ax] > 1 && cc[ax] == 0) skip = true;
-        if (!skip) {
-            double dv = 0.0;
+        const bool skip_row = open && ((nm > 1 && m == 0) || (ns > 1 && k == 0));
+        for (int f = threadIdx.x & 31; f < nf; f += 32) {
+            const long long idx = base + f;
+            const long long of = f > 0 ? -1 : of0;
+            const T v[11] = {__ldg(A.in[0] + idx), __ldg(A.in[1] + idx), __ldg(A.in[2] + idx), __ldg(A.in[3] + idx),
+                             __ldg(A.in[4] + idx), __ldg(A.in[5] + idx), __ldg(A.in[6] + idx), __ldg(A.in[7] + idx),
+                             __ldg(A.in[5] + idx + (yf ? om : of)), __ldg(A.in[6] + idx + (yf ? of : om)),
+                             __ldg(A.in[7] + idx + oz)};
+            double q[11];
+            unsigned odd = 0;
 #pragma unroll
-            for (int ax = 0; ax < 3; ++ax) {
-                const long long lo = idx + (long long)(gmap(cc[ax] - 1, g.n[ax], g.bc) - cc[ax]) * g.st[ax];
-                const double hx = A.w[0] ? (double)A.w[ax][cc[ax]] : A.h[ax];
-                dv += ((double)A.in[5 + ax][idx] - (double)A.in[5 + ax][lo]) / hx;
+            for (int i = 0; i < 11; ++i) q[i] = widen(v[i], odd);
+            if (odd) {
+#pragma unroll
+                for (int i = 0; i < 11; ++i) q[i] = (double)v[i];
             }
-            dmax = fmax(dmax, fabs(dv));
+            if (A.w[0]) {
+                if (yf) ri[1] = rcp64(hx[1] = (double)A.w[1][f]);
+                else ri[0] = rcp64(hx[0] = (double)A.w[0][f]);
+                const double vol = hx[0] * hx[1] * hx[2];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) s[i] += q[i] * vol;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) s[i] += q[i];
+            }
+            if (!skip_row && !(open && nf > 1 && f == 0)) {
+                const double dv = quot64(q[5] - q[8], hx[0], ri[0]) + quot64(q[6] - q[9], hx[1], ri[1]) +
+                                  quot64(q[7] - q[10], hx[2], ri[2]);
+                // (a NaN counts as none, as in fmax)
+                const long long d = __double_as_longlong(fabs(dv));
+                if (d <= 0x7ff0000000000000ll) dmax = max(dmax, d);
+            }
         }
     }
     __shared__ double red[256][9];
     for (int f = 0; f < 8; ++f) red[threadIdx.x][f] = s[f];
-    red[threadIdx.x][8] = dmax;
+    red[threadIdx.x][8] = __longlong_as_double(dmax);
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) {
@@ -239,6 +360,7 @@ template <class T> struct TransArgs {
     T *dst[8];
     int nr, nc;          // source: nc rows of nr elements; destination: nr rows of nc
     int nf;              // number of fields (1..8)
+    int fb;              // fields per block (blocks of one tile along gridDim.z: ceil(nf / fb))
     long long plane;     // elements per z-plane
 };
 
@@ -263,7 +385,10 @@ __global__ void __launch_bounds__(256) transpose4_kernel(TransArgs<T> A)
     static_assert(sizeof(T) == 4, "16-byte accesses of four 4-byte elements");
     __shared__ T tile[2][64][65];
     const int r0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
-    const long long zoff = (long long)blockIdx.z * A.plane;
+    // a grid of few tiles splits the fields over blocks: a block moves one
+    // field after the other, each a round trip to memory
+    const int nb = (A.nf + A.fb - 1) / A.fb, fs = (int)(blockIdx.z % nb) * A.fb, fe = min(fs + A.fb, A.nf);
+    const long long zoff = (long long)(blockIdx.z / nb) * A.plane;
     const int t = threadIdx.x;
     const int lr = t >> 4, l4 = (t & 15) * 4;  // row within a 16-row band, first element of the float4
     float4 v[4];
@@ -275,9 +400,9 @@ __global__ void __launch_bounds__(256) transpose4_kernel(TransArgs<T> A)
                                           : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
-    load(A.src[0]);
+    load(A.src[fs]);
 #pragma unroll 1
-    for (int f = 0; f < A.nf; ++f) {
+    for (int f = fs; f < fe; ++f) {
         const int b = f & 1;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -288,7 +413,7 @@ __global__ void __launch_bounds__(256) transpose4_kernel(TransArgs<T> A)
             row[3] = v[k].w;
         }
         __syncthreads();
-        if (f + 1 < A.nf) load(A.src[f + 1]);
+        if (f + 1 < fe) load(A.src[f + 1]);
         T *__restrict__ dst = A.dst[f] + zoff;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -313,22 +438,23 @@ __global__ void __launch_bounds__(256) transpose_kernel(TransArgs<T> A)
     constexpr int TR = tr_rows<T>(), KL = TR / 8;
     __shared__ T tile[2][TR][33];
     const int r0 = blockIdx.x * 32, c0 = blockIdx.y * TR;
-    const long long zoff = (long long)blockIdx.z * A.plane;
+    const int nb = (A.nf + A.fb - 1) / A.fb, fs = (int)(blockIdx.z % nb) * A.fb, fe = min(fs + A.fb, A.nf);
+    const long long zoff = (long long)(blockIdx.z / nb) * A.plane;
     const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
     const int rl = r0 + tx;
     T v[KL];
 #pragma unroll
     for (int k = 0; k < KL; ++k) {
         const int c = c0 + ty + 8 * k;
-        v[k] = (rl < A.nr && c < A.nc) ? A.src[0][zoff + (long long)c * A.nr + rl] : T(0);
+        v[k] = (rl < A.nr && c < A.nc) ? A.src[fs][zoff + (long long)c * A.nr + rl] : T(0);
     }
 #pragma unroll 1
-    for (int f = 0; f < A.nf; ++f) {
+    for (int f = fs; f < fe; ++f) {
         const int b = f & 1;
 #pragma unroll
         for (int k = 0; k < KL; ++k) tile[b][ty + 8 * k][tx] = v[k];
         __syncthreads();
-        if (f + 1 < A.nf) {
+        if (f + 1 < fe) {
             const T *__restrict__ src = A.src[f + 1] + zoff;
 #pragma unroll
             for (int k = 0; k < KL; ++k) {
