@@ -116,6 +116,26 @@ def test_batch_tuning_options_do_not_change_results(F):
         b.close()
 
 
+@pytest.mark.parametrize("bc", [W.BC_PERIODIC, W.BC_OUTFLOW])
+def test_batch_segments_of_thin_and_long_boxes(F, bc):
+    """Boxes thinner than the stencil beside boxes of several segments (the
+    sweeps of a batch are cut to one length for all its boxes): each against
+    the single-box path, whose segments differ."""
+    ws = [W.random_smooth(*d, seed=90 + i, bc=bc) for i, d in
+          enumerate([(2, 2, 1), (4, 6, 3), (8, 2, 33), (2, 40, 5), (66, 4, 7), (34, 32, 36)])]
+    b = make_batch(F, ws)
+    b.step(0.4, 2)
+    dts = b.last_dt()
+    for i, w in enumerate(ws):
+        box = F.Box(*w.dims, w.gamma, bc=w.bc, precision="fp32", h=w.h)
+        box.set_state(w.state)
+        box.step_cfl(0.4, 2)
+        assert abs(box.last_dt() - dts[i]) <= 1e-6 * dts[i], i
+        assert rel_err(b.get_state(i), box.get_state()) <= 1e-6, i
+        box.close()
+    b.close()
+
+
 def test_batch_rejects_odd_paired_extents(F):
     with pytest.raises(F.FishError) as ei:
         F.Batch([(9, 8, 8)], [1.4], [0])
