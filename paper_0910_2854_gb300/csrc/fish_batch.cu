@@ -19,9 +19,14 @@
 
 #include <algorithm>
 #include <cmath>
+#include <condition_variable>
 #include <cstdio>
+#include <functional>
+#include <memory>
+#include <mutex>
 #include <new>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/fish.h"
@@ -292,6 +297,88 @@ using namespace fish;
 namespace {
 
 constexpr int kCounters = 16;  // work-queue counters per double step (12 sweeps used)
+constexpr long long kStage = 1ll << 21;    // floats of one of the two pinned staging halves (8 MB each)
+constexpr long long kShare = 1ll << 15;    // values a host thread converts at least
+
+// Host threads of one batch for the conversion of its states between the
+// caller's FP64 and the batch's FP32, the larger part of a transfer on one
+// thread.  Created with the first large transfer, joined with the batch.
+class HostThreads {
+public:
+    ~HostThreads()
+    {
+        {
+            std::lock_guard<std::mutex> l(m_);
+            stop_ = true;
+        }
+        go_.notify_all();
+        for (auto &t : threads_) t.join();
+    }
+    // fn(i0, i1) over pieces of [0, n); returns when all are done.  One caller
+    // at a time (a batch is used by one thread).
+    void run(long long n, const std::function<void(long long, long long)> &fn)
+    {
+        const int want = (int)std::min<long long>(n / kShare, 8);
+        if (want > 1 && !started_) start();
+        const int parts = std::min(want, 1 + (int)threads_.size());
+        if (parts <= 1) {
+            fn(0, n);
+            return;
+        }
+        {
+            std::lock_guard<std::mutex> l(m_);
+            fn_ = &fn;
+            n_ = n;
+            parts_ = parts;
+            left_ = parts - 1;
+            ++round_;
+        }
+        go_.notify_all();
+        fn(0, n / parts);
+        std::unique_lock<std::mutex> l(m_);
+        done_.wait(l, [this] { return left_ == 0; });
+        fn_ = nullptr;
+    }
+
+private:
+    void start()
+    {
+        started_ = true;
+        const int n = std::min(8, (int)std::thread::hardware_concurrency()) - 1;
+        try {
+            for (int i = 0; i < n; ++i) threads_.emplace_back([this, i] { work(i + 1); });
+        } catch (...) {  // fewer threads, or none: run() makes do
+        }
+    }
+    void work(int part)
+    {
+        long long seen = 0;
+        for (;;) {
+            const std::function<void(long long, long long)> *fn = nullptr;
+            long long i0 = 0, i1 = 0;
+            {
+                std::unique_lock<std::mutex> l(m_);
+                go_.wait(l, [&] { return stop_ || round_ != seen; });
+                if (stop_) return;
+                seen = round_;
+                if (part >= parts_) continue;
+                fn = fn_;
+                i0 = n_ * part / parts_;
+                i1 = n_ * (part + 1) / parts_;
+            }
+            (*fn)(i0, i1);
+            std::lock_guard<std::mutex> l(m_);
+            if (--left_ == 0) done_.notify_one();
+        }
+    }
+    std::mutex m_;
+    std::condition_variable go_, done_;
+    std::vector<std::thread> threads_;
+    const std::function<void(long long, long long)> *fn_ = nullptr;
+    long long n_ = 0, round_ = 0;
+    int parts_ = 0, left_ = 0;
+    bool started_ = false, stop_ = false;
+};
 
 }  // namespace
 
@@ -326,6 +413,10 @@ struct fish_batch {
     bool t4 = false;              // every box allows the 16-byte transpose
     const float **tsrc = nullptr;  // device tables: per buffer parity, 8 source then 8 destination field pointers
     std::vector<void *> owned;
+    // transfers: two pinned halves of kStage floats, each with the event of its last copy
+    float *stage[2] = {};
+    cudaEvent_t staged[2] = {};
+    HostThreads host;
     bool tables = false;
     bool pending = false;         // minbits hold the CFL minima of the current states
     cudaGraphExec_t gexec = nullptr;
@@ -726,6 +817,16 @@ int batch_ready(fish_batch *b)
     return FISH_OK;
 }
 
+// The pinned staging halves (with the first transfer).
+int batch_stage(fish_batch *b)
+{
+    for (int h = 0; h < 2; ++h) {
+        if (!b->stage[h]) FISH_BCK(b, cudaMallocHost(&b->stage[h], sizeof(float) * kStage), "staging");
+        if (!b->staged[h]) FISH_BCK(b, cudaEventCreateWithFlags(&b->staged[h], cudaEventDisableTiming), "staging");
+    }
+    return FISH_OK;
+}
+
 int batch_flags(fish_batch *b)
 {
     std::vector<unsigned> fl(b->nbox);
@@ -859,13 +960,27 @@ int fish_batch_set_state(fish_batch *b, int box, const double *state)
     if (box < 0 || box >= b->nbox || !state) return bfail(b, FISH_ERR_ARG, "bad box or state");
     if ((r = batch_layout(b, 0))) return r;
     const long long N = (long long)b->dims[3 * box] * b->dims[3 * box + 1] * b->dims[3 * box + 2];
-    std::vector<float> tmp(N);
-    for (int f = 0; f < 8; ++f) {
-        for (long long i = 0; i < N; ++i) tmp[i] = (float)state[f * N + i];
-        float *dst = (f < 5 ? b->fl[b->cu][f] : b->bf[b->cb][f - 5]) + b->off[box];
-        FISH_BCK(b, cudaMemcpyAsync(dst, tmp.data(), sizeof(float) * N, cudaMemcpyHostToDevice, b->stream), "upload");
-        FISH_BCK(b, cudaStreamSynchronize(b->stream), "upload");
+    if ((r = batch_stage(b))) return r;
+    // the state converted piece by piece into the pinned halves, one converted while the other is copied
+    int h = 0;
+    for (long long o = 0; o < 8 * N; h ^= 1) {
+        const long long m = std::min(kStage, 8 * N - o);
+        FISH_BCK(b, cudaEventSynchronize(b->staged[h]), "upload");
+        float *st = b->stage[h];
+        b->host.run(m, [=](long long i0, long long i1) {
+            for (long long i = i0; i < i1; ++i) st[i] = (float)state[o + i];
+        });
+        for (long long p = 0; p < m;) {
+            const int f = (int)((o + p) / N);
+            const long long at = (o + p) % N, cnt = std::min(N - at, m - p);
+            float *dst = (f < 5 ? b->fl[b->cu][f] : b->bf[b->cb][f - 5]) + b->off[box] + at;
+            FISH_BCK(b, cudaMemcpyAsync(dst, st + p, sizeof(float) * cnt, cudaMemcpyHostToDevice, b->stream), "upload");
+            p += cnt;
+        }
+        FISH_BCK(b, cudaEventRecord(b->staged[h], b->stream), "upload");
+        o += m;
     }
+    FISH_BCK(b, cudaStreamSynchronize(b->stream), "upload");
     b->pending = false;
     return FISH_OK;
 }
@@ -877,12 +992,30 @@ int fish_batch_get_state(fish_batch *b, int box, double *state)
     if (box < 0 || box >= b->nbox || !state) return bfail(b, FISH_ERR_ARG, "bad box or state");
     if ((r = batch_layout(b, 0))) return r;
     const long long N = (long long)b->dims[3 * box] * b->dims[3 * box + 1] * b->dims[3 * box + 2];
-    std::vector<float> tmp(N);
-    for (int f = 0; f < 8; ++f) {
-        const float *src = (f < 5 ? b->fl[b->cu][f] : b->bf[b->cb][f - 5]) + b->off[box];
-        FISH_BCK(b, cudaMemcpyAsync(tmp.data(), src, sizeof(float) * N, cudaMemcpyDeviceToHost, b->stream), "download");
-        FISH_BCK(b, cudaStreamSynchronize(b->stream), "download");
-        for (long long i = 0; i < N; ++i) state[f * N + i] = tmp[i];
+    if ((r = batch_stage(b))) return r;
+    // pieces copied into the pinned halves, one converted while the next is copied
+    const auto fetch = [&](long long o, int h) -> int {
+        const long long m = std::min(kStage, 8 * N - o);
+        for (long long p = 0; p < m;) {
+            const int f = (int)((o + p) / N);
+            const long long at = (o + p) % N, cnt = std::min(N - at, m - p);
+            const float *src = (f < 5 ? b->fl[b->cu][f] : b->bf[b->cb][f - 5]) + b->off[box] + at;
+            FISH_BCK(b, cudaMemcpyAsync(b->stage[h] + p, src, sizeof(float) * cnt, cudaMemcpyDeviceToHost, b->stream),
+                     "download");
+            p += cnt;
+        }
+        FISH_BCK(b, cudaEventRecord(b->staged[h], b->stream), "download");
+        return FISH_OK;
+    };
+    int h = 0;
+    if ((r = fetch(0, 0))) return r;
+    for (long long o = 0; o < 8 * N; o += kStage, h ^= 1) {
+        if (o + kStage < 8 * N && (r = fetch(o + kStage, h ^ 1))) return r;
+        FISH_BCK(b, cudaEventSynchronize(b->staged[h]), "download");
+        const float *st = b->stage[h];
+        b->host.run(std::min(kStage, 8 * N - o), [=](long long i0, long long i1) {
+            for (long long i = i0; i < i1; ++i) state[o + i] = st[i];
+        });
     }
     return batch_flags(b);
 }
@@ -965,6 +1098,10 @@ void fish_batch_destroy(fish_batch *b)
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     for (void *p : b->owned) cudaFree(p);
+    for (int h = 0; h < 2; ++h) {
+        if (b->staged[h]) cudaEventDestroy(b->staged[h]);
+        if (b->stage[h]) cudaFreeHost(b->stage[h]);
+    }
     if (b->own) cudaStreamDestroy(b->own);
     delete b;
 }
