@@ -94,7 +94,7 @@ cudaError_t col_fluid_launch(const ColFluidArgs<typename VT<V>::S> &A, cudaStrea
         // the packed FP32 kernels index with int where the box allows it
         constexpr bool I32 = std::is_same<V, P2>::value;
         const bool small = I32 && fits_int(A);
-        if constexpr (I32 && !HSE) {
+        if constexpr (I32) {
             if (A.cfl_min)
                 return small ? fluid_run<V, HSE, GRAV, LIM, FT1, true, false, int>(A, s)
                              : fluid_run<V, HSE, GRAV, LIM, FT1, true, false, long long>(A, s);
@@ -122,7 +122,9 @@ static cudaError_t col_fluid_lim(const ColFluidArgs<typename VT<V>::S> &A, cudaS
     if constexpr (std::is_same<V, P2>::value) {
         // compile-time limiters for the throughput path (an irregular mesh
         // with Van Leer; its other limiters run on the one-column kernels)
-        if constexpr (GRAV != 2) {
+        if constexpr (HSE) {
+            if (A.wd) return cudaErrorInvalidValue;
+        } else if constexpr (GRAV != 2) {
             if (A.wd) {
                 if (A.lim == LIM_VANLEER) return col_fluid_launch<V, HSE, GRAV, LIM_VANLEER, FT1, true>(A, s);
                 return cudaErrorInvalidValue;
@@ -130,7 +132,9 @@ static cudaError_t col_fluid_lim(const ColFluidArgs<typename VT<V>::S> &A, cudaS
         }
         if (A.lim == LIM_VANLEER) return col_fluid_launch<V, HSE, GRAV, LIM_VANLEER, FT1>(A, s);
         if (A.lim == LIM_MINMOD) return col_fluid_launch<V, HSE, GRAV, LIM_MINMOD, FT1>(A, s);
-        if (A.lim == LIM_HYBRID) return col_fluid_launch<V, HSE, GRAV, LIM_HYBRID, FT1>(A, s);
+        if constexpr (!HSE) {
+            if (A.lim == LIM_HYBRID) return col_fluid_launch<V, HSE, GRAV, LIM_HYBRID, FT1>(A, s);
+        }
         return cudaErrorInvalidValue;
     } else {
         // irregular mesh: widths along d (limiter read at run time)
@@ -141,13 +145,6 @@ static cudaError_t col_fluid_lim(const ColFluidArgs<typename VT<V>::S> &A, cudaS
             // the plain FP64 sweeps with a compile-time Van Leer limiter
             if (A.lim == LIM_VANLEER) return col_fluid_launch<V, HSE, GRAV, LIM_VANLEER, FT1>(A, s);
         }
-        if constexpr (HSE && std::is_same<V, float>::value) {
-            // the hydrostatic sweeps (one column per thread): compile-time
-            // limiters (13.2 against 15.4 ms per 384^3 polytrope step with
-            // the limiter read per interface)
-            if (A.lim == LIM_VANLEER) return col_fluid_launch<V, HSE, GRAV, LIM_VANLEER, FT1>(A, s);
-            if (A.lim == LIM_MINMOD) return col_fluid_launch<V, HSE, GRAV, LIM_MINMOD, FT1>(A, s);
-        }
         return col_fluid_launch<V, HSE, GRAV, -1, FT1>(A, s);
     }
 }
@@ -155,19 +152,12 @@ static cudaError_t col_fluid_lim(const ColFluidArgs<typename VT<V>::S> &A, cudaS
 template <class V, bool FT1>
 static cudaError_t col_fluid_ft(const ColFluidArgs<typename VT<V>::S> &A, bool hse, cudaStream_t s)
 {
-    if constexpr (std::is_same<V, P2>::value) {
-        if (hse) return cudaErrorInvalidValue;  // the packed kernels carry no hydrostatic terms
-        if (A.phi && A.sg) return col_fluid_lim<V, false, 2, FT1>(A, s);
-        if (A.phi) return col_fluid_lim<V, false, 1, FT1>(A, s);
-        return col_fluid_lim<V, false, 0, FT1>(A, s);
-    } else {
-        if (hse && A.sg) return cudaErrorInvalidValue;  // split gravity and the correction exclude each other
-        if (hse && A.phi) return col_fluid_lim<V, true, 1, FT1>(A, s);
-        if (hse) return col_fluid_lim<V, true, 0, FT1>(A, s);  // correction with phi = 0
-        if (A.phi && A.sg) return col_fluid_lim<V, false, 2, FT1>(A, s);
-        if (A.phi) return col_fluid_lim<V, false, 1, FT1>(A, s);
-        return col_fluid_lim<V, false, 0, FT1>(A, s);
-    }
+    if (hse && A.sg) return cudaErrorInvalidValue;  // split gravity and the correction exclude each other
+    if (hse && A.phi) return col_fluid_lim<V, true, 1, FT1>(A, s);
+    if (hse) return col_fluid_lim<V, true, 0, FT1>(A, s);  // correction with phi = 0
+    if (A.phi && A.sg) return col_fluid_lim<V, false, 2, FT1>(A, s);
+    if (A.phi) return col_fluid_lim<V, false, 1, FT1>(A, s);
+    return col_fluid_lim<V, false, 0, FT1>(A, s);
 }
 
 template <class V>

@@ -229,26 +229,19 @@ template <class V> __device__ __forceinline__ V pdiff(V phia, V phib)
 template <class V>
 __device__ __forceinline__ void chse(const CCell<V> &a, const CCell<V> &b, V phia, V phib, V du[5], V ddu[5])
 {
-    V xa[5], xb[5];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        xa[i] = -a.u[i];
-        xb[i] = -b.u[i];
-    }
-    xa[4] = -(a.u[4] + a.p);
-    xb[4] = -(b.u[4] + b.p);
-    const V fac = vdiv(pdiff(phia, phib), a.cs * b.cs);
+    // -g = (xi_a + xi_b)/2 fac with xi = -(rho, m, E + p); the factor 1/2 goes
+    // into fac (exact)
+    const V fac = vb<V>(0.5f) * vdiv(pdiff(phia, phib), a.cs * b.cs);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
+        const V s = i < 4 ? b.u[i] + a.u[i] : (b.u[4] + b.p) + (a.u[4] + a.p);
         du[i] = b.u[i] - a.u[i];
         if constexpr (VT<V>::F64) {
-            const V g = 0.5 * (xb[i] + xa[i]) * fac;
-            ddu[i] = vminmod(du[i] - g, du[i]);
+            ddu[i] = vminmod(du[i] + s * fac, du[i]);
         } else {
-            const V sx = vb<V>(0.5f) * (xb[i] + xa[i]);
-            const V ghi = sx * fac;
-            const V glo = vfma(sx, fac, -ghi);
-            ddu[i] = vminmod((du[i] - ghi) - glo, du[i]);
+            const V ghi = s * fac;
+            const V glo = vfma(s, fac, -ghi);
+            ddu[i] = vminmod((du[i] + ghi) + glo, du[i]);
         }
     }
 }
@@ -284,14 +277,16 @@ __device__ __forceinline__ void cflux1(const CCell<V> &a, const CCell<V> &b, V p
 
 // second-order TVD flux at the interface c1|c2 from predicted cells c0..c3
 // (eq0160-eq0230; one freezing speed per interface, reading C-2; HSE form of
-// the slope differences, reading C-19).  The hybrid limiter is taken only by
+// the slope differences, reading C-19, from the jumps du, dd of chse at the
+// three interfaces of the stencil).  The hybrid limiter is taken only by
 // the one-column kernels with the limiter read at run time.
 // NU (irregular mesh, reading C-25): each one-sided difference is divided
 // by the distance of the centres it joins and the limited slope carried
 // over half the width of its own cell (w1 for F+, w2 for F-).
 template <class V, bool HSE, int LIM, bool NU = false>
 __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, const CCell<V> &c2, const CCell<V> &c3,
-                                       V ph0, V ph1, V ph2, V ph3, V F[5], int lim, V w0 = V(), V w1 = V(),
+                                       const V du0[5], const V dd0[5], const V du1[5], const V dd1[5],
+                                       const V du2[5], const V dd2[5], V F[5], int lim, V w0 = V(), V w1 = V(),
                                        V w2 = V(), V w3 = V())
 {
     V gl = w0, gc = w1, gr = w2;
@@ -362,10 +357,6 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
         const V half = vb<V>(0.5f);
         const V Dadv = vmax(vabs(c1.vn), vabs(c2.vn));
         const V Dac = vmax(c1.cf, c2.cf);
-        V du0[5], dd0[5], du1[5], dd1[5], du2[5], dd2[5];
-        chse(c0, c1, ph0, ph1, du0, dd0);
-        chse(c1, c2, ph1, ph2, du1, dd1);
-        chse(c2, c3, ph2, ph3, du2, dd2);
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             const V q0 = Dadv * du0[i] + Dac * dd0[i];
@@ -447,6 +438,7 @@ template <class V> struct FMarch {
     CCell<V> P[4];       // predicted cells (slot index mod 4)
     V q[4];              // their potential
     V F2[2][5];          // corrector fluxes
+    V hu[2][5], hd[2][5];  // HSE: jumps of the predicted cells at (r-3, r-2), (r-2, r-1) (slot r & 1)
     V phm2;              // potential of raw cell r-2
     Checks<V> chk;
     V cflr;              // largest CFL rate of the output cells (CFLF)
@@ -769,9 +761,19 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         if (PHI || HSE) M.q[s3] = M.ph[p2];
         // corrector flux at (r-3, r-2) from predicted cells r-4 .. r-1 (eq0230)
         constexpr int s0 = K & 3, s1 = (K + 1) & 3, s2 = (K + 2) & 3;
+        // (the jumps of its two older interfaces are those of the last two steps)
+        V du2[5], dd2[5];
+        if constexpr (HSE) chse(M.P[s2], M.P[s3], M.q[s2], M.q[s3], du2, dd2);
         if (!VT<V>::F64 || r >= a + 2)  // (FP64, bound by its pipe, skips the fluxes no output cell uses)
-        cflux2<V, HSE, LIM, NU>(M.P[s0], M.P[s1], M.P[s2], M.P[s3], M.q[s0], M.q[s1], M.q[s2], M.q[s3], M.F2[k2],
-                                A.lim, vb<V>(M.w4), vb<V>(M.w3), vb<V>(M.w2), vb<V>(M.w1));
+            cflux2<V, HSE, LIM, NU>(M.P[s0], M.P[s1], M.P[s2], M.P[s3], M.hu[k2], M.hd[k2], M.hu[p2], M.hd[p2], du2,
+                                    dd2, M.F2[k2], A.lim, vb<V>(M.w4), vb<V>(M.w3), vb<V>(M.w2), vb<V>(M.w1));
+        if constexpr (HSE) {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                M.hu[k2][k] = du2[k];
+                M.hd[k2][k] = dd2[k];
+            }
+        }
         V lo = lam;
         if constexpr (NU) {
             if constexpr (VT<V>::F64) lo = flux_scale<V, HSE>() * (dt / M.w3);
@@ -875,7 +877,7 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
         M.q[i] = zero;
         M.P[i].d = M.P[i].p = M.P[i].cs = M.P[i].cf = M.P[i].vn = zero;
 #pragma unroll
-        for (int k = 0; k < 5; ++k) M.P[i].u[k] = M.P[i].F[k] = M.F2[i & 1][k] = zero;
+        for (int k = 0; k < 5; ++k) M.P[i].u[k] = M.P[i].F[k] = M.F2[i & 1][k] = M.hu[i & 1][k] = M.hd[i & 1][k] = zero;
     }
     fload_mapped<V, GRAV != 0, FT1, IX>(A, X, a - 3, M.R);
     if constexpr (GRAV == 2) {
@@ -932,7 +934,7 @@ template <class V> constexpr int fluid_threads() { return VT<V>::F64 ? 32 : 128;
 // Blocks per SM the kernels are compiled for.
 template <class V, bool HSE> constexpr int fluid_resident()
 {
-    return VT<V>::F64 ? 8 : (VT<V>::W == 2 || HSE ? FISH_COL_MINB : FISH_COL_MINB1);
+    return VT<V>::F64 ? 8 : (VT<V>::W == 2 ? FISH_COL_MINB : FISH_COL_MINB1);
 }
 
 // Grid: column blocks x segments of `len` cells.

@@ -41,15 +41,17 @@ static inline bool frame_of(const Geom &g, int d, Frame &F)
     return true;
 }
 
-// The two-column FP32 kernels are used for even fast extents without the
-// hydrostatic correction and with the Van Leer, minmod or hybrid limiter.
+// The two-column FP32 kernels are used for even fast extents with the Van
+// Leer, minmod or hybrid limiter (the hydrostatic correction: Van Leer or
+// minmod on a uniform mesh; an irregular mesh: Van Leer).
 template <class T> static bool uses_pairs(const Frame &F, int lim, bool hse, bool nu = false)
 {
 #ifdef FISH_FLUID_SCALAR
     return false;
 #else
-    if (nu && lim != LIM_VANLEER) return false;
-    return sizeof(T) == 4 && F.nf % 2 == 0 && !hse && (lim == LIM_VANLEER || lim == LIM_MINMOD || lim == LIM_HYBRID);
+    if (nu && (hse || lim != LIM_VANLEER)) return false;
+    if (hse && lim == LIM_HYBRID) return false;
+    return sizeof(T) == 4 && F.nf % 2 == 0 && (lim == LIM_VANLEER || lim == LIM_MINMOD || lim == LIM_HYBRID);
 #endif
 }
 
@@ -114,7 +116,7 @@ cudaError_t Launch<T>::fluid(const T *const in[8], T *const out[5], const T *phi
         // two columns per thread (packed FP32x2) when the fast extent is even;
         // the ring-fed march if asked for and it applies
         if (uses_pairs<T>(F, lim, hse, w3 != nullptr)) {
-            if (kernels == 1) {
+            if (kernels == 1 && !hse) {
                 const cudaError_t e = ring_fluid(A, s);
                 if (e != cudaErrorNotSupported) return e;
             }

@@ -191,8 +191,8 @@ __device__ __forceinline__ void rstep(const ColFluidArgs<float> &A, FRing &R, FM
         if constexpr ((ST & ST_F2) != 0) {
             // corrector flux at (r-3, r-2) from predicted cells r-4 .. r-1 (eq0230)
             constexpr int s0 = K & 3, s1 = (K + 1) & 3, s2 = (K + 2) & 3;
-            const P2 z = vb<P2>(0.f);
-            cflux2<P2, false, LIM, false>(M.P[s0], M.P[s1], M.P[s2], M.P[s3], z, z, z, z, M.F2[k2], A.lim);
+            cflux2<P2, false, LIM, false>(M.P[s0], M.P[s1], M.P[s2], M.P[s3], nullptr, nullptr, nullptr, nullptr,
+                                          nullptr, nullptr, M.F2[k2], A.lim);
             if constexpr ((ST & ST_OUT) != 0) {
 #pragma unroll
                 for (int k = 0; k < 5; ++k) un[k] = vfma(-lam, M.F2[k2][k] - M.F2[p2][k], un[k]);
