@@ -88,10 +88,10 @@ template <class V> struct CCell {
     V p, cs, cf, vn;     // used by the hydrostatic correction only
 };
 
-// running checks for reading C-16: min rho, min p, and a sum of c_F that
-// turns NaN if any evaluated cell produced one
+// running checks for reading C-16: min rho and min p, both keeping a NaN (a
+// NaN of any input makes p one, and p > 0 and rho > 0 leave c_F real)
 template <class V> struct Checks {
-    V mn_rho, mn_p, nsum;
+    V mn_rho, mn_p;
     int hi;   // FP64: FLAG_* seen, by the bits of rho, p and c_F
 };
 
@@ -99,20 +99,19 @@ template <class V> __device__ __forceinline__ void checks_init(Checks<V> &k)
 {
     k.mn_rho = vb<V>(3.0e38f);
     k.mn_p = vb<V>(3.0e38f);
-    k.nsum = vb<V>(0.0f);
     k.hi = 0;
 }
 
 template <class V> __device__ __forceinline__ unsigned checks_flags(const Checks<V> &k)
 {
-    unsigned f = 0;
     if constexpr (VT<V>::F64) return (unsigned)k.hi;
+    unsigned f = 0;
 #pragma unroll
     for (int i = 0; i < VT<V>::W; ++i) {
-        const auto r = vget(k.mn_rho, i), p = vget(k.mn_p, i), s = vget(k.nsum, i);
-        if (!(r > 0)) f |= FLAG_RHO;
-        if (!(p > 0)) f |= FLAG_P;
-        if (s != s) f |= FLAG_NAN;
+        const auto r = vget(k.mn_rho, i), p = vget(k.mn_p, i);
+        if (r <= 0) f |= FLAG_RHO;
+        if (p <= 0) f |= FLAG_P;
+        if (r != r || p != p) f |= FLAG_NAN;
     }
     return f;
 }
@@ -206,9 +205,8 @@ __device__ __forceinline__ void ceval(const V u[5], const V bb[3], V gamma, V gm
         if (!pos64(p)) k.hi |= FLAG_P;
         if ((__double2hiint(c.cf) & 0x7fffffff) > 0x7ff00000) k.hi |= FLAG_NAN;
     } else {
-        k.mn_rho = vmin(k.mn_rho, rho);
-        k.mn_p = vmin(k.mn_p, p);
-        k.nsum = k.nsum + c.cf;
+        k.mn_rho = vminnan(k.mn_rho, rho);
+        k.mn_p = vminnan(k.mn_p, p);
     }
 }
 
@@ -247,9 +245,9 @@ __device__ __forceinline__ void chse(const CCell<V> &a, const CCell<V> &b, V phi
 }
 
 // first-order interface flux: eq0140 with D = alpha max(d_a, d_b) (eq0150),
-// or the HSE-corrected form eq0324 (reading C-3).  FP64 without the correction
-// gives twice the flux (flux_scale: the factor is exact and goes into dt/dx).
-template <class V, bool HSE> constexpr double flux_scale() { return VT<V>::F64 && !HSE ? 0.5 : 1.0; }
+// or the HSE-corrected form eq0324 (reading C-3).  Fluxes are carried doubled:
+// the 1/2 of the mean and of the dissipation, exact, goes into dt/dx.
+constexpr double FLUX_SCALE = 0.5;
 template <class V, bool HSE>
 __device__ __forceinline__ void cflux1(const CCell<V> &a, const CCell<V> &b, V phia, V phib, V alpha, V F[5])
 {
@@ -259,19 +257,16 @@ __device__ __forceinline__ void cflux1(const CCell<V> &a, const CCell<V> &b, V p
 #pragma unroll
             for (int i = 0; i < 5; ++i) F[i] = (a.F[i] + b.F[i]) - D * (b.u[i] - a.u[i]);
         } else {
-            const V half = vb<V>(0.5f);
 #pragma unroll
-            for (int i = 0; i < 5; ++i) F[i] = half * vfma(-D, b.u[i] - a.u[i], a.F[i] + b.F[i]);
+            for (int i = 0; i < 5; ++i) F[i] = vfma(-D, b.u[i] - a.u[i], a.F[i] + b.F[i]);
         }
     } else {
         V du[5], ddu[5];
         const V Dadv = alpha * vmax(vabs(a.vn), vabs(b.vn));
         const V Dac = alpha * vmax(a.cf, b.cf);
         chse(a, b, phia, phib, du, ddu);
-        const V half = vb<V>(0.5f);
 #pragma unroll
-        for (int i = 0; i < 5; ++i)
-            F[i] = half * (a.F[i] + b.F[i]) - half * Dadv * du[i] - half * Dac * ddu[i];
+        for (int i = 0; i < 5; ++i) F[i] = vfma(-Dac, ddu[i], vfma(-Dadv, du[i], a.F[i] + b.F[i]));
     }
 }
 
@@ -307,7 +302,7 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
     V sup = vb<V>(0.0f);
     if constexpr (LIM == LIM_HYBRID) sup = vmax(vabs(c1.vn) - c1.cs, vabs(c2.vn) - c2.cs);
     if constexpr (!HSE && !VT<V>::F64) {
-        // FP32: F = (F_e + F_{e+1})/2 - D du_e/2 + [phi(+) - phi(-)]/4 with the
+        // FP32: 2 F = F_e + F_{e+1} - D du_e + [phi(+) - phi(-)]/2 with the
         // split-flux slopes written as dF +- D du (each one multiply-add)
         const V D = vmax(c1.d, c2.d);
         const V nD = -D;
@@ -318,18 +313,18 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
             const V df2 = c3.F[i] - c2.F[i], du2 = c3.u[i] - c2.u[i];
             V slp, slm;
             if constexpr (NU) {
-                slp = w1 * vlimit<LIM>(vdiv(vfma(D, du0, df0), gl), vdiv(vfma(D, du1, df1), gc), lim);
-                slm = w2 * vlimit<LIM>(vdiv(vfma(nD, du1, df1), gc), vdiv(vfma(nD, du2, df2), gr), lim);
+                slp = w1 * vlimit_half<LIM>(vdiv(vfma(D, du0, df0), gl), vdiv(vfma(D, du1, df1), gc), lim);
+                slm = w2 * vlimit_half<LIM>(vdiv(vfma(nD, du1, df1), gc), vdiv(vfma(nD, du2, df2), gr), lim);
             } else if constexpr (LIM == LIM_HYBRID) {
                 const V ap = vfma(D, du0, df0), bp = vfma(D, du1, df1);
                 const V am = vfma(nD, du1, df1), bm = vfma(nD, du2, df2);
-                slp = vsel_pos(sup, vminmod(ap, bp), vvanleer(ap, bp));
-                slm = vsel_pos(sup, vminmod(am, bm), vvanleer(am, bm));
+                slp = vsel_pos(sup, vhalf(vminmod(ap, bp)), vvanleer_half(ap, bp));
+                slm = vsel_pos(sup, vhalf(vminmod(am, bm)), vvanleer_half(am, bm));
             } else {
-                slp = vlimit<LIM>(vfma(D, du0, df0), vfma(D, du1, df1), lim);
-                slm = vlimit<LIM>(vfma(nD, du1, df1), vfma(nD, du2, df2), lim);
+                slp = vlimit_half<LIM>(vfma(D, du0, df0), vfma(D, du1, df1), lim);
+                slm = vlimit_half<LIM>(vfma(nD, du1, df1), vfma(nD, du2, df2), lim);
             }
-            F[i] = vfma(vb<V>(0.5f), vfma(nD, du1, c1.F[i] + c2.F[i]), vb<V>(0.25f) * (slp - slm));
+            F[i] = vfma(nD, du1, c1.F[i] + c2.F[i]) + (slp - slm);
         }
     } else if constexpr (!HSE) {
         const V D = vmax(c1.d, c2.d);
@@ -354,7 +349,6 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
             F[i] = fp1 + fm2 + (slp - slm);
         }
     } else {
-        const V half = vb<V>(0.5f);
         const V Dadv = vmax(vabs(c1.vn), vabs(c2.vn));
         const V Dac = vmax(c1.cf, c2.cf);
 #pragma unroll
@@ -362,30 +356,20 @@ __device__ __forceinline__ void cflux2(const CCell<V> &c0, const CCell<V> &c1, c
             const V q0 = Dadv * du0[i] + Dac * dd0[i];
             const V q1 = Dadv * du1[i] + Dac * dd1[i];
             const V q2 = Dadv * du2[i] + Dac * dd2[i];
-            const V fp_l = half * ((c1.F[i] - c0.F[i]) + q0);
-            const V fp_r = half * ((c2.F[i] - c1.F[i]) + q1);
-            const V fm_l = half * ((c2.F[i] - c1.F[i]) - q1);
-            const V fm_r = half * ((c3.F[i] - c2.F[i]) - q2);
+            // twice the one-sided differences of F+ and F-, and half their limited slopes
+            const V fp_l = (c1.F[i] - c0.F[i]) + q0;
+            const V fp_r = (c2.F[i] - c1.F[i]) + q1;
+            const V fm_l = (c2.F[i] - c1.F[i]) - q1;
+            const V fm_r = (c3.F[i] - c2.F[i]) - q2;
             V slp, slm;
-            if constexpr (VT<V>::F64) {
-                // (half the limited slopes)
-                if constexpr (NU) {
-                    slp = w1 * vlimit_half<LIM>(fp_l / gl, fp_r / gc, lim);
-                    slm = w2 * vlimit_half<LIM>(fm_l / gc, fm_r / gr, lim);
-                } else {
-                    slp = vlimit_half<LIM>(fp_l, fp_r, lim);
-                    slm = vlimit_half<LIM>(fm_l, fm_r, lim);
-                }
-                F[i] = half * (c1.F[i] + c2.F[i]) - half * q1 + (slp - slm);
-                continue;
-            } else if constexpr (NU) {
-                slp = w1 * vlimit<LIM>(vdiv(fp_l, gl), vdiv(fp_r, gc), lim);
-                slm = w2 * vlimit<LIM>(vdiv(fm_l, gc), vdiv(fm_r, gr), lim);
+            if constexpr (NU) {
+                slp = w1 * vlimit_half<LIM>(vdiv(fp_l, gl), vdiv(fp_r, gc), lim);
+                slm = w2 * vlimit_half<LIM>(vdiv(fm_l, gc), vdiv(fm_r, gr), lim);
             } else {
-                slp = vlimit<LIM>(fp_l, fp_r, lim);
-                slm = vlimit<LIM>(fm_l, fm_r, lim);
+                slp = vlimit_half<LIM>(fp_l, fp_r, lim);
+                slm = vlimit_half<LIM>(fm_l, fm_r, lim);
             }
-            F[i] = half * (c1.F[i] + c2.F[i]) - half * q1 + half * (slp - slm);
+            F[i] = (c1.F[i] + c2.F[i]) - q1 + (slp - slm);
         }
     }
 }
@@ -732,8 +716,8 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         V up[5];
         V lh = lamh;
         if constexpr (NU) {
-            if constexpr (VT<V>::F64) lh = flux_scale<V, HSE>() * (dt / (2.0 * M.w1));
-            else lh = vdiv(hdt, vb<V>(M.w1));
+            if constexpr (VT<V>::F64) lh = FLUX_SCALE * (dt / (2.0 * M.w1));
+            else lh = vdiv(vb<V>(0.5f) * hdt, vb<V>(M.w1));
         }
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
@@ -776,8 +760,8 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         }
         V lo = lam;
         if constexpr (NU) {
-            if constexpr (VT<V>::F64) lo = flux_scale<V, HSE>() * (dt / M.w3);
-            else lo = vdiv(dt, vb<V>(M.w3));
+            if constexpr (VT<V>::F64) lo = FLUX_SCALE * (dt / M.w3);
+            else lo = vdiv(hdt, vb<V>(M.w3));
         }
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
@@ -860,8 +844,8 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     }
     const double dtd = *A.dt;
     const V dt = vb<V>(S(dtd));
-    const V lam = vb<V>(S(flux_scale<V, HSE>() * (dtd / A.h)));
-    const V lamh = vb<V>(S(flux_scale<V, HSE>() * (dtd / (2.0 * A.h))));
+    const V lam = vb<V>(S(FLUX_SCALE * (dtd / A.h)));
+    const V lamh = vb<V>(S(FLUX_SCALE * (dtd / (2.0 * A.h))));
     const V hdt = vb<V>(S(0.5 * dtd));
     const V rtwoh = vb<V>(S(1.0 / (2.0 * A.h)));
 
@@ -1065,8 +1049,8 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
                 const V la = vsel_pos(vbar, d0, d1);
                 const V lb = vsel_pos(vbar, d1, d2);
                 const V base = vsel_pos(vbar, w0, w1);
-                const V sg = vsel_pos(vbar, half * cw.w4, -half * cw.w3);
-                P.f[e] = vfma(sg, vlimit<LIM>(la, lb, lim), base);
+                const V sg = vsel_pos(vbar, cw.w4, -cw.w3);
+                P.f[e] = vfma(sg, vlimit_half<LIM>(la, lb, lim), base);
             }
         } else {
             // select the upwind operands, then limit once
@@ -1074,8 +1058,8 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
             const V la = vsel_pos(vbar, d0, d1);
             const V lb = vsel_pos(vbar, d1, d2);
             const V base = vsel_pos(vbar, w0, w1);
-            const V sg = vsel_pos(vbar, vb<V>(0.5f), vb<V>(-0.5f));
-            P.f[e] = vfma(sg, vlimit<LIM>(la, lb, lim), base);
+            const V sg = vsel_pos(vbar, vb<V>(1.0f), vb<V>(-1.0f));
+            P.f[e] = vfma(sg, vlimit_half<LIM>(la, lb, lim), base);
         }
         if constexpr (OUT) {
             V lo = lam;

@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(RF_THREADS, 256 / RF_THREADS) fluid_ring_kerne
         for (int q = -3; q <= -3 + FISH_RING_L && q <= n + 2; ++q) rf_produce(A, R, q);
     }
     const double dtd = *A.dt;
-    const P2 lam = vb<P2>(float(dtd / A.h));
-    const P2 lamh = vb<P2>(float(dtd / (2.0 * A.h)));
+    const P2 lam = vb<P2>(float(FLUX_SCALE * (dtd / A.h)));
+    const P2 lamh = vb<P2>(float(FLUX_SCALE * (dtd / (2.0 * A.h))));
 
     FMarch<P2> M;
     checks_init(M.chk);

@@ -85,16 +85,34 @@ __device__ __forceinline__ P2 vmax(P2 a, P2 b) { return {make_float2(fmaxf(a.v.x
 
 __device__ __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
+// minimum that keeps a NaN of either operand
+__device__ __forceinline__ float sminnan(float a, float b)
+{
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float vminnan(float a, float b) { return sminnan(a, b); }
+__device__ __forceinline__ P2 vminnan(P2 a, P2 b)
+{
+    return {make_float2(sminnan(a.v.x, b.v.x), sminnan(a.v.y, b.v.y))};
+}
 __device__ __forceinline__ P2 vmin(P2 a, P2 b) { return {make_float2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y))}; }
 
-// reciprocal: IEEE in FP64, the fast hardware reciprocal (about 1 ulp) in FP32
+// reciprocal: IEEE in FP64, the hardware's (1 ulp) in FP32
+__device__ __forceinline__ float srcp(float a)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
 __device__ __forceinline__ double vrcp(double a) { return 1.0 / a; }
-__device__ __forceinline__ float vrcp(float a) { return __fdividef(1.0f, a); }
-__device__ __forceinline__ P2 vrcp(P2 a) { return {make_float2(__fdividef(1.0f, a.v.x), __fdividef(1.0f, a.v.y))}; }
+__device__ __forceinline__ float vrcp(float a) { return srcp(a); }
+__device__ __forceinline__ P2 vrcp(P2 a) { return {make_float2(srcp(a.v.x), srcp(a.v.y))}; }
 
 // quotient: IEEE in FP64, a * rcp(b) in FP32
 __device__ __forceinline__ double vdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ float vdiv(float a, float b) { return __fmul_rn(a, __fdividef(1.0f, b)); }
+__device__ __forceinline__ float vdiv(float a, float b) { return __fmul_rn(a, srcp(b)); }
 __device__ __forceinline__ P2 vdiv(P2 a, P2 b) { return a * vrcp(b); }
 
 // select: c > 0 ? a : b, per component
@@ -166,34 +184,31 @@ __device__ __forceinline__ double vvanleer_half(double a, double b)
     const double q = quot64(ab, c, rcp64(c));
     return pos64(ab) ? q : 0.0;
 }
-__device__ __forceinline__ float vvanleer(float a, float b)
+__device__ __forceinline__ float vvanleer_half(float a, float b)
 {
     const float ab = __fmul_rn(a, b);
-    return ab > 0.0f ? __fmul_rn(ab + ab, __fdividef(1.0f, a + b)) : 0.0f;
+    return ab > 0.0f ? __fmul_rn(ab, srcp(a + b)) : 0.0f;
 }
-__device__ __forceinline__ P2 vvanleer(P2 a, P2 b)
+__device__ __forceinline__ P2 vvanleer_half(P2 a, P2 b)
 {
     const P2 ab = a * b;
-    const P2 q = (ab + ab) * vrcp(a + b);
+    const P2 q = ab * vrcp(a + b);
     return {make_float2(ab.v.x > 0.0f ? q.v.x : 0.0f, ab.v.y > 0.0f ? q.v.y : 0.0f)};
 }
 
 // limiter: 0 Van Leer, 1 minmod, 2 none (first order); LIM < 0 selects at
-// run time from lim
-template <int LIM, class V> __device__ __forceinline__ V vlimit(V a, V b, int lim)
-{
-    if constexpr (LIM == 0) return vvanleer(a, b);
-    else if constexpr (LIM == 1) return vminmod(a, b);
-    else if constexpr (LIM == 2) return vb<V>(0);
-    else return lim == 0 ? vvanleer(a, b) : (lim == 1 ? vminmod(a, b) : vb<V>(0));
-}
-// half the limiter, FP64
-template <int LIM> __device__ __forceinline__ double vlimit_half(double a, double b, int lim)
+// run time from lim.
+// Half the limiter, ab / (a + b) for Van Leer: the factor 2 cancels against
+// the 1/2 of the fluxes it enters.
+__device__ __forceinline__ double vhalf(double a) { return 0.5 * a; }
+__device__ __forceinline__ float vhalf(float a) { return 0.5f * a; }
+__device__ __forceinline__ P2 vhalf(P2 a) { return vb<P2>(0.5f) * a; }
+template <int LIM, class V> __device__ __forceinline__ V vlimit_half(V a, V b, int lim)
 {
     if constexpr (LIM == 0) return vvanleer_half(a, b);
-    else if constexpr (LIM == 1) return 0.5 * vminmod(a, b);
-    else if constexpr (LIM == 2) return 0.0;
-    else return lim == 0 ? vvanleer_half(a, b) : (lim == 1 ? 0.5 * vminmod(a, b) : 0.0);
+    else if constexpr (LIM == 1) return vhalf(vminmod(a, b));
+    else if constexpr (LIM == 2) return vb<V>(0);
+    else return lim == 0 ? vvanleer_half(a, b) : (lim == 1 ? vhalf(vminmod(a, b)) : vb<V>(0));
 }
 
 // ---- memory access -----------------------------------------------------------
