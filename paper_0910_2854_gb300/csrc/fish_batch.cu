@@ -56,7 +56,9 @@ struct BatchItem {
     int a, b;
 };
 
-template <int LIM, bool CFLF>
+// (IX as in the single-box sweeps: 32-bit byte offsets, or int indices for a
+// batch of more than 2^30 cells)
+template <int LIM, bool CFLF, class IX>
 __global__ void __launch_bounds__(128, FISH_COL_MINB)
     fluid_batch_kernel(const ColFluidArgs<float> A, const BatchBox *__restrict__ boxes,
                        const BatchItem *__restrict__ items, int nitems, int *counter, const double *dt,
@@ -99,13 +101,13 @@ __global__ void __launch_bounds__(128, FISH_COL_MINB)
         if (groups == 0) return;
         const int first = I.first;
         for (int g = 0; g < groups; ++g)
-            fluid_columns<P2, false, false, LIM, true, CFLF, false, int, false>(Ab, (long long)first + 128ll * g + threadIdx.x, I.a, I.b);
+            fluid_columns<P2, false, false, LIM, true, CFLF, false, IX, false>(Ab, (long long)first + 128ll * g + threadIdx.x, I.a, I.b);
     }
 }
 
 // ROWS: warps per work-item group, each on one of ROWS consecutive rows of a
 // segment (the tile height; blocks of 32 * ROWS threads)
-template <int LIM, int ROWS>
+template <int LIM, int ROWS, class IX>
 __global__ void __launch_bounds__(32 * ROWS, FISH_CT_MINB * 4 / ROWS)
     ct_batch_kernel(const ColCTArgs<float> A, const BatchBox *__restrict__ boxes,
                     const BatchItem *__restrict__ items, int nitems, int *counter, const double *dt)
@@ -149,7 +151,7 @@ __global__ void __launch_bounds__(32 * ROWS, FISH_CT_MINB * 4 / ROWS)
         for (int g = 0; g < groups; ++g) {
             const long long q = (long long)first / ROWS + g;
             const long long ob = (q / nseg) * ROWS + (threadIdx.x >> 5);
-            ct_columns<float, LIM, true>(Ab, ob * nseg + q % nseg, threadIdx.x & 31, I.a, I.b);
+            ct_columns<float, LIM, true, false, IX>(Ab, ob * nseg + q % nseg, threadIdx.x & 31, I.a, I.b);
         }
     }
 }
@@ -707,20 +709,17 @@ int batch_fluid(fish_batch *b, int d, bool cfl, int counter)
     A.alpha = 1.0f;
     const int grid = b->fluid_blocks;
     int *ctr = b->counters + counter;
-    if (b->lim == FISH_LIM_VANLEER) {
-        if (cfl)
-            fluid_batch_kernel<LIM_VANLEER, true><<<grid, 128, 0, b->stream>>>(
-                A, b->boxes[d], b->fitems[d], b->nfitems[d], ctr, b->dt, b->flags, b->minbits);
-        else
-            fluid_batch_kernel<LIM_VANLEER, false><<<grid, 128, 0, b->stream>>>(
-                A, b->boxes[d], b->fitems[d], b->nfitems[d], ctr, b->dt, b->flags, b->minbits);
+    const auto launch = [&](auto kernel) {
+        kernel<<<grid, 128, 0, b->stream>>>(A, b->boxes[d], b->fitems[d], b->nfitems[d], ctr, b->dt, b->flags,
+                                            b->minbits);
+    };
+    const bool vl = b->lim == FISH_LIM_VANLEER;
+    if (b->total <= (1ll << 30)) {
+        if (vl) launch(cfl ? fluid_batch_kernel<LIM_VANLEER, true, unsigned> : fluid_batch_kernel<LIM_VANLEER, false, unsigned>);
+        else launch(cfl ? fluid_batch_kernel<LIM_MINMOD, true, unsigned> : fluid_batch_kernel<LIM_MINMOD, false, unsigned>);
     } else {
-        if (cfl)
-            fluid_batch_kernel<LIM_MINMOD, true><<<grid, 128, 0, b->stream>>>(
-                A, b->boxes[d], b->fitems[d], b->nfitems[d], ctr, b->dt, b->flags, b->minbits);
-        else
-            fluid_batch_kernel<LIM_MINMOD, false><<<grid, 128, 0, b->stream>>>(
-                A, b->boxes[d], b->fitems[d], b->nfitems[d], ctr, b->dt, b->flags, b->minbits);
+        if (vl) launch(cfl ? fluid_batch_kernel<LIM_VANLEER, true, int> : fluid_batch_kernel<LIM_VANLEER, false, int>);
+        else launch(cfl ? fluid_batch_kernel<LIM_MINMOD, true, int> : fluid_batch_kernel<LIM_MINMOD, false, int>);
     }
     FISH_BCK(b, cudaGetLastError(), "batch fluid launch");
     b->cu = 1 - b->cu;
@@ -746,21 +745,16 @@ int batch_ct(fish_batch *b, int d, int counter)
     A.boo = b->bf[1 - b->cb][other];
     A.lim = b->lim;
     int *ctr = b->counters + counter;
-    const bool vl = b->lim == FISH_LIM_VANLEER;
-    if (b->ctrows == 8) {
-        if (vl)
-            ct_batch_kernel<LIM_VANLEER, 8><<<b->ct_blocks, 256, 0, b->stream>>>(A, b->boxes[d], b->citems[d],
-                                                                               b->ncitems[d], ctr, b->dt);
-        else
-            ct_batch_kernel<LIM_MINMOD, 8><<<b->ct_blocks, 256, 0, b->stream>>>(A, b->boxes[d], b->citems[d],
-                                                                              b->ncitems[d], ctr, b->dt);
+    const auto launch = [&](auto kernel) {
+        kernel<<<b->ct_blocks, 32 * b->ctrows, 0, b->stream>>>(A, b->boxes[d], b->citems[d], b->ncitems[d], ctr, b->dt);
+    };
+    const bool vl = b->lim == FISH_LIM_VANLEER, r8 = b->ctrows == 8;
+    if (b->total <= (1ll << 30)) {
+        if (vl) launch(r8 ? ct_batch_kernel<LIM_VANLEER, 8, unsigned> : ct_batch_kernel<LIM_VANLEER, 4, unsigned>);
+        else launch(r8 ? ct_batch_kernel<LIM_MINMOD, 8, unsigned> : ct_batch_kernel<LIM_MINMOD, 4, unsigned>);
     } else {
-        if (vl)
-            ct_batch_kernel<LIM_VANLEER, 4><<<b->ct_blocks, 128, 0, b->stream>>>(A, b->boxes[d], b->citems[d],
-                                                                               b->ncitems[d], ctr, b->dt);
-        else
-            ct_batch_kernel<LIM_MINMOD, 4><<<b->ct_blocks, 128, 0, b->stream>>>(A, b->boxes[d], b->citems[d],
-                                                                              b->ncitems[d], ctr, b->dt);
+        if (vl) launch(r8 ? ct_batch_kernel<LIM_VANLEER, 8, int> : ct_batch_kernel<LIM_VANLEER, 4, int>);
+        else launch(r8 ? ct_batch_kernel<LIM_MINMOD, 8, int> : ct_batch_kernel<LIM_MINMOD, 4, int>);
     }
     FISH_BCK(b, cudaGetLastError(), "batch constrained-transport launch");
     b->cb = 1 - b->cb;
@@ -1035,13 +1029,13 @@ int fish_batch_step(fish_batch *b, double k, int nsteps)
         }
         // persistent grids: every resident block slot, times the tuning factor
         int occ_f = 0, occ_c = 0;
-        FISH_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, fluid_batch_kernel<LIM_VANLEER, true>, 128, 0),
+        FISH_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, (fluid_batch_kernel<LIM_VANLEER, true, unsigned>), 128, 0),
                  "occupancy");
         if (b->ctrows == 8)
-            FISH_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, ct_batch_kernel<LIM_VANLEER, 8>, 256, 0),
+            FISH_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, (ct_batch_kernel<LIM_VANLEER, 8, unsigned>), 256, 0),
                      "occupancy");
         else
-            FISH_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, ct_batch_kernel<LIM_VANLEER, 4>, 128, 0),
+            FISH_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, (ct_batch_kernel<LIM_VANLEER, 4, unsigned>), 128, 0),
                      "occupancy");
         b->fluid_blocks = std::max(1, occ_f) * b->sms * b->grid_factor;
         b->ct_blocks = std::max(1, occ_c) * b->sms * b->grid_factor;

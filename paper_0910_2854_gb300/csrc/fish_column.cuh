@@ -430,8 +430,17 @@ template <class V> struct FMarch {
     V dprev;             // split gravity: potential (FP64) or its difference (FP32) of raw cell r-1
 };
 
-// IX: element index type (int where every index of the launch fits, else
-// long long): a load then costs one wide multiply-add for its address.
+// stride along the sweep as an IX
+template <class IX, class S> __device__ __forceinline__ IX ix_sd(const ColFluidArgs<S> &A)
+{
+    return (IX)A.sd * ix_unit<S, IX>();
+}
+template <class IX, class S> __device__ __forceinline__ IX ix_sd(const ColCTArgs<S> &A)
+{
+    return (IX)A.sd * ix_unit<S, IX>();
+}
+// IX: how elements are addressed, long long indices or (unsigned) 32-bit byte
+// offsets where all fit.
 template <class S, class IX = long long> struct FCtx {
     IX base;             // offset of cell 0 of the first column
     IX ofm;              // offset of the fast-axis face below the first column
@@ -460,14 +469,15 @@ __device__ __forceinline__ void fpf_setup(const ColFluidArgs<S> &A, const S *bfp
     if (r >= (grav ? 10 : 9)) return;
     const S *f = r < 5 ? A.u[r] : (r == 5 ? A.bd : (r == 6 ? bfp : (r == 9 ? A.phi : bop)));
     const IX r0 = base0 + (r == 8 ? oom0 : (IX)0);
-    const IX line = (r0 & ~(IX)31) + (IX)(32 * (lane & 1));
-    if (line <= r0 + (IX)(span - 1)) P.p = f + line;
+    constexpr IX un = ix_unit<S, IX>();
+    const IX line = (r0 & ~((IX)31 * un)) + (IX)(32 * (lane & 1)) * un;
+    if (line <= r0 + (IX)(span - 1) * un) P.p = ix_at(f, line);
 }
 
 template <class S, class IX>
 __device__ __forceinline__ void fpf_step(const ColFluidArgs<S> &A, const FPf<S, IX> &P, int c)
 {
-    if (P.p) pf_l2(P.p + (IX)c * (IX)A.sd);
+    if (P.p) pf_l2(ix_at(P.p, (IX)c * ix_sd<IX>(A)));
 }
 
 // load raw cell s (any s): every index through the boundary map; a ghost
@@ -477,22 +487,22 @@ __device__ __forceinline__ void fload_mapped(const ColFluidArgs<typename VT<V>::
                                              const FCtx<typename VT<V>::S, IX> &X, int s, FRaw<V> &R)
 {
     const int cc = gmap(s, A.n, A.bc);
-    const IX i = X.base + (IX)cc * (IX)A.sd;
-    const IX im = X.base + (IX)gmap(cc - 1, A.n, A.bc) * (IX)A.sd;
+    const IX i = X.base + (IX)cc * ix_sd<IX>(A);
+    const IX im = X.base + (IX)gmap(cc - 1, A.n, A.bc) * ix_sd<IX>(A);
     const auto *bfp = FT1 ? A.bt1 : A.bt2;
     const auto *bop = FT1 ? A.bt2 : A.bt1;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) R.u[k] = vload<V>(A.u[k], i);
-    R.bd = vload<V>(A.bd, i);
-    R.bdm = vload<V>(A.bd, im);
-    R.bf = vload<V>(bfp, i);
-    R.bfm = __ldg(bfp + i + X.ofm);
-    R.bo = vload<V>(bop, i);
-    R.bom = vload<V>(bop, i + X.oom);
+    for (int k = 0; k < 5; ++k) R.u[k] = vget_at<V>(A.u[k], i);
+    R.bd = vget_at<V>(A.bd, i);
+    R.bdm = vget_at<V>(A.bd, im);
+    R.bf = vget_at<V>(bfp, i);
+    R.bfm = __ldg(ix_at(bfp, i + X.ofm));
+    R.bo = vget_at<V>(bop, i);
+    R.bom = vget_at<V>(bop, i + X.oom);
     if (GRAV) {
         // FP32 reads the difference to the next cell: zero between the copies
         // of an outflow boundary cell (and across its face)
-        R.phi = vload<V>(A.phi, i);
+        R.phi = vget_at<V>(A.phi, i);
         if constexpr (!VT<V>::F64)
             if (A.bc == BC_OUTFLOW && (s < 0 || s >= A.n)) R.phi = vb<V>(0.0f);
     }
@@ -523,27 +533,27 @@ __device__ __forceinline__ void fload_next(const ColFluidArgs<typename VT<V>::S>
     const auto *bfp = FT1 ? A.bt1 : A.bt2;
     const auto *bop = FT1 ? A.bt2 : A.bt1;
     const int cc = wrap_cell(c, A.n, A.bc);
-    const IX i = X.base + (IX)cc * (IX)A.sd;
+    const IX i = X.base + (IX)cc * ix_sd<IX>(A);
     if (!(c >= A.n && A.bc == BC_OUTFLOW)) R.bdm = R.bd;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) R.u[k] = vload<V>(A.u[k], i);
-    R.bd = vload<V>(A.bd, i);
-    R.bf = vload<V>(bfp, i);
-    R.bfm = __ldg(bfp + i + X.ofm);
-    R.bo = vload<V>(bop, i);
-    R.bom = vload<V>(bop, i + X.oom);
+    for (int k = 0; k < 5; ++k) R.u[k] = vget_at<V>(A.u[k], i);
+    R.bd = vget_at<V>(A.bd, i);
+    R.bf = vget_at<V>(bfp, i);
+    R.bfm = __ldg(ix_at(bfp, i + X.ofm));
+    R.bo = vget_at<V>(bop, i);
+    R.bom = vget_at<V>(bop, i + X.oom);
     if constexpr (PHI) {
-        R.phi = vload<V>(A.phi, i);
+        R.phi = vget_at<V>(A.phi, i);
         if constexpr (!VT<V>::F64)
             if (c != cc && A.bc == BC_OUTFLOW) R.phi = vb<V>(0.0f);
     }
     if constexpr (NU) R.w = A.wd[cc];
 }
 
-// L2 prefetch distance of the steady-state loops (cells ahead of the load)
-#ifndef FISH_PF_DIST
-#define FISH_PF_DIST 2
-#endif
+// L2 prefetch distance of the fluid march (cells ahead of the load): four in
+// long segments (2552 -> 2513 us at 640^3), two in short ones, which belong to
+// boxes that fit in L2 and would fetch the next segment's cells.
+__device__ __forceinline__ int pf_dist(int len) { return len >= 96 ? 4 : 2; }
 
 #ifndef FISH_FL_PF_NEIGH
 #define FISH_FL_PF_NEIGH 1   // also the lower other-axis face (a neighbour row)
@@ -556,14 +566,14 @@ __device__ __forceinline__ void fprefetch(const ColFluidArgs<typename VT<V>::S> 
     const auto *bfp = FT1 ? A.bt1 : A.bt2;
     const auto *bop = FT1 ? A.bt2 : A.bt1;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) pf_l2(A.u[k] + i);
-    pf_l2(A.bd + i);
-    pf_l2(bfp + i);
-    pf_l2(bop + i);
+    for (int k = 0; k < 5; ++k) pf_l2(ix_at(A.u[k], i));
+    pf_l2(ix_at(A.bd, i));
+    pf_l2(ix_at(bfp, i));
+    pf_l2(ix_at(bop, i));
 #if FISH_FL_PF_NEIGH
-    pf_l2(bop + i + X.oom);
+    pf_l2(ix_at(bop, i + X.oom));
 #endif
-    if (GRAV) pf_l2(A.phi + i);
+    if (GRAV) pf_l2(ix_at(A.phi, i));
 }
 
 // Stages of a march step: the evaluation of the raw cell alone, with the
@@ -599,13 +609,13 @@ __device__ __forceinline__ V sg_image_dk(const ColFluidArgs<typename VT<V>::S> &
 {
     const int cc = gmap(r, A.n, A.bc);
     if constexpr (VT<V>::F64) {
-        const V pp = vload<V>(A.phi, X.base + (IX)gmap(cc + 1, A.n, A.bc) * (IX)A.sd);
-        const V pm = vload<V>(A.phi, X.base + (IX)gmap(cc - 1, A.n, A.bc) * (IX)A.sd);
+        const V pp = vget_at<V>(A.phi, X.base + (IX)gmap(cc + 1, A.n, A.bc) * ix_sd<IX>(A));
+        const V pm = vget_at<V>(A.phi, X.base + (IX)gmap(cc - 1, A.n, A.bc) * ix_sd<IX>(A));
         return (pp - pm) / (2.0 * A.h);
     } else {
-        const V dc = vload<V>(A.phi, X.base + (IX)cc * (IX)A.sd);
+        const V dc = vget_at<V>(A.phi, X.base + (IX)cc * ix_sd<IX>(A));
         V dl = vb<V>(0.0f);
-        if (cc > 0 || A.bc == BC_PERIODIC) dl = vload<V>(A.phi, X.base + (IX)gmap(cc - 1, A.n, A.bc) * (IX)A.sd);
+        if (cc > 0 || A.bc == BC_PERIODIC) dl = vget_at<V>(A.phi, X.base + (IX)gmap(cc - 1, A.n, A.bc) * ix_sd<IX>(A));
         return (dc + dl) * rtwoh;
     }
 }
@@ -629,7 +639,7 @@ static __shared__ float2 cfl_bb_ring[4 * 3 * 128];
 template <class V, bool HSE, int GM, int LIM, bool FT1, bool CFLF, bool NU, int K, int ST, class IX = long long,
           bool PFW = FISH_FL_PF_WARP != 0>
 __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, const FCtx<typename VT<V>::S, IX> &X,
-                                      FMarch<V> &M, int r, int a, V lam, V lamh, V hdt, V dt, V rtwoh,
+                                      FMarch<V> &M, int r, int a, int pfd, V lam, V lamh, V hdt, V dt, V rtwoh,
                                       const FPf<typename VT<V>::S, IX> &PF)
 {
     constexpr bool GRAV = GM == 1, SG = GM == 2, PHI = GM != 0;
@@ -669,21 +679,21 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
     // load raw cell r+1
     fload_next<V, PHI, FT1, NU, IX>(A, X, r + 1, M.R);
     if constexpr (ST == ST_ALL) {
-        const int pf = min(r + 1 + FISH_PF_DIST, A.n - 1);
+        const int pf = min(r + 1 + pfd, A.n - 1);
         if constexpr (PFW) fpf_step(A, PF, pf);
-        else fprefetch<V, PHI, FT1, IX>(A, X, X.base + (IX)pf * (IX)A.sd);
+        else fprefetch<V, PHI, FT1, IX>(A, X, X.base + (IX)pf * ix_sd<IX>(A));
     }
     // old state of the output cell o = r-3
     const int o = r - 3;
     const bool out = ST == ST_ALL && o >= a;
-    const IX io = X.base + (IX)o * (IX)A.sd;
+    const IX io = X.base + (IX)o * ix_sd<IX>(A);
     V un[5];
     if constexpr (ST == ST_ALL) {
 #pragma unroll
         for (int k = 0; k < 5; ++k) un[k] = ur[k];
         if (out) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) un[k] = vload<V>(A.u[k], io);
+            for (int k = 0; k < 5; ++k) un[k] = vget_at<V>(A.u[k], io);
         }
     }
     if constexpr (SG) {
@@ -786,7 +796,7 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
         if constexpr (SG) sg_kick<V>(un, M.q[s1], hdt);  // output cell: second half kick
         if (out) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) vstore(A.uo[k], io, un[k]);
+            for (int k = 0; k < 5; ++k) vstore(ix_at(A.uo[k], io), 0, un[k]);
             if constexpr (CFLF) {
                 // CFL rate of the updated cell with its cell-centred field,
                 // formed when the cell entered as raw cell o = r-3 (slot
@@ -827,9 +837,10 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     const int fp = (int)(cid % cols), ob = (int)(cid / cols);
     const int f0 = fp * W;
     FCtx<S, IX> X;
-    X.base = (IX)A.off + (IX)f0 + (IX)ob * (IX)A.so;
-    X.ofm = (IX)(gmap(f0 - 1, A.nf, A.bc) - f0);
-    X.oom = (IX)(gmap(ob - 1, A.no, A.bc) - ob) * (IX)A.so;
+    constexpr IX un = ix_unit<S, IX>();
+    X.base = ((IX)A.off + (IX)f0 + (IX)ob * (IX)A.so) * un;
+    X.ofm = (IX)(gmap(f0 - 1, A.nf, A.bc) - f0) * un;
+    X.oom = (IX)(gmap(ob - 1, A.no, A.bc) - ob) * (IX)A.so * un;
     // per-warp L2 prefetch over the span of the warp's first lane (32 groups
     // of W columns; a warp that crosses a row end prefetches its first row)
     FPf<S, IX> PF;
@@ -839,7 +850,7 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
         const int l0 = __ffs(am) - 1;
         const IX b0 = __shfl_sync(am, X.base, l0);
         const IX m0 = __shfl_sync(am, X.oom, l0);
-        const int span = min(32 * W, A.nf - (int)(b0 - (IX)A.off) % A.nf);
+        const int span = min(32 * W, A.nf - (int)(b0 / un - (IX)A.off) % A.nf);
         fpf_setup(A, FT1 ? A.bt1 : A.bt2, FT1 ? A.bt2 : A.bt1, b0, m0, span, GRAV != 0, (int)(threadIdx.x & 31), PF);
     }
     const double dtd = *A.dt;
@@ -849,6 +860,7 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     const V hdt = vb<V>(S(0.5 * dtd));
     const V rtwoh = vb<V>(S(1.0 / (2.0 * A.h)));
 
+    const int pfd = pf_dist(b - a);
     FMarch<V> M;
     checks_init(M.chk);
     const V zero = vb<V>(0.0f);
@@ -873,20 +885,20 @@ __device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>:
     if constexpr (PFW) {
         // the first cells, so that their loads do not each wait for memory
 #pragma unroll
-        for (int c = -2; c < FISH_PF_DIST; ++c) fpf_step(A, PF, max(min(a + c, A.n - 1), 0));
+        for (int c = -2; c < 2; ++c) fpf_step(A, PF, max(min(a + c, A.n - 1), 0));
     }
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_RAW, IX, PFW>(A, X, M, a - 3, a, lam, lamh, hdt, dt, rtwoh, PF);
-    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_FLUX, IX, PFW>(A, X, M, a - 2, a, lam, lamh, hdt, dt, rtwoh, PF);
+    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_RAW, IX, PFW>(A, X, M, a - 3, a, pfd, lam, lamh, hdt, dt, rtwoh, PF);
+    fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_FLUX, IX, PFW>(A, X, M, a - 2, a, pfd, lam, lamh, hdt, dt, rtwoh, PF);
     const int last = b + 2;
 #pragma unroll 1
     for (int r = a - 1;; r += 4) {
-        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ST_ALL, IX, PFW>(A, X, M, r, a, lam, lamh, hdt, dt, rtwoh, PF);
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 3, ST_ALL, IX, PFW>(A, X, M, r, a, pfd, lam, lamh, hdt, dt, rtwoh, PF);
         if (r >= last) break;
-        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ST_ALL, IX, PFW>(A, X, M, r + 1, a, lam, lamh, hdt, dt, rtwoh, PF);
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 0, ST_ALL, IX, PFW>(A, X, M, r + 1, a, pfd, lam, lamh, hdt, dt, rtwoh, PF);
         if (r + 1 >= last) break;
-        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_ALL, IX, PFW>(A, X, M, r + 2, a, lam, lamh, hdt, dt, rtwoh, PF);
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 1, ST_ALL, IX, PFW>(A, X, M, r + 2, a, pfd, lam, lamh, hdt, dt, rtwoh, PF);
         if (r + 2 >= last) break;
-        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_ALL, IX, PFW>(A, X, M, r + 3, a, lam, lamh, hdt, dt, rtwoh, PF);
+        fstep<V, HSE, GRAV, LIM, FT1, CFLF, NU, 2, ST_ALL, IX, PFW>(A, X, M, r + 3, a, pfd, lam, lamh, hdt, dt, rtwoh, PF);
         if (r + 3 >= last) break;
     }
     const unsigned fl = checks_flags(M.chk);
@@ -1080,8 +1092,8 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
 // lane beneath it, whose edge flux arrives by a warp shuffle.  Raw inputs of
 // cell s+1 are loaded while cell s is computed.
 // ---------------------------------------------------------------------------
-// IX: element index type (int where every index of the launch fits, else
-// long long); a load then costs one wide multiply-add for its address.
+// IX: how elements are addressed, long long indices or (unsigned) 32-bit byte
+// offsets where all fit.
 template <class S, class IX = long long> struct CTCtx {
     IX base;             // element offset of the lane's first column in cell 0
     IX ofp;              // offset to the fast-axis column above the lane's last column
@@ -1116,33 +1128,33 @@ __device__ __forceinline__ void ctload(const ColCTArgs<typename VT<V>::S> &A, co
                                        int s, CTRaw<V> &R)
 {
     const int sm = wrap_cell(s, A.n, A.bc);
-    const IX i = X.base + (IX)sm * (IX)A.sd;
+    const IX i = X.base + (IX)sm * ix_sd<IX>(A);
     if constexpr (NU) R.w = A.wd[sm];  // a ghost has the width of its image (reading C-23)
-    R.rc = vload<V>(A.rho, i);
-    R.mc = vload<V>(A.md, i);
-    R.ro = vload<V>(A.rho, i + X.oop);
-    R.mo = vload<V>(A.md, i + X.oop);
-    R.rm = vload<V>(A.rho, i + X.oom);
-    R.mm = vload<V>(A.md, i + X.oom);
-    R.rf = __ldg(A.rho + i + X.ofp);
-    R.mf = __ldg(A.md + i + X.ofp);
-    R.bF = vload<V>(A.bf, i);
-    R.bO = vload<V>(A.bo, i);
-    R.bOm = vload<V>(A.bo, i + X.oom);
+    R.rc = vget_at<V>(A.rho, i);
+    R.mc = vget_at<V>(A.md, i);
+    R.ro = vget_at<V>(A.rho, i + X.oop);
+    R.mo = vget_at<V>(A.md, i + X.oop);
+    R.rm = vget_at<V>(A.rho, i + X.oom);
+    R.mm = vget_at<V>(A.md, i + X.oom);
+    R.rf = __ldg(ix_at(A.rho, i + X.ofp));
+    R.mf = __ldg(ix_at(A.md, i + X.ofp));
+    R.bF = vget_at<V>(A.bf, i);
+    R.bO = vget_at<V>(A.bo, i);
+    R.bOm = vget_at<V>(A.bo, i + X.oom);
     if constexpr (VT<V>::W == 2) {
         if (X.fixy) {
             fixy_(R.rc, true); fixy_(R.mc, true); fixy_(R.ro, true); fixy_(R.mo, true);
             fixy_(R.rm, true); fixy_(R.mm, true); fixy_(R.bF, true); fixy_(R.bO, true); fixy_(R.bOm, true);
         }
     }
-    R.bdo = vload<V>(A.bd, X.base + (IX)max(min(s - 4, A.n - 1), 0) * (IX)A.sd);
+    R.bdo = vget_at<V>(A.bd, X.base + (IX)max(min(s - 4, A.n - 1), 0) * ix_sd<IX>(A));
 }
 
 // prefetch into L2 the fields of interior cell i (the neighbour rows too
 // with FISH_CT_PF_NEIGH: with the warps of a block on consecutive rows they
 // are mostly the own rows of sibling warps)
 #ifndef FISH_CT_PF_DIST
-#define FISH_CT_PF_DIST 1
+#define FISH_CT_PF_DIST 2   // against 1: 156 -> 148 us at 256^3, 2161 -> 2035 us at 640^3
 #endif
 #ifndef FISH_CT_PF_NEIGH
 #define FISH_CT_PF_NEIGH 1
@@ -1151,18 +1163,18 @@ template <class V, class IX = long long>
 __device__ __forceinline__ void ctprefetch(const ColCTArgs<typename VT<V>::S> &A,
                                            const CTCtx<typename VT<V>::S, IX> &X, IX i)
 {
-    pf_l2(A.rho + i);
-    pf_l2(A.md + i);
+    pf_l2(ix_at(A.rho, i));
+    pf_l2(ix_at(A.md, i));
 #if FISH_CT_PF_NEIGH
-    pf_l2(A.rho + i + X.oom);
-    pf_l2(A.md + i + X.oom);
-    pf_l2(A.rho + i + X.oop);
-    pf_l2(A.md + i + X.oop);
-    pf_l2(A.bo + i + X.oom);
+    pf_l2(ix_at(A.rho, i + X.oom));
+    pf_l2(ix_at(A.md, i + X.oom));
+    pf_l2(ix_at(A.rho, i + X.oop));
+    pf_l2(ix_at(A.md, i + X.oop));
+    pf_l2(ix_at(A.bo, i + X.oom));
 #endif
-    pf_l2(A.bf + i);
-    pf_l2(A.bo + i);
-    pf_l2(A.bd + i);
+    pf_l2(ix_at(A.bf, i));
+    pf_l2(ix_at(A.bo, i));
+    pf_l2(ix_at(A.bd, i));
 }
 
 // FP32 one-column CT (uniform mesh): the two face pencils above a column,
@@ -1218,7 +1230,7 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
     const V bdo = M.R.bdo;
     // load cell s+1
     ctload<V, NU, IX>(A, X, s + 1, M.R);
-    ctprefetch<V, IX>(A, X, X.base + (IX)max(min(s + 1 + FISH_CT_PF_DIST, A.n - 1), 0) * (IX)A.sd);
+    ctprefetch<V, IX>(A, X, X.base + (IX)max(min(s + 1 + FISH_CT_PF_DIST, A.n - 1), 0) * ix_sd<IX>(A));
     const V half = vb<V>(0.5f);
     // face velocities (eq0361): the mean of the two cells across the face,
     // or on an irregular mesh their linear interpolation to it (reading C-27)
@@ -1272,9 +1284,9 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
         if constexpr (VT<V>::W == 2) fdn = vshift_lo(sh.v.y, fup);
         else fdn = sh;
         if (X.active && s - 4 >= a) {
-            const IX io = X.base + (IX)(s - 4) * (IX)A.sd;
-            vstore(A.bfo, io, nF);
-            vstore(A.boo, io, nO);
+            const IX io = X.base + (IX)(s - 4) * ix_sd<IX>(A);
+            vstore(ix_at(A.bfo, io), 0, nF);
+            vstore(ix_at(A.boo, io), 0, nO);
             const V tF = fup - fdn, tO = fpo - M.POm.f[e];
             V r;
             if constexpr (VT<V>::F64) {
@@ -1283,7 +1295,7 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
             } else {
                 r = vfma(lamo, tO, vfma(lamf, tF, bdo));
             }
-            vstore(A.bdo, io, r);
+            vstore(ix_at(A.bdo, io), 0, r);
         }
     }
 }
@@ -1322,10 +1334,11 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
         X.fixy = W == 2;
     }
     const int cfp = gmap(cl + W, A.nf, A.bc);
-    X.base = (IX)A.off + (IX)cb + (IX)ob * (IX)A.so;
-    X.ofp = (IX)(cfp - cb);
-    X.oom = (IX)(gmap(ob - 1, A.no, A.bc) - ob) * (IX)A.so;
-    X.oop = (IX)(gmap(ob + 1, A.no, A.bc) - ob) * (IX)A.so;
+    constexpr IX un = ix_unit<S, IX>();
+    X.base = ((IX)A.off + (IX)cb + (IX)ob * (IX)A.so) * un;
+    X.ofp = (IX)(cfp - cb) * un;
+    X.oom = (IX)(gmap(ob - 1, A.no, A.bc) - ob) * (IX)A.so * un;
+    X.oop = (IX)(gmap(ob + 1, A.no, A.bc) - ob) * (IX)A.so * un;
     const double dtd = *A.dt;
     const V dtv = vb<V>(S(dtd));
     constexpr double sc = VT<V>::F64 ? CT_SCALE : 1.0;

@@ -221,6 +221,24 @@ template <> __device__ __forceinline__ P2 vload<P2>(const float *p, long long i)
     return {__ldg(reinterpret_cast<const float2 *>(p + i))};
 }
 
+// Element positions: an index (long long, or int where all fit), or as
+// `unsigned` a byte offset from the field's start, which the load takes beside
+// the field's address without arithmetic of its own.
+template <class S, class IX> __device__ __forceinline__ constexpr IX ix_unit() { return (IX)1; }
+template <> __device__ __forceinline__ constexpr unsigned ix_unit<float, unsigned>() { return 4u; }
+template <> __device__ __forceinline__ constexpr unsigned ix_unit<double, unsigned>() { return 8u; }
+template <class S, class IX> __device__ __forceinline__ S *ix_at(S *p, IX i)
+{
+    if constexpr (sizeof(IX) == 4 && (IX)-1 > (IX)0)
+        return reinterpret_cast<S *>(reinterpret_cast<uintptr_t>(p) + i);
+    else
+        return p + i;
+}
+template <class V, class IX> __device__ __forceinline__ V vget_at(const typename VT<V>::S *p, IX i)
+{
+    return vload<V>(ix_at(p, i), 0);
+}
+
 // Hint that the line holding p will be read soon: fetch it into L2 (no
 // register is written and nothing waits for it).
 __device__ __forceinline__ void pf_l2(const void *p) { asm volatile("prefetch.L2 [%0];" ::"l"(p)); }
