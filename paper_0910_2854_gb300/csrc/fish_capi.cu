@@ -917,29 +917,45 @@ int planes_check(fish_ctx *c, int k0, int nk, const void *buf)
     return FISH_OK;
 }
 
-int fish_get_planes(fish_ctx *c, int k0, int nk, void *dst)
+// Copy the planes between the fields and the buffer: one kernel for a buffer
+// in the memory of the fields' own device, else a copy per field.
+static int planes_copy(fish_ctx *c, int k0, int nk, char *buf, bool get)
 {
-    int r = planes_check(c, k0, nk, dst);
-    if (r) return r;
-    const size_t es = esize(c), plane = (size_t)c->n[0] * c->n[1];
+    const size_t plane = (size_t)c->n[0] * c->n[1] * esize(c), bytes = (size_t)nk * plane;
+    if (nk == 0) return FISH_OK;
+    char *fld[8], *out[8];
+    for (int f = 0; f < 8; ++f) {
+        fld[f] = (char *)field_ptr(c, f) + (size_t)k0 * plane;
+        out[f] = buf + (size_t)f * bytes;
+    }
+    cudaPointerAttributes pb, pf;
+    const bool known = cudaPointerGetAttributes(&pb, buf) == cudaSuccess &&
+                       cudaPointerGetAttributes(&pf, fld[0]) == cudaSuccess;
+    if (!known) (void)cudaGetLastError();
+    if (known && pb.type == cudaMemoryTypeDevice && pf.type == cudaMemoryTypeDevice && pb.device == pf.device) {
+        const void *const *src = (const void *const *)(get ? fld : out);
+        void *const *dst = (void *const *)(get ? out : fld);
+        FISH_CK(c, fish::launch_copy8(src, dst, bytes, c->stream), "plane copy");
+        c->launches += 1;
+        return FISH_OK;
+    }
     for (int f = 0; f < 8; ++f)
-        FISH_CK(c, cudaMemcpyAsync((char *)dst + (size_t)f * nk * plane * es,
-                                   (const char *)field_ptr(c, f) + (size_t)k0 * plane * es, (size_t)nk * plane * es,
-                                   cudaMemcpyDefault, c->stream),
+        FISH_CK(c, cudaMemcpyAsync(get ? out[f] : fld[f], get ? fld[f] : out[f], bytes, cudaMemcpyDefault, c->stream),
                 "plane copy");
     return FISH_OK;
+}
+
+int fish_get_planes(fish_ctx *c, int k0, int nk, void *dst)
+{
+    const int r = planes_check(c, k0, nk, dst);
+    return r ? r : planes_copy(c, k0, nk, (char *)dst, true);
 }
 
 int fish_set_planes(fish_ctx *c, int k0, int nk, const void *src)
 {
     int r = planes_check(c, k0, nk, src);
     if (r) return r;
-    const size_t es = esize(c), plane = (size_t)c->n[0] * c->n[1];
-    for (int f = 0; f < 8; ++f)
-        FISH_CK(c, cudaMemcpyAsync((char *)field_ptr(c, f) + (size_t)k0 * plane * es,
-                                   (const char *)src + (size_t)f * nk * plane * es, (size_t)nk * plane * es,
-                                   cudaMemcpyDefault, c->stream),
-                "plane copy");
+    if ((r = planes_copy(c, k0, nk, (char *)const_cast<void *>(src), false))) return r;
     c->cfl_pending = false;  // the state changed outside a graph replay
     return FISH_OK;
 }

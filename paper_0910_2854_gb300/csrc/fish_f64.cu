@@ -37,6 +37,45 @@ cudaError_t launch_cfl_finish(unsigned long long *minbits, double k, double *dt,
     return cudaGetLastError();
 }
 
+// Eight contiguous copies in one launch (blockIdx.y: the field), in units of U:
+// the plane slabs of a ghost exchange are small, and a copy each costs more in
+// launches than in traffic.
+template <class U> struct Copy8Args {
+    const U *src[8];
+    U *dst[8];
+    size_t n;
+};
+template <class U> static __global__ void __launch_bounds__(256) copy8_kernel(const Copy8Args<U> A)
+{
+    const U *src = A.src[blockIdx.y];
+    U *dst = A.dst[blockIdx.y];
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < A.n; i += (size_t)gridDim.x * blockDim.x)
+        dst[i] = src[i];
+}
+template <class U>
+static cudaError_t copy8(const void *const src[8], void *const dst[8], size_t n, cudaStream_t s)
+{
+    Copy8Args<U> A;
+    for (int f = 0; f < 8; ++f) {
+        A.src[f] = (const U *)src[f];
+        A.dst[f] = (U *)dst[f];
+    }
+    A.n = n / sizeof(U);
+    const size_t blocks = (A.n + 1023) / 1024;
+    copy8_kernel<U><<<dim3((unsigned)(blocks < 1 ? 1 : (blocks < 608 ? blocks : 608)), 8), 256, 0, s>>>(A);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy8(const void *const src[8], void *const dst[8], size_t n, cudaStream_t s)
+{
+    // 16 bytes at a time where every slab is so aligned, else words
+    size_t al = n;
+    for (int f = 0; f < 8; ++f) al |= (size_t)src[f] | (size_t)dst[f];
+    if (al % 16 == 0) return copy8<uint4>(src, dst, n, s);
+    if (al % 4 == 0) return copy8<unsigned>(src, dst, n, s);
+    return copy8<unsigned char>(src, dst, n, s);
+}
+
 static __global__ void reset_min_kernel(unsigned long long *p) { *p = 0x7FF0000000000000ull; }
 
 cudaError_t launch_reset_min(unsigned long long *minbits, cudaStream_t s)

@@ -46,6 +46,8 @@ template <class T> struct Launch {
     static cudaError_t to_f32(const T *src, float *dst, long long n, cudaStream_t s);
 };
 
+// copy n bytes from src[f] to dst[f] for the 8 fields in one kernel (device buffers)
+cudaError_t launch_copy8(const void *const src[8], void *const dst[8], size_t n, cudaStream_t s);
 cudaError_t launch_cfl_finish(unsigned long long *minbits, double k, double *dt, double *dt_copy,
                               cudaStream_t s);
 cudaError_t launch_set_scalar(double *p, double v, cudaStream_t s);

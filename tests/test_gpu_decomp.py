@@ -54,3 +54,36 @@ def test_single_rank_slab_equals_single_box(F, precision):
         assert float(np.max(np.abs(got - exp) / scale)) <= 2e-6
     box.close()
     ref.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("dims", [(5, 3, 7), (8, 4, 6), (33, 1, 9)])
+def test_planes_to_device_host_and_unaligned_buffers(F, precision, dims):
+    """Plane slabs through a device buffer (one kernel, 16-byte units or, from
+    an odd offset or odd planes, words) and a host buffer (copies) are the
+    state's planes, and write back to where they came from."""
+    import torch
+    w = W.random_smooth(*dims, seed=12)
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    box = F.Box(*dims, w.gamma, bc=w.bc, precision=precision, h=w.h)
+    box.set_state(w.state)
+    ref = torch.as_tensor(box.get_state()).to(dt)
+    nx, ny, nz = dims
+    for k0, nk in ((0, 1), (1, 2), (nz - 1, 1), (0, nz), (2, 0)):
+        n = 8 * nk * nx * ny
+        for buf in (torch.zeros(n + 1, dtype=dt, device="cuda")[:n], torch.zeros(n + 1, dtype=dt, device="cuda")[1:],
+                    torch.zeros(n, dtype=dt).pin_memory()):
+            if n == 0 and buf.data_ptr() == 0:
+                continue
+            torch.cuda.synchronize()
+            box.get_planes(k0, nk, buf)
+            box.sync()
+            assert torch.equal(buf.cpu().reshape(8, nk, ny, nx), ref[:, k0:k0 + nk])
+            buf.mul_(2.0)
+            torch.cuda.synchronize()
+            box.set_planes(k0, nk, buf)
+            box.sync()
+            got = torch.as_tensor(box.get_state()).to(dt)
+            assert torch.equal(got[:, k0:k0 + nk], 2.0 * ref[:, k0:k0 + nk])
+            box.set_state(w.state)
+    box.close()
