@@ -48,6 +48,12 @@ struct fish_ctx {
     void *bf[2][3] = {};   // face fields b_x, b_y, b_z (two buffers)
     int cu = 0, cb = 0;    // current buffer of each group
     int layout = 0;        // 0: x fastest (y, z sweeps); 1: y fastest (x sweeps)
+    // Whether callers of the plane copies are to find x fastest although the
+    // fields are y fastest: the state was handed over, or read, x fastest, and
+    // no operator has run since
+    bool x_fastest = false;
+    bool fresh = false;    // a state was set and nothing has needed a layout yet
+    int first_need = 1;    // the layout that was needed first after the last fish_set_state*
     void *phi = nullptr;   // FP64: potential, x-fastest layout
     void *phiT = nullptr;  // FP64: potential, y-fastest layout
     void *phiD[3] = {};    // FP32: phi(next cell along d) - phi(cell) formed in FP64, in the layout of the d sweeps
@@ -217,9 +223,47 @@ template <class T> int transpose_state(fish_ctx *c)
 
 int set_layout(fish_ctx *c, int layout)
 {
+    c->x_fastest = false;
+    if (c->fresh) c->first_need = layout;
+    c->fresh = false;
     if (c->layout == layout) return FISH_OK;
     // a layout change is only needed when both sizes are > 1
     return c->prec == FISH_PREC_FP64 ? transpose_state<double>(c) : transpose_state<float>(c);
+}
+
+// Whether kernels may read and write `p` like the fields: memory of their device.
+bool beside_fields(fish_ctx *c, const void *p)
+{
+    cudaPointerAttributes a, f;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess && cudaPointerGetAttributes(&f, field_ptr(c, 0)) == cudaSuccess)
+        return a.type == cudaMemoryTypeDevice && f.type == cudaMemoryTypeDevice && a.device == f.device;
+    (void)cudaGetLastError();
+    return false;
+}
+
+// Copy or, with `turn`, transpose (per z-plane, see transpose_state) the
+// fields to or from a device buffer of the same type, fields one after the
+// other and x fastest.
+template <class T> int copy_state(fish_ctx *c, T *buf, bool get, bool turn)
+{
+    const T *src[8];
+    T *dst[8];
+    for (int f = 0; f < 8; ++f) {
+        T *fld = (T *)field_ptr(c, f), *out = buf + (long long)f * c->N;
+        src[f] = get ? fld : out;
+        dst[f] = get ? out : fld;
+    }
+    if (turn) {
+        // source rows of nr, nc of them: y rows for the fields (layout 1), x rows for the buffer
+        const int nr = get ? c->n[1] : c->n[0], nc = get ? c->n[0] : c->n[1];
+        FISH_CK(c, Launch<T>::transpose(src, dst, 8, nr, nc, c->n[2], c->stream), "transpose launch");
+        c->launches += 1;
+    } else {
+        for (int f = 0; f < 8; ++f)
+            FISH_CK(c, cudaMemcpyAsync(dst[f], src[f], c->N * sizeof(T), cudaMemcpyDeviceToDevice, c->stream), "copy");
+        c->launches += 8;
+    }
+    return FISH_OK;
 }
 
 // layout an operator along d reads coalesced: y fastest for x sweeps
@@ -411,6 +455,15 @@ int sync_mesh(fish_ctx *c)
     return FISH_OK;
 }
 
+// a new state is about to be written to the fields, x fastest
+void state_set(fish_ctx *c)
+{
+    c->cfl_pending = false;
+    c->layout = 0;
+    c->x_fastest = false;
+    c->fresh = true;
+}
+
 int ready(fish_ctx *c)
 {
     if (!c) return FISH_ERR_ARG;
@@ -525,8 +578,7 @@ int fish_set_state(fish_ctx *c, const double *state)
     if (!c || !state) return FISH_ERR_ARG;
     int r = ensure_alloc(c);
     if (r) return r;
-    c->cfl_pending = false;
-    c->layout = 0;
+    state_set(c);
     if (c->prec == FISH_PREC_FP64) {
         for (int f = 0; f < 8; ++f)
             FISH_CK(c, cudaMemcpyAsync(field_ptr(c, f), state + (long long)f * c->N, c->N * sizeof(double),
@@ -553,23 +605,27 @@ int fish_set_state_device(fish_ctx *c, const void *state, int dtype)
     if (!c || !state || (dtype != FISH_F64 && dtype != FISH_F32)) return FISH_ERR_ARG;
     int r = ensure_alloc(c);
     if (r) return r;
-    c->cfl_pending = false;
-    c->layout = 0;
+    state_set(c);
+    if ((dtype == FISH_F64) == (c->prec == FISH_PREC_FP64)) {
+        // the upload turns the state where the layout of the x sweeps is the
+        // first one needed (every double step; one pass over the state less)
+        const bool turn = c->first_need == 1 && beside_fields(c, state);
+        r = dtype == FISH_F64 ? copy_state<double>(c, (double *)const_cast<void *>(state), false, turn)
+                              : copy_state<float>(c, (float *)const_cast<void *>(state), false, turn);
+        if (!r && turn) {
+            c->layout = 1;
+            c->x_fastest = true;
+        }
+        return r;
+    }
     for (int f = 0; f < 8; ++f) {
         void *dst = field_ptr(c, f);
-        if (dtype == FISH_F64) {
-            const double *src = (const double *)state + (long long)f * c->N;
-            if (c->prec == FISH_PREC_FP64)
-                FISH_CK(c, cudaMemcpyAsync(dst, src, c->N * 8, cudaMemcpyDeviceToDevice, c->stream), "copy");
-            else
-                FISH_CK(c, Launch<float>::from_f64(src, (float *)dst, c->N, c->stream), "convert");
-        } else {
-            const float *src = (const float *)state + (long long)f * c->N;
-            if (c->prec == FISH_PREC_FP32)
-                FISH_CK(c, cudaMemcpyAsync(dst, src, c->N * 4, cudaMemcpyDeviceToDevice, c->stream), "copy");
-            else
-                FISH_CK(c, Launch<double>::from_f32(src, (double *)dst, c->N, c->stream), "convert");
-        }
+        if (dtype == FISH_F64)
+            FISH_CK(c, Launch<float>::from_f64((const double *)state + (long long)f * c->N, (float *)dst, c->N, c->stream),
+                    "convert");
+        else
+            FISH_CK(c, Launch<double>::from_f32((const float *)state + (long long)f * c->N, (double *)dst, c->N, c->stream),
+                    "convert");
         c->launches += 1;
     }
     return FISH_OK;
@@ -581,8 +637,7 @@ int fish_set_state_host(fish_ctx *c, const void *state, int dtype)
     if (dtype == FISH_F64) return fish_set_state(c, (const double *)state);
     int r = ensure_alloc(c);
     if (r) return r;
-    c->cfl_pending = false;
-    c->layout = 0;
+    state_set(c);
     if (c->prec == FISH_PREC_FP32) {
         for (int f = 0; f < 8; ++f)
             FISH_CK(c, cudaMemcpyAsync(field_ptr(c, f), (const float *)state + (long long)f * c->N,
@@ -884,22 +939,25 @@ int fish_get_state_device(fish_ctx *c, void *state, int dtype)
     int r = ready(c);
     if (r) return r;
     if (!state || (dtype != FISH_F64 && dtype != FISH_F32)) return FISH_ERR_ARG;
+    if ((dtype == FISH_F64) == (c->prec == FISH_PREC_FP64)) {
+        // the copy turns the state where it is in the layout of the x sweeps;
+        // the fields stay as they are for the next double step
+        const bool turn = c->layout == 1 && beside_fields(c, state);
+        if (!turn && (r = set_layout(c, 0))) return r;
+        r = dtype == FISH_F64 ? copy_state<double>(c, (double *)state, true, turn)
+                              : copy_state<float>(c, (float *)state, true, turn);
+        if (!r && turn) c->x_fastest = true;
+        return r;
+    }
     if ((r = set_layout(c, 0))) return r;
     for (int f = 0; f < 8; ++f) {
         const void *src = field_ptr(c, f);
-        if (dtype == FISH_F64) {
-            double *dst = (double *)state + (long long)f * c->N;
-            if (c->prec == FISH_PREC_FP64)
-                FISH_CK(c, cudaMemcpyAsync(dst, src, c->N * 8, cudaMemcpyDeviceToDevice, c->stream), "copy");
-            else
-                FISH_CK(c, Launch<float>::to_f64((const float *)src, dst, c->N, c->stream), "convert");
-        } else {
-            float *dst = (float *)state + (long long)f * c->N;
-            if (c->prec == FISH_PREC_FP32)
-                FISH_CK(c, cudaMemcpyAsync(dst, src, c->N * 4, cudaMemcpyDeviceToDevice, c->stream), "copy");
-            else
-                FISH_CK(c, Launch<double>::to_f32((const double *)src, dst, c->N, c->stream), "convert");
-        }
+        if (dtype == FISH_F64)
+            FISH_CK(c, Launch<float>::to_f64((const float *)src, (double *)state + (long long)f * c->N, c->N, c->stream),
+                    "convert");
+        else
+            FISH_CK(c, Launch<double>::to_f32((const double *)src, (float *)state + (long long)f * c->N, c->N, c->stream),
+                    "convert");
         c->launches += 1;
     }
     return FISH_OK;
@@ -914,7 +972,7 @@ int planes_check(fish_ctx *c, int k0, int nk, const void *buf)
     int r = ready(c);
     if (r) return r;
     if (!buf || nk < 0 || k0 < 0 || k0 + nk > c->n[2]) return fail(c, FISH_ERR_ARG, "bad plane range");
-    return FISH_OK;
+    return c->x_fastest || c->fresh ? set_layout(c, 0) : FISH_OK;
 }
 
 // Copy the planes between the fields and the buffer: one kernel for a buffer
@@ -928,11 +986,7 @@ static int planes_copy(fish_ctx *c, int k0, int nk, char *buf, bool get)
         fld[f] = (char *)field_ptr(c, f) + (size_t)k0 * plane;
         out[f] = buf + (size_t)f * bytes;
     }
-    cudaPointerAttributes pb, pf;
-    const bool known = cudaPointerGetAttributes(&pb, buf) == cudaSuccess &&
-                       cudaPointerGetAttributes(&pf, fld[0]) == cudaSuccess;
-    if (!known) (void)cudaGetLastError();
-    if (known && pb.type == cudaMemoryTypeDevice && pf.type == cudaMemoryTypeDevice && pb.device == pf.device) {
+    if (beside_fields(c, buf)) {
         const void *const *src = (const void *const *)(get ? fld : out);
         void *const *dst = (void *const *)(get ? out : fld);
         FISH_CK(c, fish::launch_copy8(src, dst, bytes, c->stream), "plane copy");

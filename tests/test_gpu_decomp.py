@@ -87,3 +87,41 @@ def test_planes_to_device_host_and_unaligned_buffers(F, precision, dims):
             assert torch.equal(got[:, k0:k0 + nk], 2.0 * ref[:, k0:k0 + nk])
             box.set_state(w.state)
     box.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_planes_are_x_fastest_after_set_and_get_state(F, precision):
+    """The state is kept y fastest after fish_set_state_device and
+    fish_get_state_device where the x sweeps come first; plane copies behind
+    them still move x-fastest planes, operators and reads see the same state,
+    whatever was needed first after the last upload."""
+    import torch
+    dims = (6, 10, 5)
+    w = W.random_smooth(*dims, seed=13)
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    dev = torch.as_tensor(w.state, device="cuda").to(dt)
+    nx, ny, nz = dims
+    box = F.Box(*dims, w.gamma, bc=w.bc, precision=precision, h=w.h)
+    out, pl = torch.empty_like(dev), torch.empty(8 * 2 * nx * ny, dtype=dt, device="cuda")
+    ref = None
+    for first in ("planes", "x", "y", "planes", "get", "step", "y", "x", "planes"):
+        box.set_state(dev)
+        if first == "planes":
+            box.get_planes(1, 2, pl)
+            box.sync()
+            assert torch.equal(pl.reshape(8, 2, ny, nx), dev[:, 1:3])
+            box.set_planes(1, 2, pl)
+        elif first == "get":
+            assert torch.equal(box.get_state_device(out), dev)
+        if first in ("x", "y"):
+            box.fluid(0 if first == "x" else 1, 1e-3)
+            box.set_state(dev)
+        box.step(1e-3)
+        got = box.get_state_device(out).clone()
+        ref = got if ref is None else ref
+        assert torch.equal(got, ref), first
+        box.get_planes(1, 2, pl)
+        box.sync()
+        assert torch.equal(pl.reshape(8, 2, ny, nx), ref[:, 1:3]), first
+        assert np.array_equal(box.get_state(), ref.double().cpu().numpy())
+    box.close()
