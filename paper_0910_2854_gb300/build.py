@@ -7,6 +7,7 @@ Translation units compiled in parallel, then linked:
   fish_p2.cu   -- FP32 two-column sweep kernels (packed FP32x2), Van Leer
   fish_p2_mm.cu, fish_p2_hy.cu -- the same with the minmod / hybrid limiter
   fish_p2_hse.cu -- the same with the hydrostatic correction
+  fish_tile.cu -- FP64 thread-per-cell sweeps of small boxes, -fmad=false
   fish_capi.cu -- host-side C ABI
   fish_noalloc.cu -- the allocation-free diagnostics entry point
   fish_batch.cu -- batches of independent boxes (FP32)
@@ -34,6 +35,7 @@ UNITS = {
     "fish_p2_mm.cu": ["-prec-sqrt=false", "-ftz=true"],
     "fish_p2_hy.cu": ["-prec-sqrt=false", "-ftz=true"],
     "fish_p2_hse.cu": ["-prec-sqrt=false", "-ftz=true"],
+    "fish_tile.cu": ["-fmad=false"],
     "fish_capi.cu": [],
     "fish_noalloc.cu": [],
     "fish_batch.cu": ["-prec-sqrt=false", "-ftz=true"],

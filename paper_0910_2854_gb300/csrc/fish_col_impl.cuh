@@ -51,15 +51,6 @@ static inline int col_segments(int n, long long blocks, int slots, int lone, dou
     return len;
 }
 
-static inline int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return 152;
-    return sms;
-}
-
 // Launch fluid_col_kernel over all columns: one thread per column group, the
 // sweep in segments.
 template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF, bool NU, class IX>

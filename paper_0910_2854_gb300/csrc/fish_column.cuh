@@ -1413,6 +1413,15 @@ __global__ void __launch_bounds__(32 * ct_rows<V>(), ct_resident<V>())
 // launchers (defined in fish_col_impl.cuh, instantiated per lane-vector type
 // in their own translation units so they compile in parallel)
 // ---------------------------------------------------------------------------
+static inline int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return 152;
+    return sms;
+}
+
 // L_d with the lane-vector type V: hse selects the hydrostatic correction,
 // ft1 says whether the fast axis is t1 (FP32 callers always order the frame
 // so that it is).  Limiter from A.lim.

@@ -5,6 +5,7 @@
 #include "fish_column.cuh"
 #include "fish_kernels.cuh"
 #include "fish_launch.h"
+#include "fish_tile.cuh"
 
 namespace fish {
 
@@ -53,6 +54,20 @@ template <class T> static bool uses_pairs(const Frame &F, int lim, bool hse, boo
     if (hse && lim == LIM_HYBRID) return false;
     return sizeof(T) == 4 && F.nf % 2 == 0 && (lim == LIM_VANLEER || lim == LIM_MINMOD || lim == LIM_HYBRID);
 #endif
+}
+
+// Output cells per tile of the FP64 thread-per-cell kernels for `groups` tiles
+// side by side and n cells along the sweep, or 0 where the column marches are
+// faster: as few cells as give at most one tile per SM, else TILE_MAX cells for
+// up to `most` tiles per SM.  L_d against the march: 12^3 (30 tiles) 29 against
+// 60 us, 32^3 (128) 49 / 78, 72 x 60 x 51 (920) 295 / 277; B_d: 12^3 16 / 31,
+// 32^3 (256) 39 / 43, 72 x 60 x 51 (1080) 122 / 85.
+static inline int tile_cells(long long groups, int n, int most)
+{
+    const int sms = sm_count();
+    for (int len = 2; len <= TILE_MAX; ++len)
+        if (groups * ((n + len - 1) / len) <= sms) return len;
+    return groups * ((n + TILE_MAX - 1) / TILE_MAX) <= (long long)most * sms ? TILE_MAX : 0;
 }
 
 template <class T> bool Launch<T>::fluid_fuses_cfl(const Geom &g, int d, int lim, bool hse)
@@ -111,6 +126,8 @@ cudaError_t Launch<T>::fluid(const T *const in[8], T *const out[5], const T *phi
     A.wd = w3 ? w3[d] : nullptr;
     A.sg = split_gravity ? 1 : 0;
     if constexpr (sizeof(T) == 8) {
+        const int len = tile_cells(((long long)F.nf * F.no + 31) / 32, F.n, 4);
+        if (len) return tile_fluid(A, hse, F.ft1, len, s);
         return col_fluid<double>(A, hse, F.ft1, s);
     } else {
         // two columns per thread (packed FP32x2) when the fast extent is even;
@@ -165,6 +182,8 @@ cudaError_t Launch<T>::ct(const T *rho, const T *md, const T *const b[3], T *con
         A.wo = w3[F.other];
     }
     if constexpr (sizeof(T) == 8) {
+        const int len = tile_cells((long long)((F.nf + 30) / 31) * F.no, F.n, 2);
+        if (len) return tile_ct(A, F.ft1, len, s);
         return col_ct<double>(A, F.ft1, s);
     } else {
 #ifdef FISH_CT_PAIRS

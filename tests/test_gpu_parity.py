@@ -630,3 +630,21 @@ def test_sweep_segments(F, n, bc, precision):
             gb.ct(d, dt)
             assert rel_err(gb.get_state(), ob.state) <= (1e-12 if precision == "fp64" else 1e-5), (d, kw)
             gb.close()
+
+
+@pytest.mark.parametrize("bc", [W.BC_PERIODIC, W.BC_OUTFLOW])
+@pytest.mark.parametrize("dims", [(160, 128, 1), (160, 128, 9), (31, 40, 37), (64, 62, 40)])
+def test_fp64_marches_beside_the_small_box_kernels(F, dims, bc):
+    """FP64 boxes on both sides of the rule that takes a thread per cell for
+    few columns: many thin columns (marches, cut into segments), and boxes
+    where B_d marches while L_d does not or both sit near the limit."""
+    w = W.random_smooth(*dims, seed=95, bc=bc)
+    ob, gb = pair(F, w, "fp64")
+    dt = 0.4 * ob.cfl(1.0)
+    for d in range(3):
+        ob.fluid(d, dt)
+        gb.fluid(d, dt)
+        ob.ct(d, dt)
+        gb.ct(d, dt)
+    assert rel_err(gb.get_state(), ob.state) <= 1e-12
+    gb.close()
