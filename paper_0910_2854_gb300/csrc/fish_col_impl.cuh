@@ -126,6 +126,11 @@ static cudaError_t col_fluid_lim(const ColFluidArgs<typename VT<V>::S> &A, cudaS
         if constexpr (GRAV != 2) {
             if (A.wd) return col_fluid_launch<V, HSE, GRAV, -1, FT1, true>(A, s);
         }
+        if constexpr (std::is_same<V, float>::value && !HSE && GRAV == 0) {
+            // the plain sweeps of odd fast extents with compile-time limiters
+            if (A.lim == LIM_VANLEER) return col_fluid_launch<V, HSE, GRAV, LIM_VANLEER, FT1>(A, s);
+            if (A.lim == LIM_MINMOD) return col_fluid_launch<V, HSE, GRAV, LIM_MINMOD, FT1>(A, s);
+        }
         if constexpr (VT<V>::F64 && !HSE && GRAV == 0 && FISH_F64_VL) {
             // the plain FP64 sweeps with a compile-time Van Leer limiter
             if (A.lim == LIM_VANLEER) return col_fluid_launch<V, HSE, GRAV, LIM_VANLEER, FT1>(A, s);
@@ -193,6 +198,7 @@ template <class V> cudaError_t col_ct(const ColCTArgs<typename VT<V>::S> &A, boo
         if (A.lim == LIM_MINMOD) return col_ct_launch<V, LIM_MINMOD, true>(A, s);
         return cudaErrorInvalidValue;
     } else {
+        if (nu && A.lim == LIM_VANLEER) return col_ct_launch<V, LIM_VANLEER, true, true>(A, s);
         if (nu) return col_ct_launch<V, -1, true, true>(A, s);
         // FP32: compile-time limiters for the throughput path
         if (A.lim == LIM_VANLEER) return col_ct_launch<V, LIM_VANLEER, true>(A, s);
