@@ -964,16 +964,19 @@ template <class V> struct CWid {
     V w0, w1, w2, w3, w4, w5;
 };
 
-// Edge velocity between cells a and b of a face pencil (eq0364): the mean,
-// or with NU the linear interpolation to the interface (reading C-27).
+// Sign of the edge velocity between cells a and b of a face pencil (eq0364):
+// of the sum, or with NU of the linear interpolation to the interface (reading
+// C-27), whose positive denominator is left out.
 template <class V, bool NU> __device__ __forceinline__ V cedge(V va, V vb_, V wa, V wb)
 {
-    if constexpr (!NU) return vb<V>(0.5f) * (va + vb_);
-    else return vdiv(vfma(wb, va, wa * vb_), wa + wb);
+    if constexpr (!NU) return va + vb_;
+    else return vfma(wb, va, wa * vb_);
 }
 
-// FP64 B_d: the velocities a face pencil is advanced with are eight times the
-// smoothed ones, so the factors dt/dx of its fluxes carry an eighth.
+// B_d: the velocities a face pencil is advanced with are eight times the
+// smoothed ones (the 1/2 of the mean eq0361 and the 1/4 of the smoothing eq0362
+// are left out, exactly), and so are its products and fluxes; the factors dt/dx
+// carry an eighth.
 constexpr double CT_SCALE = 0.125;
 
 // Advance a face pencil by cell s (K = s mod 4) with face velocity vt and
@@ -987,12 +990,9 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
     constexpr int k1 = (K + 3) & 3, k2 = (K + 2) & 3, kp = (K + 1) & 3;
     constexpr int e = K & 1, o = (K + 1) & 1;
     if constexpr (VT<V>::F64) {
-        // The formulas below with vt twice the face velocity and the factor
-        // 1/4 of the smoothing left out: velocities, products and fluxes are
-        // eight times theirs, exactly, and lamh, lam an eighth (CT_SCALE).  The
-        // upwind sides are kept as bits and the differences of the predicted
-        // products in registers; the upwind operands are selected before the
-        // one limiter.
+        // The upwind sides are kept as bits and the differences of the
+        // predicted products in registers; the upwind operands are selected
+        // before the one limiter.
         const V vh = __fma_rn(2.0, P.vt[k1], vt) + P.vt[k2];
         P.vh[k1] = vh;
         P.w[o] = vh * P.bf[k1];
@@ -1029,7 +1029,7 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         return;
     }
     // smoothed face velocity at s-1 (eq0362) and the cell product w_{s-1}
-    const V vh = vb<V>(0.25f) * (vfma(vb<V>(2.0f), P.vt[k1], vt) + P.vt[k2]);
+    const V vh = vfma(vb<V>(2.0f), P.vt[k1], vt) + P.vt[k2];
     P.vh[k1] = vh;
     P.w[o] = vmul(vh, P.bf[k1]);
     {
@@ -1042,7 +1042,7 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         // predictor half step of the face field at s-2
         V bp;
         V lh = lamh;
-        if constexpr (NU) lh = vdiv(vb<V>(0.5f) * dt, cw.w2);
+        if constexpr (NU) lh = vdiv(vb<V>(float(0.5 * CT_SCALE)) * dt, cw.w2);
         bp = vfma(-lh, P.f1[e] - P.f1[o], P.bf[k2]);
         P.wp[k2] = vmul(P.vh[k2], bp);
     }
@@ -1057,25 +1057,23 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
             const V half = vb<V>(0.5f);
             const V gl = half * (cw.w5 + cw.w4), gc = half * (cw.w4 + cw.w3), gr = half * (cw.w3 + cw.w2);
             {
-                const V d0 = vdiv(w0 - wm, gl), d1 = vdiv(w1 - w0, gc), d2 = vdiv(w2 - w1, gr);
-                const V la = vsel_pos(vbar, d0, d1);
-                const V lb = vsel_pos(vbar, d1, d2);
+                const V d1 = vdiv(w1 - w0, gc);
+                const V dx = vdiv(vsel_pos(vbar, w0 - wm, w2 - w1), vsel_pos(vbar, gl, gr));
                 const V base = vsel_pos(vbar, w0, w1);
                 const V sg = vsel_pos(vbar, cw.w4, -cw.w3);
-                P.f[e] = vfma(sg, vlimit_half<LIM>(la, lb, lim), base);
+                P.f[e] = vfma(sg, vlimit_half<LIM>(d1, dx, lim), base);
             }
         } else {
-            // select the upwind operands, then limit once
-            const V d0 = w0 - wm, d1 = w1 - w0, d2 = w2 - w1;
-            const V la = vsel_pos(vbar, d0, d1);
-            const V lb = vsel_pos(vbar, d1, d2);
+            // the upwind side's operands, then one limiter: both sides limit
+            // the middle difference against their outer one
+            const V dx = vsel_pos(vbar, w0 - wm, w2 - w1);
             const V base = vsel_pos(vbar, w0, w1);
             const V sg = vsel_pos(vbar, vb<V>(1.0f), vb<V>(-1.0f));
-            P.f[e] = vfma(sg, vlimit_half<LIM>(la, lb, lim), base);
+            P.f[e] = vfma(sg, vlimit_half<LIM>(w1 - w0, dx, lim), base);
         }
         if constexpr (OUT) {
             V lo = lam;
-            if constexpr (NU) lo = vdiv(dt, cw.w4);
+            if constexpr (NU) lo = vdiv(vb<V>(float(CT_SCALE)) * dt, cw.w4);
             bnew = vfma(-lo, P.f[e] - P.f[o], P.bf[K]);
         }
     }
@@ -1099,6 +1097,7 @@ template <class S, class IX = long long> struct CTCtx {
     IX ofp;              // offset to the fast-axis column above the lane's last column
     IX oom, oop;         // offsets to the other-axis rows below / above (mapped)
     bool active;         // lane stores its columns
+    bool edge_lo, edge_hi;  // first / last row of the block
     bool fixy;           // halo lane at an outflow edge: its upper column is a copy of the lower
     S wfa, wfb;          // irregular mesh: widths of the lane's column and the one above (fast axis)
     S woa, wop, wom;     // widths of the lane's row and the rows above / below (other axis)
@@ -1150,14 +1149,10 @@ __device__ __forceinline__ void ctload(const ColCTArgs<typename VT<V>::S> &A, co
     R.bdo = vget_at<V>(A.bd, X.base + (IX)max(min(s - 4, A.n - 1), 0) * ix_sd<IX>(A));
 }
 
-// prefetch into L2 the fields of interior cell i (the neighbour rows too
-// with FISH_CT_PF_NEIGH: with the warps of a block on consecutive rows they
-// are mostly the own rows of sibling warps)
+// prefetch into L2 the fields of interior cell i; the neighbour rows by the
+// warps at the edges of a block only, the others' are their siblings' own rows
 #ifndef FISH_CT_PF_DIST
 #define FISH_CT_PF_DIST 2   // against 1: 156 -> 148 us at 256^3, 2161 -> 2035 us at 640^3
-#endif
-#ifndef FISH_CT_PF_NEIGH
-#define FISH_CT_PF_NEIGH 1
 #endif
 template <class V, class IX = long long>
 __device__ __forceinline__ void ctprefetch(const ColCTArgs<typename VT<V>::S> &A,
@@ -1165,13 +1160,15 @@ __device__ __forceinline__ void ctprefetch(const ColCTArgs<typename VT<V>::S> &A
 {
     pf_l2(ix_at(A.rho, i));
     pf_l2(ix_at(A.md, i));
-#if FISH_CT_PF_NEIGH
-    pf_l2(ix_at(A.rho, i + X.oom));
-    pf_l2(ix_at(A.md, i + X.oom));
-    pf_l2(ix_at(A.rho, i + X.oop));
-    pf_l2(ix_at(A.md, i + X.oop));
-    pf_l2(ix_at(A.bo, i + X.oom));
-#endif
+    if (X.edge_lo) {
+        pf_l2(ix_at(A.rho, i + X.oom));
+        pf_l2(ix_at(A.md, i + X.oom));
+        pf_l2(ix_at(A.bo, i + X.oom));
+    }
+    if (X.edge_hi) {
+        pf_l2(ix_at(A.rho, i + X.oop));
+        pf_l2(ix_at(A.md, i + X.oop));
+    }
     pf_l2(ix_at(A.bf, i));
     pf_l2(ix_at(A.bo, i));
     pf_l2(ix_at(A.bd, i));
@@ -1235,23 +1232,20 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
     // face velocities (eq0361): the mean of the two cells across the face,
     // or on an irregular mesh their linear interpolation to it (reading C-27)
     V vtF, vtO, vtOm;
-    if constexpr (!NU && VT<V>::F64) {
-        // (twice the mean, see cface)
+    // (twice, see CT_SCALE)
+    if constexpr (!NU) {
         vtF = vc + vfp;
         vtO = vc + vop;
         vtOm = vom + vc;
-    } else if constexpr (!NU) {
-        vtF = half * (vc + vfp);
-        vtO = half * (vc + vop);
-        vtOm = half * (vom + vc);
     } else if constexpr (VT<V>::F64) {
         vtF = 2.0 * ((X.wfb * vc + X.wfa * vfp) / (X.wfa + X.wfb));
         vtO = 2.0 * ((X.wop * vc + X.woa * vop) / (X.woa + X.wop));
         vtOm = 2.0 * ((X.woa * vom + X.wom * vc) / (X.wom + X.woa));
     } else {
-        vtF = vdiv(vfma(V(X.wfb), vc, V(X.wfa) * vfp), V(X.wfa + X.wfb));
-        vtO = vdiv(vfma(V(X.wop), vc, V(X.woa) * vop), V(X.woa + X.wop));
-        vtOm = vdiv(vfma(V(X.woa), vom, V(X.wom) * vc), V(X.wom + X.woa));
+        const V two = vb<V>(2.0f);
+        vtF = two * vdiv(vfma(V(X.wfb), vc, V(X.wfa) * vfp), V(X.wfa + X.wfb));
+        vtO = two * vdiv(vfma(V(X.wop), vc, V(X.woa) * vop), V(X.woa + X.wop));
+        vtOm = two * vdiv(vfma(V(X.woa), vom, V(X.wom) * vc), V(X.wom + X.woa));
     }
     V nF, nO, dummy;
     // (FP64, bound by its pipe, skips the corrector until its fluxes are used)
@@ -1311,7 +1305,8 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
 // The march of warp gw (31 W columns of one row) of the box described by A
 // over the output cells a .. b-1.
 template <class V, int LIM, bool FT1, bool NU = false, class IX = long long>
-__device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A, long long gw, int lane, int a, int b)
+__device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A, long long gw, int lane, int a, int b,
+                                           bool edge_lo, bool edge_hi)
 {
     using S = typename VT<V>::S;
     constexpr int W = VT<V>::W;
@@ -1321,6 +1316,8 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
     const int seg = (int)(gw % nseg), ob = (int)(gw / nseg);
     int cl = seg * SEGC + (lane - 1) * W;       // first logical column of the lane
     CTCtx<S, IX> X;
+    X.edge_lo = edge_lo;
+    X.edge_hi = edge_hi || ob + 1 == A.no;
     X.active = lane >= 1 && cl < A.nf;
     if (lane >= 1 && cl >= A.nf) cl = A.nf - W;  // idle lane: repeat a valid column
     int cb;                                      // physical first column
@@ -1341,7 +1338,7 @@ __device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A
     X.oop = (IX)(gmap(ob + 1, A.no, A.bc) - ob) * (IX)A.so * un;
     const double dtd = *A.dt;
     const V dtv = vb<V>(S(dtd));
-    constexpr double sc = VT<V>::F64 ? CT_SCALE : 1.0;
+    constexpr double sc = CT_SCALE;
     const V lamh = vb<V>(S(sc * (dtd / (2.0 * A.h))));
     const V lam = vb<V>(S(sc * (dtd / A.h)));
     V lamf = vb<V>(S(sc * (dtd / A.hf)));
@@ -1406,7 +1403,9 @@ __global__ void __launch_bounds__(32 * ct_rows<V>(), ct_resident<V>())
     const long long nseg = (A.nf + SEGC - 1) / SEGC;
     const long long seg = blockIdx.x % nseg, ob = (blockIdx.x / nseg) * ct_rows<V>() + (threadIdx.x >> 5);
     const int a = blockIdx.y * len;
-    ct_columns<V, LIM, FT1, NU, IX>(A, ob * nseg + seg, threadIdx.x & 31, a, min(A.n, a + len));
+    const int row = threadIdx.x >> 5;
+    ct_columns<V, LIM, FT1, NU, IX>(A, ob * nseg + seg, threadIdx.x & 31, a, min(A.n, a + len), row == 0,
+                                    row == ct_rows<V>() - 1);
 }
 
 // ---------------------------------------------------------------------------
