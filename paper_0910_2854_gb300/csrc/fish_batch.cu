@@ -56,17 +56,60 @@ struct BatchItem {
     int a, b;
 };
 
+// The sweep arguments of one box: the field pointers, which all boxes share,
+// from the kernel's parameters (the constant bank), the box's geometry from
+// shared memory.  With the pointers in shared memory too every access loads its
+// own first.
+struct BatchFluid {
+    using Real = float;
+    const float *const (&u)[5], *const &bd, *const &bt1, *const &bt2;
+    float *const (&uo)[5];
+    const float *const &phi, *const &wd;
+    const int &lim, &sg;
+    const float &alpha;
+    const double *const &dt;
+    const long long &off, &sd, &so;
+    const int &n, &nf, &no, &bc;
+    const float &gamma, &gm1;
+    const double &h;
+    unsigned *const &flags;
+    unsigned long long *const &cfl_min;
+    const float (&rh)[3];
+    __device__ BatchFluid(const ColFluidArgs<float> &P, const ColFluidArgs<float> &B)
+        : u(P.u), bd(P.bd), bt1(P.bt1), bt2(P.bt2), uo(P.uo), phi(P.phi), wd(P.wd), lim(P.lim), sg(P.sg),
+          alpha(P.alpha), dt(B.dt), off(B.off), sd(B.sd), so(B.so), n(B.n), nf(B.nf), no(B.no), bc(B.bc),
+          gamma(B.gamma), gm1(B.gm1), h(B.h), flags(B.flags), cfl_min(B.cfl_min), rh(B.rh)
+    {
+    }
+};
+struct BatchCT {
+    using Real = float;
+    const float *const &rho, *const &md, *const &bd, *const &bf, *const &bo;
+    float *const &bdo, *const &bfo, *const &boo;
+    const float *const &wd, *const &wf, *const &wo;
+    const int &lim;
+    const double *dt;
+    long long off, sd, so;   // (copies: this march has the registers)
+    int n, nf, no, bc;
+    double h, hf, ho;
+    __device__ BatchCT(const ColCTArgs<float> &P, const ColCTArgs<float> &B)
+        : rho(P.rho), md(P.md), bd(P.bd), bf(P.bf), bo(P.bo), bdo(P.bdo), bfo(P.bfo), boo(P.boo), wd(P.wd), wf(P.wf),
+          wo(P.wo), lim(P.lim), dt(B.dt), off(B.off), sd(B.sd), so(B.so), n(B.n), nf(B.nf), no(B.no), bc(B.bc), h(B.h),
+          hf(B.hf), ho(B.ho)
+    {
+    }
+};
+
 // (IX as in the single-box sweeps: 32-bit byte offsets, or int indices for a
 // batch of more than 2^30 cells)
 template <int LIM, bool CFLF, class IX>
 __global__ void __launch_bounds__(128, FISH_COL_MINB)
-    fluid_batch_kernel(const ColFluidArgs<float> A, const BatchBox *__restrict__ boxes,
+    fluid_batch_kernel(const __grid_constant__ ColFluidArgs<float> A, const BatchBox *__restrict__ boxes,
                        const BatchItem *__restrict__ items, int nitems, int *counter, const double *dt,
                        unsigned *flags, unsigned long long *minbits)
 {
-    // the work item's arguments, set up by thread 0, stay in shared memory:
-    // a register copy of the per-box fields spills the march, which holds
-    // about 250 registers (10.4 against 10.6 ms per batch step)
+    // the work item's geometry, set up by thread 0, stays in shared memory: a
+    // register copy spills the march, which holds about 250 registers
     __shared__ ColFluidArgs<float> Ab;
     __shared__ BatchItem I;
     for (;;) {
@@ -101,7 +144,7 @@ __global__ void __launch_bounds__(128, FISH_COL_MINB)
         if (groups == 0) return;
         const int first = I.first;
         for (int g = 0; g < groups; ++g)
-            fluid_columns<P2, false, false, LIM, true, CFLF, false, IX, false>(Ab, (long long)first + 128ll * g + threadIdx.x, I.a, I.b);
+            fluid_columns<P2, false, false, LIM, true, CFLF, false, IX, false>(BatchFluid(A, Ab), (long long)first + 128ll * g + threadIdx.x, I.a, I.b);
     }
 }
 
@@ -109,12 +152,11 @@ __global__ void __launch_bounds__(128, FISH_COL_MINB)
 // segment (the tile height; blocks of 32 * ROWS threads)
 template <int LIM, int ROWS, class IX>
 __global__ void __launch_bounds__(32 * ROWS, FISH_CT_MINB * 4 / ROWS)
-    ct_batch_kernel(const ColCTArgs<float> A, const BatchBox *__restrict__ boxes,
+    ct_batch_kernel(const __grid_constant__ ColCTArgs<float> A, const BatchBox *__restrict__ boxes,
                     const BatchItem *__restrict__ items, int nitems, int *counter, const double *dt)
 {
-    // the work item's arguments, set up by thread 0 in shared memory and
-    // copied to registers by every thread (the CT march, at 128 registers,
-    // runs faster with them in registers: 10.4 against 11.0 ms per batch step)
+    // the work item's geometry, set up by thread 0 in shared memory and
+    // copied to registers by every thread
     __shared__ ColCTArgs<float> Abs;
     __shared__ BatchItem I;
     for (;;) {
@@ -144,7 +186,7 @@ __global__ void __launch_bounds__(32 * ROWS, FISH_CT_MINB * 4 / ROWS)
         const int groups = I.groups;
         if (groups == 0) return;
         const int first = I.first;
-        const ColCTArgs<float> Ab = Abs;
+        const BatchCT Ab(A, Abs);
         // a group of ROWS warps takes one segment of ROWS consecutive rows
         // (neighbour-row loads served from L1, as in the single-box kernel)
         const long long nseg = (Ab.nf + 30) / 31;

@@ -40,6 +40,7 @@ namespace fish {
 // arguments
 // ---------------------------------------------------------------------------
 template <class S> struct ColFluidArgs {
+    using Real = S;
     const S *u[5];          // rho, m_d, m_t1, m_t2, E of the current buffer (sweep frame)
     const S *bd, *bt1, *bt2;  // face fields b_d, b_t1, b_t2 (sweep frame)
     S *uo[5];               // outputs, sweep frame
@@ -64,6 +65,7 @@ template <class S> struct ColFluidArgs {
 };
 
 template <class S> struct ColCTArgs {
+    using Real = S;
     const S *rho, *md;      // density and momentum along d (unchanged by B_d)
     const S *bd, *bf, *bo;  // b_d and the face fields of the fast and other transverse axes
     S *bdo, *bfo, *boo;     // outputs (other buffer)
@@ -430,15 +432,13 @@ template <class V> struct FMarch {
     V dprev;             // split gravity: potential (FP64) or its difference (FP32) of raw cell r-1
 };
 
-// stride along the sweep as an IX
-template <class IX, class S> __device__ __forceinline__ IX ix_sd(const ColFluidArgs<S> &A)
+// stride along the sweep as an IX (AR: the argument type, ColFluidArgs or
+// ColCTArgs or, in the batch, a view with their members)
+template <class IX, class AR> __device__ __forceinline__ IX ix_sd(const AR &A)
 {
-    return (IX)A.sd * ix_unit<S, IX>();
+    return (IX)A.sd * ix_unit<typename AR::Real, IX>();
 }
-template <class IX, class S> __device__ __forceinline__ IX ix_sd(const ColCTArgs<S> &A)
-{
-    return (IX)A.sd * ix_unit<S, IX>();
-}
+
 // IX: how elements are addressed, long long indices or (unsigned) 32-bit byte
 // offsets where all fit.
 template <class S, class IX = long long> struct FCtx {
@@ -460,8 +460,8 @@ template <class S, class IX> struct FPf {
     const S *p;   // the lane's line in cell 0 (nullptr: lane idle); cell c: p + c * sd
 };
 
-template <class S, class IX>
-__device__ __forceinline__ void fpf_setup(const ColFluidArgs<S> &A, const S *bfp, const S *bop, IX base0, IX oom0,
+template <class S, class IX, class AR>
+__device__ __forceinline__ void fpf_setup(const AR &A, const S *bfp, const S *bop, IX base0, IX oom0,
                                           int span, bool grav, int lane, FPf<S, IX> &P)
 {
     P.p = nullptr;
@@ -474,16 +474,16 @@ __device__ __forceinline__ void fpf_setup(const ColFluidArgs<S> &A, const S *bfp
     if (line <= r0 + (IX)(span - 1) * un) P.p = ix_at(f, line);
 }
 
-template <class S, class IX>
-__device__ __forceinline__ void fpf_step(const ColFluidArgs<S> &A, const FPf<S, IX> &P, int c)
+template <class S, class IX, class AR>
+__device__ __forceinline__ void fpf_step(const AR &A, const FPf<S, IX> &P, int c)
 {
     if (P.p) pf_l2(ix_at(P.p, (IX)c * ix_sd<IX>(A)));
 }
 
 // load raw cell s (any s): every index through the boundary map; a ghost
 // cell copies the mapped cell as a whole, its lower b_d face included
-template <class V, bool GRAV, bool FT1, class IX = long long>
-__device__ __forceinline__ void fload_mapped(const ColFluidArgs<typename VT<V>::S> &A,
+template <class V, bool GRAV, bool FT1, class IX = long long, class AR>
+__device__ __forceinline__ void fload_mapped(const AR &A,
                                              const FCtx<typename VT<V>::S, IX> &X, int s, FRaw<V> &R)
 {
     const int cc = gmap(s, A.n, A.bc);
@@ -526,8 +526,8 @@ __device__ __forceinline__ int wrap_cell(int c, int n, int bc)
 // Load raw cell c, the one after the cell whose raw data R holds: its lower
 // b_d face is that cell's upper one, and for the ghosts above an outflow box,
 // which copy cell n-1 as a whole, that of cell n-1.
-template <class V, bool PHI, bool FT1, bool NU, class IX = long long>
-__device__ __forceinline__ void fload_next(const ColFluidArgs<typename VT<V>::S> &A,
+template <class V, bool PHI, bool FT1, bool NU, class IX = long long, class AR>
+__device__ __forceinline__ void fload_next(const AR &A,
                                            const FCtx<typename VT<V>::S, IX> &X, int c, FRaw<V> &R)
 {
     const auto *bfp = FT1 ? A.bt1 : A.bt2;
@@ -559,8 +559,8 @@ __device__ __forceinline__ int pf_dist(int len) { return len >= 96 ? 4 : 2; }
 #define FISH_FL_PF_NEIGH 1   // also the lower other-axis face (a neighbour row)
 #endif
 // prefetch into L2 the fields the fluid march will load for interior cell i
-template <class V, bool GRAV, bool FT1, class IX = long long>
-__device__ __forceinline__ void fprefetch(const ColFluidArgs<typename VT<V>::S> &A,
+template <class V, bool GRAV, bool FT1, class IX = long long, class AR>
+__device__ __forceinline__ void fprefetch(const AR &A,
                                           const FCtx<typename VT<V>::S, IX> &X, IX i)
 {
     const auto *bfp = FT1 ? A.bt1 : A.bt2;
@@ -603,8 +603,8 @@ template <class V> __device__ __forceinline__ void sg_kick(V u[5], V dk, V tau)
 // Centred potential difference (eq02513) of the image cell of ghost r (its
 // copy along d): FP64 from the potential, FP32 from the stored differences
 // D_c = phi_{c+1} - phi_c (D_{-1} = 0 at an outflow boundary).
-template <class V, class IX = long long>
-__device__ __forceinline__ V sg_image_dk(const ColFluidArgs<typename VT<V>::S> &A,
+template <class V, class IX = long long, class AR>
+__device__ __forceinline__ V sg_image_dk(const AR &A,
                                          const FCtx<typename VT<V>::S, IX> &X, int r, V rtwoh)
 {
     const int cc = gmap(r, A.n, A.bc);
@@ -637,8 +637,8 @@ static __shared__ float2 cfl_bb_ring[4 * 3 * 128];
 // (else t2).  NU: irregular mesh along d (eq037): the cells' own widths
 // replace h (the widths of raw cells r .. r-4 ride along in M.w0 .. M.w4).
 template <class V, bool HSE, int GM, int LIM, bool FT1, bool CFLF, bool NU, int K, int ST, class IX = long long,
-          bool PFW = FISH_FL_PF_WARP != 0>
-__device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, const FCtx<typename VT<V>::S, IX> &X,
+          bool PFW = FISH_FL_PF_WARP != 0, class AR>
+__device__ __forceinline__ void fstep(const AR &A, const FCtx<typename VT<V>::S, IX> &X,
                                       FMarch<V> &M, int r, int a, int pfd, V lam, V lamh, V hdt, V dt, V rtwoh,
                                       const FPf<typename VT<V>::S, IX> &PF)
 {
@@ -827,8 +827,8 @@ __device__ __forceinline__ void fstep(const ColFluidArgs<typename VT<V>::S> &A, 
 // multiple of 32 column groups), or per lane and field (the batch, whose
 // short rows leave warps that straddle two rows)
 template <class V, bool HSE, int GRAV, int LIM, bool FT1, bool CFLF, bool NU = false, class IX = long long,
-          bool PFW = FISH_FL_PF_WARP != 0>
-__device__ __forceinline__ void fluid_columns(const ColFluidArgs<typename VT<V>::S> &A, long long cid, int a, int b)
+          bool PFW = FISH_FL_PF_WARP != 0, class AR>
+__device__ __forceinline__ void fluid_columns(const AR &A, long long cid, int a, int b)
 {
     using S = typename VT<V>::S;
     constexpr int W = VT<V>::W;
@@ -1122,8 +1122,8 @@ template <class V> __device__ __forceinline__ void fixy_(V &a, bool f)
 // b_d of the cell s-4 that leaves when s enters (clamped to the box: before
 // the segment's first output cell, and in the load behind its last step, it is
 // not used).
-template <class V, bool NU, class IX = long long>
-__device__ __forceinline__ void ctload(const ColCTArgs<typename VT<V>::S> &A, const CTCtx<typename VT<V>::S, IX> &X,
+template <class V, bool NU, class IX = long long, class AR>
+__device__ __forceinline__ void ctload(const AR &A, const CTCtx<typename VT<V>::S, IX> &X,
                                        int s, CTRaw<V> &R)
 {
     const int sm = wrap_cell(s, A.n, A.bc);
@@ -1154,8 +1154,8 @@ __device__ __forceinline__ void ctload(const ColCTArgs<typename VT<V>::S> &A, co
 #ifndef FISH_CT_PF_DIST
 #define FISH_CT_PF_DIST 2   // against 1: 156 -> 148 us at 256^3, 2161 -> 2035 us at 640^3
 #endif
-template <class V, class IX = long long>
-__device__ __forceinline__ void ctprefetch(const ColCTArgs<typename VT<V>::S> &A,
+template <class V, class IX = long long, class AR>
+__device__ __forceinline__ void ctprefetch(const AR &A,
                                            const CTCtx<typename VT<V>::S, IX> &X, IX i)
 {
     pf_l2(ix_at(A.rho, i));
@@ -1201,8 +1201,8 @@ template <class V> __device__ __forceinline__ V shfl_up1(V a)
 // inputs of s are in M.R, the step loads those of s+1.  a: first output cell of
 // the segment, so that cell s-4 is an output cell from s = a+4 on (the stages
 // before work on windows that are still zero and their results are not used).
-template <class V, int LIM, bool FT1, bool NU, int K, class IX = long long>
-__device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, const CTCtx<typename VT<V>::S, IX> &X,
+template <class V, int LIM, bool FT1, bool NU, int K, class IX = long long, class AR>
+__device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::S, IX> &X,
                                        CTMarch<V> &M, int s, int a, V lamh, V lam, V lamf, V lamo, V dt)
 {
     // widths of cells s .. s-5 for this step (the width of cell s arrived
@@ -1304,8 +1304,8 @@ __device__ __forceinline__ void ctstep(const ColCTArgs<typename VT<V>::S> &A, co
 // own repeat a valid column and store nothing.
 // The march of warp gw (31 W columns of one row) of the box described by A
 // over the output cells a .. b-1.
-template <class V, int LIM, bool FT1, bool NU = false, class IX = long long>
-__device__ __forceinline__ void ct_columns(const ColCTArgs<typename VT<V>::S> &A, long long gw, int lane, int a, int b,
+template <class V, int LIM, bool FT1, bool NU = false, class IX = long long, class AR>
+__device__ __forceinline__ void ct_columns(const AR &A, long long gw, int lane, int a, int b,
                                            bool edge_lo, bool edge_hi)
 {
     using S = typename VT<V>::S;
