@@ -271,8 +271,9 @@ template <class T> struct DiagArgs {
 };
 
 // A warp takes rows of the fastest memory axis (fixed by the grid, so the
-// order of the sums is fixed).  Bound by the FP64 pipe: eight sums per cell and
-// the divergence with quotients behind shared reciprocals of the widths.
+// order of the sums is fixed).  Bound by the FP64 pipe: eight sums per cell and,
+// for cells that may hold the maximum, the divergence with quotients behind
+// shared reciprocals of the widths.
 template <class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) diag_kernel(DiagArgs<T> A)
 {
@@ -284,6 +285,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) diag_kernel(DiagA
     const long long of0 = gmap(-1, nf, g.bc);  // to the lower neighbour of a row's first cell
     double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     long long dmax = 0;  // bits of the largest |div b|
+    float dlow = 0.0f;   // FP32 states: a lower bound of the warp's largest
     double hx[3], ri[3];
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
@@ -327,13 +329,24 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) diag_kernel(DiagA
                 for (int i = 0; i < 8; ++i) s[i] += q[i];
             }
             if (!skip_row && !(open && nf > 1 && f == 0)) {
+                if constexpr (sizeof(T) == 4) {
+                    // in FP32 first, with a bound of its rounding: only a
+                    // cell that may exceed the maximum is evaluated in FP64
+                    const float e0 = (float)(v[5] - v[8]) * (float)ri[0], e1 = (float)(v[6] - v[9]) * (float)ri[1],
+                                e2 = (float)(v[7] - v[10]) * (float)ri[2];
+                    const float top = fabsf(e0 + e1 + e2) + 1e-6f * (fabsf(e0) + fabsf(e1) + fabsf(e2));
+                    if (dlow > 1e-30f && top < dlow) continue;
+                }
                 const double dv = quot64(q[5] - q[8], hx[0], ri[0]) + quot64(q[6] - q[9], hx[1], ri[1]) +
                                   quot64(q[7] - q[10], hx[2], ri[2]);
                 // (a NaN counts as none, as in fmax)
                 const long long d = __double_as_longlong(fabs(dv));
                 if (d <= 0x7ff0000000000000ll) dmax = max(dmax, d);
+                if constexpr (sizeof(T) == 4) dlow = fmaxf(dlow, 0.999999f * (float)__longlong_as_double(dmax));
             }
         }
+        if constexpr (sizeof(T) == 4)
+            dlow = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dlow)));
     }
     __shared__ double red[256][9];
     for (int f = 0; f < 8; ++f) red[threadIdx.x][f] = s[f];
