@@ -310,15 +310,15 @@ def time_operators(F, box, torch, reps=3):
 # capture of the 384^3 turbulence box (dram__bytes_read.sum +
 # dram__bytes_write.sum over its cells).  Set an entry to None when that
 # kernel changes until it is captured again.
-TRAFFIC_B_PER_CELL = {"fluid": 52.1, "ct": 32.1}
+TRAFFIC_B_PER_CELL = {"fluid": 52.2, "ct": 34.1}
 
 
 # FP64 pipe instructions (DADD + DMUL + DFMA, thread level) per cell of one
 # launch of each FP64 kernel kind, from the ncu capture of the Orszag-Tang
-# 128^3 box.  The FP64 path
+# 256^3 box.  The FP64 path
 # is bound by GB300's FP64 pipe, so its roofline is this rate against the
 # probed FMA rate of the device (fish_probe_fp64_fma).
-FP64_OPS_PER_CELL = {"fluid": 537, "ct": 170}
+FP64_OPS_PER_CELL = {"fluid": 383, "ct": 110}
 
 
 def traffic_per_cell(kernel_key):
