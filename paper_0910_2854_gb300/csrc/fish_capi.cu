@@ -241,6 +241,10 @@ bool beside_fields(fish_ctx *c, const void *p)
     return false;
 }
 
+// Whether a copy of the state to or from `p` can turn its layout (the
+// transposes have a grid layer per z-plane; a longer box is copied as it is).
+bool can_turn(fish_ctx *c, const void *p) { return c->n[2] <= 65535 && beside_fields(c, p); }
+
 // Copy or, with `turn`, transpose (per z-plane, see transpose_state) the
 // fields to or from a device buffer of the same type, fields one after the
 // other and x fastest.
@@ -609,7 +613,7 @@ int fish_set_state_device(fish_ctx *c, const void *state, int dtype)
     if ((dtype == FISH_F64) == (c->prec == FISH_PREC_FP64)) {
         // the upload turns the state where the layout of the x sweeps is the
         // first one needed (every double step; one pass over the state less)
-        const bool turn = c->first_need == 1 && beside_fields(c, state);
+        const bool turn = c->first_need == 1 && can_turn(c, state);
         r = dtype == FISH_F64 ? copy_state<double>(c, (double *)const_cast<void *>(state), false, turn)
                               : copy_state<float>(c, (float *)const_cast<void *>(state), false, turn);
         if (!r && turn) {
@@ -942,7 +946,7 @@ int fish_get_state_device(fish_ctx *c, void *state, int dtype)
     if ((dtype == FISH_F64) == (c->prec == FISH_PREC_FP64)) {
         // the copy turns the state where it is in the layout of the x sweeps;
         // the fields stay as they are for the next double step
-        const bool turn = c->layout == 1 && beside_fields(c, state);
+        const bool turn = c->layout == 1 && can_turn(c, state);
         if (!turn && (r = set_layout(c, 0))) return r;
         r = dtype == FISH_F64 ? copy_state<double>(c, (double *)state, true, turn)
                               : copy_state<float>(c, (float *)state, true, turn);

@@ -125,3 +125,18 @@ def test_planes_are_x_fastest_after_set_and_get_state(F, precision):
         assert torch.equal(pl.reshape(8, 2, ny, nx), ref[:, 1:3]), first
         assert np.array_equal(box.get_state(), ref.double().cpu().numpy())
     box.close()
+
+
+@pytest.mark.parametrize("nz", [65535, 65536])
+def test_state_of_a_box_longer_than_a_launch_grid(F, nz):
+    """A layout change takes a grid layer per z-plane (at most 65535); state
+    uploads and downloads of longer boxes do without one."""
+    import torch
+    w = W.random_smooth(2, 4, nz, seed=3)
+    dev = torch.as_tensor(w.state, device="cuda").float()
+    box = F.Box(2, 4, nz, w.gamma, bc=w.bc, precision="fp32", h=w.h)
+    box.set_state(dev)
+    assert torch.equal(box.get_state_device(torch.empty_like(dev)), dev)
+    box.fluid(2, 1e-3)
+    assert torch.isfinite(box.get_state_device(torch.empty_like(dev))).all()
+    box.close()
