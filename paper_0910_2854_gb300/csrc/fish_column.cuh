@@ -1228,11 +1228,10 @@ __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::
     // load cell s+1
     ctload<V, NU, IX>(A, X, s + 1, M.R);
     ctprefetch<V, IX>(A, X, X.base + (IX)max(min(s + 1 + FISH_CT_PF_DIST, A.n - 1), 0) * ix_sd<IX>(A));
-    const V half = vb<V>(0.5f);
-    // face velocities (eq0361): the mean of the two cells across the face,
-    // or on an irregular mesh their linear interpolation to it (reading C-27)
+    // twice the face velocities (see CT_SCALE; eq0361): the mean of the two
+    // cells across the face, or on an irregular mesh their linear
+    // interpolation to it (reading C-27)
     V vtF, vtO, vtOm;
-    // (twice, see CT_SCALE)
     if constexpr (!NU) {
         vtF = vc + vfp;
         vtO = vc + vop;

@@ -83,8 +83,6 @@ __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); 
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ P2 vmax(P2 a, P2 b) { return {make_float2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y))}; }
 
-__device__ __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
-__device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
 // minimum that keeps a NaN of either operand
 __device__ __forceinline__ float sminnan(float a, float b)
 {
@@ -97,7 +95,6 @@ __device__ __forceinline__ P2 vminnan(P2 a, P2 b)
 {
     return {make_float2(sminnan(a.v.x, b.v.x), sminnan(a.v.y, b.v.y))};
 }
-__device__ __forceinline__ P2 vmin(P2 a, P2 b) { return {make_float2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y))}; }
 
 // reciprocal: IEEE in FP64, the hardware's (1 ulp) in FP32
 __device__ __forceinline__ float srcp(float a)
@@ -156,7 +153,6 @@ __device__ __forceinline__ P2 vquot(P2 a, P2 b) { return vdiv(a, b); }
 __device__ __forceinline__ bool pos64(double a) { return __double_as_longlong(a) > 0; }
 
 // ---- limiters (eq0190 minmod, eq0200 Van Leer; sign(0) = 0, reading C-8) --
-template <class S> __device__ __forceinline__ S ssgn(S a) { return a > S(0) ? S(1) : (a < S(0) ? S(-1) : S(0)); }
 
 __device__ __forceinline__ double vminmod(double a, double b)
 {
