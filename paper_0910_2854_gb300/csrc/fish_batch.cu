@@ -458,8 +458,9 @@ struct fish_batch {
     bool t4 = false;              // every box allows the 16-byte transpose
     const float **tsrc = nullptr;  // device tables: per buffer parity, 8 source then 8 destination field pointers
     std::vector<void *> owned;
-    // transfers: two pinned halves of kStage floats, each with the event of its last copy
+    // transfers: two halves of kStage floats, pinned (or pageable: `paged`), each with the event of its last copy
     float *stage[2] = {};
+    std::unique_ptr<float[]> paged[2];
     cudaEvent_t staged[2] = {};
     HostThreads host;
     bool tables = false;
@@ -854,11 +855,17 @@ int batch_ready(fish_batch *b)
     return FISH_OK;
 }
 
-// The pinned staging halves (with the first transfer).
+// The staging halves (with the first transfer): pinned, or pageable where the
+// system grants no pinned memory.
 int batch_stage(fish_batch *b)
 {
     for (int h = 0; h < 2; ++h) {
-        if (!b->stage[h]) FISH_BCK(b, cudaMallocHost(&b->stage[h], sizeof(float) * kStage), "staging");
+        if (!b->stage[h] && cudaMallocHost(&b->stage[h], sizeof(float) * kStage) != cudaSuccess) {
+            (void)cudaGetLastError();
+            b->paged[h].reset(new (std::nothrow) float[kStage]);
+            b->stage[h] = b->paged[h].get();
+            if (!b->stage[h]) return bfail(b, FISH_ERR_CUDA, "staging: out of host memory");
+        }
         if (!b->staged[h]) FISH_BCK(b, cudaEventCreateWithFlags(&b->staged[h], cudaEventDisableTiming), "staging");
     }
     return FISH_OK;
@@ -1137,7 +1144,7 @@ void fish_batch_destroy(fish_batch *b)
     for (void *p : b->owned) cudaFree(p);
     for (int h = 0; h < 2; ++h) {
         if (b->staged[h]) cudaEventDestroy(b->staged[h]);
-        if (b->stage[h]) cudaFreeHost(b->stage[h]);
+        if (b->stage[h] && !b->paged[h]) cudaFreeHost(b->stage[h]);
     }
     if (b->own) cudaStreamDestroy(b->own);
     delete b;
