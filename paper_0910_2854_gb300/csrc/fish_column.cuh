@@ -596,7 +596,10 @@ template <class V> __device__ __forceinline__ void sg_kick(V u[5], V dk, V tau)
         const V mo = u[1];
         const V dm = -(tau * u[0]) * dk;
         u[1] = mo + dm;
-        u[4] = u[4] + vdiv(dm * vfma(vb<V>(0.5f), dm, mo), u[0]);
+        const V dE = dm * vfma(vb<V>(0.5f), dm, mo);
+        // (one column: the quotient unrounded in the sum, as earlier versions had it)
+        if constexpr (VT<V>::W == 1) u[4] = vfma(dE, vrcp(u[0]), u[4]);
+        else u[4] = u[4] + vdiv(dE, u[0]);
     }
 }
 
@@ -983,9 +986,11 @@ constexpr double CT_SCALE = 0.125;
 // field bf.  With OUT, bnew receives the updated face field of cell s-4 and
 // f[K & 1] holds the corrector flux at (s-4)'.  NU: irregular mesh along d
 // (widths in cw, eq037 and reading C-25/C-27; dt for the per-cell factors).
+// fin: the newest product difference of a float pencil takes its product
+// unrounded (see ct_rounding).
 template <class V, int LIM, int K, bool OUT, bool NU = false>
 __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V &bnew, int lim, bool live,
-                                      const CWid<V> &cw = CWid<V>(), V dt = V())
+                                      const CWid<V> &cw = CWid<V>(), V dt = V(), bool fin = false)
 {
     constexpr int k1 = (K + 3) & 3, k2 = (K + 2) & 3, kp = (K + 1) & 3;
     constexpr int e = K & 1, o = (K + 1) & 1;
@@ -1038,9 +1043,9 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         const V vbar = cedge<V, NU>(P.vh[k2], vh, cw.w2, cw.w1);
         P.f1[e] = vsel_pos(vbar, P.w[e], P.w[o]);
     }
+    V bp;
     {
         // predictor half step of the face field at s-2
-        V bp;
         V lh = lamh;
         if constexpr (NU) lh = vdiv(vb<V>(float(0.5 * CT_SCALE)) * dt, cw.w2);
         bp = vfma(-lh, P.f1[e] - P.f1[o], P.bf[k2]);
@@ -1066,7 +1071,9 @@ __device__ __forceinline__ void cface(CFace<V> &P, V vt, V bf, V lamh, V lam, V 
         } else {
             // the upwind side's operands, then one limiter: both sides limit
             // the middle difference against their outer one
-            const V dx = vsel_pos(vbar, w0 - wm, w2 - w1);
+            V d2 = w2 - w1;
+            if constexpr (std::is_same<V, float>::value) d2 = fin ? fmaf(P.vh[k2], bp, -w1) : d2;
+            const V dx = vsel_pos(vbar, w0 - wm, d2);
             const V base = vsel_pos(vbar, w0, w1);
             const V sg = vsel_pos(vbar, vb<V>(1.0f), vb<V>(-1.0f));
             P.f[e] = vfma(sg, vlimit_half<LIM>(w1 - w0, dx, lim), base);
@@ -1099,6 +1106,7 @@ template <class S, class IX = long long> struct CTCtx {
     bool active;         // lane stores its columns
     bool edge_lo, edge_hi;  // first / last row of the block
     bool fixy;           // halo lane at an outflow edge: its upper column is a copy of the lower
+    int fused, fin;      // see ct_rounding
     S wfa, wfb;          // irregular mesh: widths of the lane's column and the one above (fast axis)
     S woa, wop, wom;     // widths of the lane's row and the rows above / below (other axis)
 };
@@ -1197,11 +1205,32 @@ template <class V> __device__ __forceinline__ V shfl_up1(V a)
     else return __shfl_up_sync(0xffffffffu, a, 1);
 }
 
+// Where the one-column FP32 march rounds.  At a change of sign of an edge
+// velocity one rounding picks another upwind cell, so the results stay those
+// of earlier versions (of a run that is continued, of a study compared with
+// one) only if every rounding does; these are where earlier kernels had them:
+// - the sum of two velocities takes the neighbour's quotient m / rho as the
+//   unrounded product of one multiply-add in the cells -1 .. fused - 1 and
+//   `fin`, and rounded in the others (of a sweep of fewer than eight cells: in
+//   all but cell -1), but in cell -4 the sum across the other-axis face takes
+//   the cell's own quotient so;
+// - the lower other-axis pencil takes its newest product unrounded in the
+//   difference formed at cell `fin` (a cell no march reaches if there is none).
+// The loop has a copy of its steps for the cells in the middle, where only the
+// first holds: 139.1 -> 139.6 us at 256^3 and 1964 -> 1978 us at 640^3 against
+// one form for all cells, 142.2 and 2008 us with the choice made in each step.
+__device__ __forceinline__ void ct_rounding(int n, int &fused, int &fin)
+{
+    fused = n >= 8 ? (n - 1) / 4 * 4 : 0;
+    fin = n >= 8 && n % 4 == 0 ? n + 3 : n + 4;
+}
+
 // One cell s of the CT march (K = slot of cell s in the windows); the raw
 // inputs of s are in M.R, the step loads those of s+1.  a: first output cell of
 // the segment, so that cell s-4 is an output cell from s = a+4 on (the stages
 // before work on windows that are still zero and their results are not used).
-template <class V, int LIM, bool FT1, bool NU, int K, class IX = long long, class AR>
+// MID: s is one of the cells 0 .. fused - 1 of ct_rounding.
+template <class V, int LIM, bool FT1, bool NU, int K, bool MID, class IX = long long, class AR>
 __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::S, IX> &X,
                                        CTMarch<V> &M, int s, int a, V lamh, V lam, V lamf, V lamo, V dt)
 {
@@ -1216,11 +1245,28 @@ __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::
         M.cw.w0 = M.R.w;
     }
     // consume the raw inputs of cell s
+    constexpr bool PK = ct_packs<V, NU>();
     const V vc = vquot(M.R.mc, M.R.rc);
-    const V vop = vquot(M.R.mo, M.R.ro);
-    const V vom = vquot(M.R.mm, M.R.rm);
-    V vfp;
-    if constexpr (VT<V>::F64) vfp = vquot(M.R.mf, M.R.rf);
+    V vop, vom, vfp, vtF, vtO, vtOm;
+    if constexpr (PK) {
+        // the sums of the velocities across the three faces (see ct_rounding)
+        const float rf = srcp(M.R.rf), ro = srcp(M.R.ro), rm = srcp(M.R.rm);
+        if (MID || (s >= -1 && s < X.fused) || s == X.fin) {
+            vtF = fmaf(M.R.mf, rf, vc);
+            vtO = fmaf(M.R.mo, ro, vc);
+            vtOm = fmaf(M.R.mm, rm, vc);
+        } else {
+            vtF = vc + __fmul_rn(M.R.mf, rf);
+            vtO = vc + __fmul_rn(M.R.mo, ro);
+            vtOm = vc + __fmul_rn(M.R.mm, rm);
+            if (s == -4) vtO = fmaf(M.R.mc, srcp(M.R.rc), __fmul_rn(M.R.mo, ro));
+        }
+    } else {
+        vop = vquot(M.R.mo, M.R.ro);
+        vom = vquot(M.R.mm, M.R.rm);
+    }
+    if constexpr (PK) {
+    } else if constexpr (VT<V>::F64) vfp = vquot(M.R.mf, M.R.rf);
     else if constexpr (VT<V>::W == 2) vfp = vshift_hi(vc, __fdividef(M.R.mf, M.R.rf));
     else vfp = vdiv(V(M.R.mf), V(M.R.rf));
     const V bF = M.R.bF, bO = M.R.bO, bOm = M.R.bOm;
@@ -1231,8 +1277,8 @@ __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::
     // twice the face velocities (see CT_SCALE; eq0361): the mean of the two
     // cells across the face, or on an irregular mesh their linear
     // interpolation to it (reading C-27)
-    V vtF, vtO, vtOm;
-    if constexpr (!NU) {
+    if constexpr (PK) {
+    } else if constexpr (!NU) {
         vtF = vc + vfp;
         vtO = vc + vop;
         vtOm = vom + vc;
@@ -1249,7 +1295,6 @@ __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::
     V nF, nO, dummy;
     // (FP64, bound by its pipe, skips the corrector until its fluxes are used)
     const bool live = s >= a + 3;
-    constexpr bool PK = ct_packs<V, NU>();
     if constexpr (PK) {
         P2 n2;
         cface<P2, LIM, K, true, false>(M.PFO, P2{make_float2(vtF, vtO)}, P2{make_float2(bF, bO)}, vb<P2>(lamh),
@@ -1260,7 +1305,7 @@ __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::
         cface<V, LIM, K, true, NU>(M.PF, vtF, bF, lamh, lam, nF, A.lim, live, M.cw, dt);
         cface<V, LIM, K, true, NU>(M.PO, vtO, bO, lamh, lam, nO, A.lim, live, M.cw, dt);
     }
-    cface<V, LIM, K, false, NU>(M.POm, vtOm, bOm, lamh, lam, dummy, A.lim, live, M.cw, dt);
+    cface<V, LIM, K, false, NU>(M.POm, vtOm, bOm, lamh, lam, dummy, A.lim, live, M.cw, dt, PK && !MID && s == X.fin);
     {
         constexpr int e = K & 1;
         // edge flux of the fast-axis face below: the upper pencil of the lane beneath
@@ -1329,6 +1374,7 @@ __device__ __forceinline__ void ct_columns(const AR &A, long long gw, int lane, 
         cb = 0;
         X.fixy = W == 2;
     }
+    ct_rounding(A.n, X.fused, X.fin);
     const int cfp = gmap(cl + W, A.nf, A.bc);
     constexpr IX un = ix_unit<S, IX>();
     X.base = ((IX)A.off + (IX)cb + (IX)ob * (IX)A.so) * un;
@@ -1371,16 +1417,25 @@ __device__ __forceinline__ void ct_columns(const AR &A, long long gw, int lane, 
     M.cw.w0 = M.cw.w1 = M.cw.w2 = M.cw.w3 = M.cw.w4 = M.cw.w5 = vb<V>(1.0f);
     ctload<V, NU, IX>(A, X, a - 4, M.R);
     const int last = b + 3;
+    // four steps; whether the last one was among them
+    const auto four = [&](auto mid, int s) {
+        constexpr bool MID = decltype(mid)::value;
+        ctstep<V, LIM, FT1, NU, 0, MID, IX>(A, X, M, s, a, lamh, lam, lamf, lamo, dtv);
+        if (s >= last) return true;
+        ctstep<V, LIM, FT1, NU, 1, MID, IX>(A, X, M, s + 1, a, lamh, lam, lamf, lamo, dtv);
+        if (s + 1 >= last) return true;
+        ctstep<V, LIM, FT1, NU, 2, MID, IX>(A, X, M, s + 2, a, lamh, lam, lamf, lamo, dtv);
+        if (s + 2 >= last) return true;
+        ctstep<V, LIM, FT1, NU, 3, MID, IX>(A, X, M, s + 3, a, lamh, lam, lamf, lamo, dtv);
+        return s + 3 >= last;
+    };
 #pragma unroll 1
     for (int s = a - 4;; s += 4) {
-        ctstep<V, LIM, FT1, NU, 0, IX>(A, X, M, s, a, lamh, lam, lamf, lamo, dtv);
-        if (s >= last) break;
-        ctstep<V, LIM, FT1, NU, 1, IX>(A, X, M, s + 1, a, lamh, lam, lamf, lamo, dtv);
-        if (s + 1 >= last) break;
-        ctstep<V, LIM, FT1, NU, 2, IX>(A, X, M, s + 2, a, lamh, lam, lamf, lamo, dtv);
-        if (s + 2 >= last) break;
-        ctstep<V, LIM, FT1, NU, 3, IX>(A, X, M, s + 3, a, lamh, lam, lamf, lamo, dtv);
-        if (s + 3 >= last) break;
+        if (!ct_packs<V, NU>() || (s >= 0 && s + 3 < X.fused)) {
+            if (four(std::true_type{}, s)) break;
+        } else {
+            if (four(std::false_type{}, s)) break;
+        }
     }
 }
 

@@ -64,8 +64,7 @@ __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a
 __device__ __forceinline__ P2 vfma(P2 a, P2 b, P2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
 
 // a*b, rounded: never contracted into a following addition in FP32, so that
-// one pencil advanced as float (the lower face of a row, the batch, the single
-// box) and as a component of a P2 gets the same bits
+// the compiler's choice does not show in the bits of a pencil advanced as float
 __device__ __forceinline__ double vmul(double a, double b) { return a * b; }
 __device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ P2 vmul(P2 a, P2 b) { return a * b; }
