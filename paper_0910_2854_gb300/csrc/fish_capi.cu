@@ -241,9 +241,14 @@ bool beside_fields(fish_ctx *c, const void *p)
     return false;
 }
 
-// Whether a copy of the state to or from `p` can turn its layout (the
-// transposes have a grid layer per z-plane; a longer box is copied as it is).
-bool can_turn(fish_ctx *c, const void *p) { return c->n[2] <= 65535 && beside_fields(c, p); }
+// Whether a copy of the state to or from `p` can turn its layout: a transpose
+// reads and writes whole elements, and its grid has a layer per z-plane.  A
+// longer box and a buffer that is not aligned to its elements are copied as
+// they are.
+bool can_turn(fish_ctx *c, const void *p)
+{
+    return c->n[2] <= 65535 && (size_t)p % esize(c) == 0 && beside_fields(c, p);
+}
 
 // Copy or, with `turn`, transpose (per z-plane, see transpose_state) the
 // fields to or from a device buffer of the same type, fields one after the

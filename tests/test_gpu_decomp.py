@@ -140,3 +140,33 @@ def test_state_of_a_box_longer_than_a_launch_grid(F, nz):
     box.fluid(2, 1e-3)
     assert torch.isfinite(box.get_state_device(torch.empty_like(dev))).all()
     box.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_state_in_a_buffer_not_aligned_to_its_elements(F, precision):
+    """Such a device buffer (a C caller's) is copied; only an aligned one is
+    turned by a kernel."""
+    import ctypes
+    import torch
+    dims = (6, 10, 5)
+    w = W.random_smooth(*dims, seed=14)
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    dev = torch.as_tensor(w.state, device="cuda").to(dt)
+    raw = dev.reshape(-1).view(torch.uint8)
+    code = F.FISH_F32 if precision == "fp32" else F.FISH_F64
+    box, ref = (F.Box(*dims, w.gamma, bc=w.bc, precision=precision, h=w.h) for _ in range(2))
+    ref.set_state(dev)
+    ref.step(1e-3)
+    want = ref.get_state_device(torch.empty_like(dev))
+    for shift in (1, 2, dev.element_size() // 2 + 1):
+        buf = torch.zeros(raw.numel() + 16, dtype=torch.uint8, device="cuda")
+        buf[shift:shift + raw.numel()] = raw
+        torch.cuda.synchronize()
+        p = ctypes.c_void_p(buf.data_ptr() + shift)
+        box._check(box._lib.fish_set_state_device(box.ctx, p, code), "set")
+        box.step(1e-3)
+        box._check(box._lib.fish_get_state_device(box.ctx, p, code), "get")
+        box.sync()
+        assert torch.equal(buf[shift:shift + raw.numel()].clone().view(dt).reshape(dev.shape), want)
+    box.close()
+    ref.close()
