@@ -242,12 +242,15 @@ bool beside_fields(fish_ctx *c, const void *p)
 }
 
 // Whether a copy of the state to or from `p` can turn its layout: a transpose
-// reads and writes whole elements, and its grid has a layer per z-plane.  A
-// longer box and a buffer that is not aligned to its elements are copied as
-// they are.
+// reads and writes whole elements, and its grid has a layer per z-plane and,
+// one way or the other, a row of blocks per 32 x or y cells at the most.  A
+// longer box, which may never run an x sweep, and a buffer that is not aligned
+// to its elements are copied as they are.
 bool can_turn(fish_ctx *c, const void *p)
 {
-    return c->n[2] <= 65535 && (size_t)p % esize(c) == 0 && beside_fields(c, p);
+    constexpr int most = 65535;
+    return c->n[0] <= 32 * most && c->n[1] <= 32 * most && c->n[2] <= most && (size_t)p % esize(c) == 0 &&
+           beside_fields(c, p);
 }
 
 // Copy or, with `turn`, transpose (per z-plane, see transpose_state) the

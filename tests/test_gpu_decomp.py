@@ -127,17 +127,22 @@ def test_planes_are_x_fastest_after_set_and_get_state(F, precision):
     box.close()
 
 
-@pytest.mark.parametrize("nz", [65535, 65536])
-def test_state_of_a_box_longer_than_a_launch_grid(F, nz):
-    """A layout change takes a grid layer per z-plane (at most 65535); state
-    uploads and downloads of longer boxes do without one."""
+@pytest.mark.parametrize("dims,sweep", [((2, 4, 65535), 2), ((2, 4, 65536), 2), ((4200001, 2, 1), 1),
+                                        ((2, 4200001, 1), 1), ((1, 4200001, 1), 1)])
+def test_state_of_a_box_longer_than_a_launch_grid(F, dims, sweep):
+    """A layout change takes a grid layer per z-plane (at most 65535) and a row
+    of blocks per tile along x or y (as many); state uploads and downloads of
+    longer boxes, and the sweeps along y and z, do without one."""
     import torch
-    w = W.random_smooth(2, 4, nz, seed=3)
-    dev = torch.as_tensor(w.state, device="cuda").float()
-    box = F.Box(2, 4, nz, w.gamma, bc=w.bc, precision="fp32", h=w.h)
+    u = np.random.RandomState(3).random_sample((8, dims[2], dims[1], dims[0]))
+    dev = torch.as_tensor(u, device="cuda").float().mul_(0.1)
+    dev[0] += 1.0
+    dev[4] += 1.0
+    box = F.Box(*dims, 1.4, bc=W.BC_PERIODIC, precision="fp32", h=(0.1, 0.1, 0.1))
     box.set_state(dev)
     assert torch.equal(box.get_state_device(torch.empty_like(dev)), dev)
-    box.fluid(2, 1e-3)
+    box.fluid(sweep, 1e-3)
+    box.ct(sweep, 1e-3)
     assert torch.isfinite(box.get_state_device(torch.empty_like(dev))).all()
     box.close()
 
