@@ -90,17 +90,19 @@ template <class V> struct CCell {
     V p, cs, cf, vn;     // used by the hydrostatic correction only
 };
 
-// running checks for reading C-16: min rho and min p, both keeping a NaN (a
-// NaN of any input makes p one, and p > 0 and rho > 0 leave c_F real)
+// running checks for reading C-16.  FP32: min rho, min p, and a sum of c_F
+// that turns NaN if any evaluated cell has none (a maximum of speeds drops a
+// NaN, so this is the only trace of one); FP64: FLAG_* by the bits
 template <class V> struct Checks {
-    V mn_rho, mn_p;
-    int hi;   // FP64: FLAG_* seen, by the bits of rho, p and c_F
+    V mn_rho, mn_p, nsum;
+    int hi;
 };
 
 template <class V> __device__ __forceinline__ void checks_init(Checks<V> &k)
 {
     k.mn_rho = vb<V>(3.0e38f);
     k.mn_p = vb<V>(3.0e38f);
+    k.nsum = vb<V>(0.0f);
     k.hi = 0;
 }
 
@@ -110,10 +112,10 @@ template <class V> __device__ __forceinline__ unsigned checks_flags(const Checks
     unsigned f = 0;
 #pragma unroll
     for (int i = 0; i < VT<V>::W; ++i) {
-        const auto r = vget(k.mn_rho, i), p = vget(k.mn_p, i);
-        if (r <= 0) f |= FLAG_RHO;
-        if (p <= 0) f |= FLAG_P;
-        if (r != r || p != p) f |= FLAG_NAN;
+        const auto r = vget(k.mn_rho, i), p = vget(k.mn_p, i), s = vget(k.nsum, i);
+        if (!(r > 0)) f |= FLAG_RHO;
+        if (!(p > 0)) f |= FLAG_P;
+        if (s != s) f |= FLAG_NAN;
     }
     return f;
 }
@@ -207,8 +209,9 @@ __device__ __forceinline__ void ceval(const V u[5], const V bb[3], V gamma, V gm
         if (!pos64(p)) k.hi |= FLAG_P;
         if ((__double2hiint(c.cf) & 0x7fffffff) > 0x7ff00000) k.hi |= FLAG_NAN;
     } else {
-        k.mn_rho = vminnan(k.mn_rho, rho);
-        k.mn_p = vminnan(k.mn_p, p);
+        k.mn_rho = vmin(k.mn_rho, rho);
+        k.mn_p = vmin(k.mn_p, p);
+        k.nsum = k.nsum + c.cf;
     }
 }
 

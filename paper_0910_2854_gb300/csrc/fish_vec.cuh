@@ -82,18 +82,8 @@ __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); 
 __device__ __forceinline__ float vmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ P2 vmax(P2 a, P2 b) { return {make_float2(fmaxf(a.v.x, b.v.x), fmaxf(a.v.y, b.v.y))}; }
 
-// minimum that keeps a NaN of either operand
-__device__ __forceinline__ float sminnan(float a, float b)
-{
-    float r;
-    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float vminnan(float a, float b) { return sminnan(a, b); }
-__device__ __forceinline__ P2 vminnan(P2 a, P2 b)
-{
-    return {make_float2(sminnan(a.v.x, b.v.x), sminnan(a.v.y, b.v.y))};
-}
+__device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ P2 vmin(P2 a, P2 b) { return {make_float2(fminf(a.v.x, b.v.x), fminf(a.v.y, b.v.y))}; }
 
 // reciprocal: IEEE in FP64, the hardware's (1 ulp) in FP32
 __device__ __forceinline__ float srcp(float a)

@@ -304,6 +304,34 @@ def test_nonphysical_state_reported(F):
     box.close()
 
 
+@pytest.mark.parametrize("dims", [(8, 6, 4), (7, 5, 4)])
+def test_nonphysical_state_named_fp32(F, dims):
+    """What the sweeps find is named by its kind: a density or pressure of zero
+    or less (a NaN is neither), and a fast speed that is none, here one whose
+    a^2 overflows while rho and p are positive."""
+    def flags(**values):
+        st = np.zeros((8,) + dims[::-1])
+        st[0], st[4], st[5] = 1.0, 1.0, 0.1
+        for k, v in values.items():
+            st[int(k[1:]), 2, 3, 4] = v
+        box = F.Box(*dims, 5.0 / 3.0, precision="fp32")
+        box.set_state(st)
+        box.fluid(0, 1e-35)
+        try:
+            box.sync()
+            return "none"
+        except F.FishError as e:
+            return str(e).split("flags ")[1].split(":")[0]
+        finally:
+            box.close()
+
+    assert flags() == "none"
+    assert flags(q0=-1.0) in ("0x1", "0x5")
+    assert flags(q4=-1.0) in ("0x2", "0x6")
+    assert flags(q0=np.nan) == "0x4"
+    assert flags(q0=1e-12, q4=1e30) == "0x4"
+
+
 def test_bad_arguments_rejected(F):
     with pytest.raises(F.FishError) as ei:
         F.Box(0, 4, 4, 5 / 3)
