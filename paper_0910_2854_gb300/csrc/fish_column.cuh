@@ -205,8 +205,8 @@ __device__ __forceinline__ void ceval(const V u[5], const V bb[3], V gamma, V gm
         c.F[4] = vfma(nb0, bv, (u[4] + ptot) * v0);
     }
     if constexpr (VT<V>::F64) {
-        if (!pos64(rho)) k.hi |= FLAG_RHO;
-        if (!pos64(p)) k.hi |= FLAG_P;
+        if (nonpos64(rho)) k.hi |= FLAG_RHO;
+        if (nonpos64(p)) k.hi |= FLAG_P;
         if ((__double2hiint(c.cf) & 0x7fffffff) > 0x7ff00000) k.hi |= FLAG_NAN;
     } else {
         k.mn_rho = vmin(k.mn_rho, rho);

@@ -140,6 +140,12 @@ __device__ __forceinline__ float vquot(float a, float b) { return vdiv(a, b); }
 __device__ __forceinline__ P2 vquot(P2 a, P2 b) { return vdiv(a, b); }
 // a > 0 by the bits (no FP64 pipe operation)
 __device__ __forceinline__ bool pos64(double a) { return __double_as_longlong(a) > 0; }
+// a <= 0 by the bits: a zero or the sign bit, and no NaN (beyond -infinity)
+__device__ __forceinline__ bool nonpos64(double a)
+{
+    const long long i = __double_as_longlong(a);
+    return i == 0 || i <= (long long)0xfff0000000000000ull;
+}
 
 // ---- limiters (eq0190 minmod, eq0200 Van Leer; sign(0) = 0, reading C-8) --
 

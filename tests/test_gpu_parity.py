@@ -304,8 +304,9 @@ def test_nonphysical_state_reported(F):
     box.close()
 
 
-@pytest.mark.parametrize("dims", [(8, 6, 4), (7, 5, 4)])
-def test_nonphysical_state_named_fp32(F, dims):
+@pytest.mark.parametrize("precision,dims", [("fp32", (8, 6, 4)), ("fp32", (7, 5, 4)), ("fp64", (8, 6, 4)),
+                                            ("fp64", (160, 128, 9))])
+def test_nonphysical_state_named(F, precision, dims):
     """What the sweeps find is named by its kind: a density or pressure of zero
     or less (a NaN is neither), and a fast speed that is none, here one whose
     a^2 overflows while rho and p are positive."""
@@ -314,9 +315,9 @@ def test_nonphysical_state_named_fp32(F, dims):
         st[0], st[4], st[5] = 1.0, 1.0, 0.1
         for k, v in values.items():
             st[int(k[1:]), 2, 3, 4] = v
-        box = F.Box(*dims, 5.0 / 3.0, precision="fp32")
+        box = F.Box(*dims, 5.0 / 3.0, precision=precision)
         box.set_state(st)
-        box.fluid(0, 1e-35)
+        box.fluid(0, 1e-35 if precision == "fp32" else 1e-305)
         try:
             box.sync()
             return "none"
@@ -329,7 +330,10 @@ def test_nonphysical_state_named_fp32(F, dims):
     assert flags(q0=-1.0) in ("0x1", "0x5")
     assert flags(q4=-1.0) in ("0x2", "0x6")
     assert flags(q0=np.nan) == "0x4"
-    assert flags(q0=1e-12, q4=1e30) == "0x4"
+    assert flags(q0=np.copysign(np.nan, -1.0)) == "0x4"
+    assert flags(q0=-0.0) in ("0x1", "0x3", "0x5", "0x7")
+    big = (1e-12, 1e30) if precision == "fp32" else (1e-20, 1e300)
+    assert flags(q0=big[0], q4=big[1]) == "0x4"
 
 
 def test_bad_arguments_rejected(F):
