@@ -82,19 +82,21 @@ __device__ __forceinline__ float narrow(double d, unsigned &odd)
 // in FP32 behind the FP64 pressure, with margins for the FP32 rounding: with
 // c^2 = a^2 + B^2, t = a^2 / c^2 and s = b_t^2 / (rho c^2),
 //   c_F^2 = c^2 (1 + sqrt((2 t - 1)^2 + 4 t s)) / 2.
-// Infinite where an operand is no normal FP32 number or zero, NaN included.
+// Infinite where an operand is no normal FP32 number or zero, NaN included, and
+// where the density or the pressure is not positive by far more than rounding:
+// the FP64 path, which such a cell then takes, finds whether they are.
 __device__ __forceinline__ float cfl_bound_f64(const double u[5], const double b[3], double gamma, double gm1,
-                                               const float rh[3], unsigned &flags)
+                                               const float rh[3])
 {
     const double ri = rcp64(u[0]);
     const double v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
     const double k2 = u[1] * v[0] + u[2] * v[1] + u[3] * v[2];
     const double b2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
-    const double p = gm1 * __fma_rn(-0.5, b2, __fma_rn(-0.5, k2, u[4]));
-    if (!pos64(u[0])) flags |= FLAG_RHO;
-    if (!pos64(p)) flags |= FLAG_P;
+    const double e = __fma_rn(-0.5, b2, __fma_rn(-0.5, k2, u[4]));
+    const double p = gm1 * e;
     const double g2 = gamma * p, s2 = g2 + b2;   // rho a^2, rho c^2
     unsigned odd = 0;
+    const bool sure = pos64(u[0]) && narrow(e, odd) > 1e-12f * narrow(u[4], odd);
     const float s2f = narrow(s2, odd), f2 = narrow(b2, odd);
     const float c2 = narrow(s2 * ri, odd), rs = __fdividef(1.0f, s2f), t = narrow(g2, odd) * rs;
     float r = 0.0f;
@@ -107,7 +109,8 @@ __device__ __forceinline__ float cfl_bound_f64(const double u[5], const double b
         r = fmaxf(r, (fabsf(narrow(v[d], odd)) + cf) * rh[d]);
     }
     // (b_n^2 against b^2 must not under- or overflow either)
-    return odd || !(s2f > 1e-30f && s2f < 1e30f && c2 > 1e-30f && r < 1e30f) ? __int_as_float(0x7f800000) : r * 1.00001f;
+    const bool ok = sure && !odd && s2f > 1e-30f && s2f < 1e30f && c2 > 1e-30f && r < 1e30f;
+    return ok ? r * 1.00001f : __int_as_float(0x7f800000);
 }
 
 // CFL minimum over the box: a warp per row along the fastest memory axis (no
@@ -190,7 +193,7 @@ __global__ void __launch_bounds__(256) cfl_kernel(CFLArgs<T> A)
             const T u0[5] = {__ldg(A.in[0] + idx), __ldg(A.in[1] + idx), __ldg(A.in[2] + idx), __ldg(A.in[3] + idx),
                              __ldg(A.in[4] + idx)};
             if constexpr (sizeof(T) == 8) {
-                const float bound = cfl_bound_f64(u0, bc, A.gamma, A.gm1, rh, flags);
+                const float bound = cfl_bound_f64(u0, bc, A.gamma, A.gm1, rh);
                 if (!(fbest > 1e-30f && bound < fbest)) {
                     // per axis in the paper's frame, the oracle's operation order
 #pragma unroll

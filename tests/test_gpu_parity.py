@@ -336,6 +336,41 @@ def test_nonphysical_state_named(F, precision, dims):
     assert flags(q0=big[0], q4=big[1]) == "0x4"
 
 
+def test_cfl_fp64_reports_what_its_own_pressure_is(F):
+    """The FP64 time step looks at most cells through a bound only; a cell
+    whose pressure is within rounding of zero is reported exactly when the
+    plain evaluation of eq0050 (in the frame of one of the axes) is not
+    positive."""
+    rng = np.random.RandomState(11)
+    st = np.zeros((8, 3, 4, 5))
+    st[0], st[4] = 1.0, 9.0
+    box = F.Box(5, 4, 3, 5.0 / 3.0, precision="fp64")
+    for _ in range(80):
+        rho, m, b = rng.uniform(0.5, 2.0), rng.uniform(-1.0, 1.0, 3), rng.uniform(-1.0, 1.0, 3)
+        st[5:] = b[:, None, None, None]
+        v = m / rho
+        kin, mag = [], []
+        for d in range(3):
+            a = [(d + k) % 3 for k in range(3)]
+            kin.append(0.5 * (m[a[0]] * v[a[0]] + m[a[1]] * v[a[1]] + m[a[2]] * v[a[2]]))
+            mag.append(0.5 * (b[a[0]] * b[a[0]] + b[a[1]] * b[a[1]] + b[a[2]] * b[a[2]]))
+        e0 = kin[0] + mag[0]
+        for k in range(-2, 3):
+            e = e0 + k * np.spacing(e0)
+            q = st.copy()
+            q[0, 1, 2, 3], q[1:4, 1, 2, 3], q[4, 1, 2, 3] = rho, m, e
+            box.set_state(q)
+            try:
+                box.cfl_dt(0.4)
+                got = False
+            except F.FishError as err:
+                assert err.code == F.FISH_ERR_NONPHYSICAL
+                got = True
+                box.clear_error()
+            assert got == any(e - kin[d] - mag[d] <= 0.0 for d in range(3)), (rho, m, b, k)
+    box.close()
+
+
 def test_bad_arguments_rejected(F):
     with pytest.raises(F.FishError) as ei:
         F.Box(0, 4, 4, 5 / 3)
