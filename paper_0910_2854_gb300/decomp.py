@@ -22,10 +22,13 @@ The CFL time step is the minimum over the ranks' own planes (an all-reduce).
 The host side here only moves planes and drives the box's operators; the
 arithmetic runs in the box (the CUDA library on a GPU).  The box needs:
 apply(op, d, dt), get_planes(k0, nk, out), set_planes(k0, nk, src),
-cfl_dt_planes(k, k0, nk) and sync(); the exchange uses torch.distributed
-(NCCL on GPUs, gloo on CPU) point-to-point messages.
+cfl_dt_planes(k, k0, nk) and sync(), and where it queues its work on a CUDA
+stream, that stream as `stream`; the exchange uses torch.distributed (NCCL on
+GPUs, gloo on CPU) point-to-point messages.
 """
 from __future__ import annotations
+
+import contextlib
 
 HALO = 4
 FLUID, CT = 0, 1
@@ -76,6 +79,16 @@ class SlabRun:
         self.exchanges = 0
 
     # -- ghost planes ---------------------------------------------------------
+    def _on_box_stream(self):
+        """The box's stream as torch's current one: the messages then come
+        after the planes the box has written and before those it reads,
+        whatever else the caller's stream holds."""
+        s = getattr(self.box, "stream", None)
+        if s is None:
+            return contextlib.nullcontext()
+        import torch
+        return torch.cuda.stream(s)
+
     def exchange(self):
         """Refill the ghost planes from the neighbours."""
         b, H, nk, lo, hi = self.box, HALO, self.nk, self.lo, self.hi
@@ -89,34 +102,38 @@ class SlabRun:
         if not hi_edge:
             b.get_planes(lo + nk - H, H, self._send_hi)
         b.sync()
+        below, above = self._recv_lo, self._recv_hi
         if self.world == 1:
-            if self.periodic:
-                self._recv_lo.copy_(self._send_hi)
-                self._recv_hi.copy_(self._send_lo)
+            # a single periodic rank is its own neighbour on both sides
+            below, above = self._send_hi, self._send_lo
         else:
-            # every rank posts: send up, receive from below, send down,
-            # receive from above.  Tags keep the two directions apart where a
-            # library matches by tag (gloo); where it matches in order (NCCL),
-            # the common posting order pairs them (with two ranks on a
-            # periodic ring both neighbours are the same rank).
-            d = self.dist
-            up, down = (self.rank + 1) % self.world, (self.rank - 1) % self.world
-            ops = []
-            if not hi_edge:
-                ops.append(d.P2POp(d.isend, self._send_hi, up, tag=1))
-            if not lo_edge:
-                ops.append(d.P2POp(d.irecv, self._recv_lo, down, tag=1))
-                ops.append(d.P2POp(d.isend, self._send_lo, down, tag=2))
-            if not hi_edge:
-                ops.append(d.P2POp(d.irecv, self._recv_hi, up, tag=2))
-            if ops:
-                for r in d.batch_isend_irecv(ops):
-                    r.wait()
+            with self._on_box_stream():
+                self._messages(lo_edge, hi_edge)
         if not lo_edge:
-            b.set_planes(0, H, self._recv_lo)
+            b.set_planes(0, H, below)
         if not hi_edge:
-            b.set_planes(lo + nk, H, self._recv_hi)
+            b.set_planes(lo + nk, H, above)
         self.exchanges += 1
+
+    def _messages(self, lo_edge, hi_edge):
+        # every rank posts: send up, receive from below, send down,
+        # receive from above.  Tags keep the two directions apart where a
+        # library matches by tag (gloo); where it matches in order (NCCL),
+        # the common posting order pairs them (with two ranks on a
+        # periodic ring both neighbours are the same rank).
+        d = self.dist
+        up, down = (self.rank + 1) % self.world, (self.rank - 1) % self.world
+        ops = []
+        if not hi_edge:
+            ops.append(d.P2POp(d.isend, self._send_hi, up, tag=1))
+        if not lo_edge:
+            ops.append(d.P2POp(d.irecv, self._recv_lo, down, tag=1))
+            ops.append(d.P2POp(d.isend, self._send_lo, down, tag=2))
+        if not hi_edge:
+            ops.append(d.P2POp(d.irecv, self._recv_hi, up, tag=2))
+        if ops:
+            for r in d.batch_isend_irecv(ops):
+                r.wait()
 
     # -- the method --------------------------------------------------------------
     def cfl_dt(self, k):

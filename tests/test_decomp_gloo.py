@@ -125,3 +125,59 @@ def test_slab_bounds_cover_the_box():
         assert spans[0][0] == 0 and sum(nk for _, nk in spans) == nz
         assert all(a[0] + a[1] == b[0] for a, b in zip(spans, spans[1:]))
         assert max(nk for _, nk in spans) - min(nk for _, nk in spans) <= 1
+
+
+@pytest.mark.parametrize("world", [1, 2])
+def test_exchange_stays_on_the_box_stream(monkeypatch, world):
+    """A CUDA box queues get_planes and set_planes on its own stream: what lies
+    between them is on that stream too, the messages with it as the current
+    one, and no copy on the caller's (a single rank's planes come straight from
+    the buffers they were read into)."""
+    import contextlib
+    import torch
+    from paper_0910_2854_gb300 import decomp
+    current, messages, planes = [None], [], {}
+
+    @contextlib.contextmanager
+    def use(stream):
+        old, current[0] = current[0], stream
+        yield
+        current[0] = old
+
+    class Request:
+        def wait(self):
+            messages.append(current[0])
+
+    class Dist:
+        isend, irecv = "isend", "irecv"
+
+        def P2POp(self, op, buf, peer, tag):
+            return op
+
+        def batch_isend_irecv(self, ops):
+            messages.append(current[0])
+            return [Request() for _ in ops]
+
+    class Box:
+        stream = "the box's stream"
+
+        def get_planes(self, k0, nk, out):
+            planes[k0] = out
+
+        def set_planes(self, k0, nk, src):
+            planes[-1 - k0] = src
+
+        def sync(self):
+            pass
+
+    monkeypatch.setattr(torch.cuda, "stream", use)
+    run = decomp.SlabRun(Box(), 2, 2, 8 * world, 0, world, True, dist=Dist(), device="cpu", dtype=torch.float64)
+    run.exchange()
+    H = decomp.HALO
+    if world == 1:
+        # ghosts below [0, H) take the top planes [lo + nk - H, ..), those above the lowest
+        assert planes[-1] is planes[run.lo + run.nk - H] and planes[-1 - run.lo - run.nk] is planes[run.lo]
+        assert messages == []
+    else:
+        assert messages == [Box.stream] * 5
+    assert current == [None]

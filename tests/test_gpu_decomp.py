@@ -57,6 +57,32 @@ def test_single_rank_slab_equals_single_box(F, precision):
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_slab_beside_other_work_on_the_current_stream(F, precision):
+    """The ghost exchange does not depend on when torch's current stream gets
+    to it: a step queued behind other work there gives the same bits."""
+    import torch
+    from paper_0910_2854_gb300.decomp import SlabRun, slab_extent
+    w = W.random_smooth(24, 20, 16, seed=15)
+    nx, ny, nz = w.dims
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    _, _, lo, hi = slab_extent(nz, 0, 1, True)
+    st = torch.as_tensor(np.concatenate([w.state[:, nz - lo:], w.state, w.state[:, :hi]], axis=1), device="cuda").to(dt)
+    out = []
+    for busy in (False, True):
+        box = F.Box(nx, ny, nz + lo + hi, w.gamma, bc=w.bc, precision=precision, h=w.h)
+        run = SlabRun(box, nx, ny, nz, 0, 1, True, device="cuda", dtype=dt)
+        box.set_state(st)
+        for _ in range(2):
+            if busy:
+                torch.cuda._sleep(50_000_000)  # (clocks: some 25 ms)
+            run.step_cfl(0.4, 1)
+        torch.cuda.synchronize()
+        out.append(box.get_state()[:, lo:lo + nz])
+        box.close()
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("dims", [(5, 3, 7), (8, 4, 6), (33, 1, 9)])
 def test_planes_to_device_host_and_unaligned_buffers(F, precision, dims):
     """Plane slabs through a device buffer (one kernel, 16-byte units or, from
