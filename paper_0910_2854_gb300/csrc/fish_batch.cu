@@ -360,7 +360,7 @@ public:
         for (auto &t : threads_) t.join();
     }
     // fn(i0, i1) over pieces of [0, n); returns when all are done.  One caller
-    // at a time (a batch is used by one thread).
+    // at a time (the batch's transfers take turns).
     void run(long long n, const std::function<void(long long, long long)> &fn)
     {
         const int want = (int)std::min<long long>(n / kShare, 8);
@@ -463,6 +463,7 @@ struct fish_batch {
     std::unique_ptr<float[]> paged[2];
     cudaEvent_t staged[2] = {};
     HostThreads host;
+    std::mutex transfer;          // the caller's threads may move several boxes at a time; the halves serve one
     bool tables = false;
     bool pending = false;         // minbits hold the CFL minima of the current states
     cudaGraphExec_t gexec = nullptr;
@@ -1002,6 +1003,7 @@ int fish_batch_set_state(fish_batch *b, int box, const double *state)
     int r = batch_ready(b);
     if (r) return r;
     if (box < 0 || box >= b->nbox || !state) return bfail(b, FISH_ERR_ARG, "bad box or state");
+    std::lock_guard<std::mutex> lock(b->transfer);
     if ((r = batch_layout(b, 0))) return r;
     const long long N = (long long)b->dims[3 * box] * b->dims[3 * box + 1] * b->dims[3 * box + 2];
     if ((r = batch_stage(b))) return r;
@@ -1034,6 +1036,7 @@ int fish_batch_get_state(fish_batch *b, int box, double *state)
     int r = batch_ready(b);
     if (r) return r;
     if (box < 0 || box >= b->nbox || !state) return bfail(b, FISH_ERR_ARG, "bad box or state");
+    std::lock_guard<std::mutex> lock(b->transfer);
     if ((r = batch_layout(b, 0))) return r;
     const long long N = (long long)b->dims[3 * box] * b->dims[3 * box + 1] * b->dims[3 * box + 2];
     if ((r = batch_stage(b))) return r;

@@ -136,6 +136,23 @@ def test_batch_segments_of_thin_and_long_boxes(F, bc):
     b.close()
 
 
+def test_batch_transfers_from_several_threads(F):
+    """Boxes handed over and fetched by several host threads at a time (a call
+    converts on threads and staging memory that the batch has once)."""
+    from concurrent.futures import ThreadPoolExecutor
+    dims = [(64, 48, 40), (32, 32, 32), (96, 64, 50), (16, 20, 8), (80, 40, 64), (64, 64, 64)]
+    b = F.Batch(dims, [1.4] * len(dims), [W.BC_PERIODIC] * len(dims))
+    with ThreadPoolExecutor(6) as pool:
+        for seed in range(3):
+            rng = np.random.RandomState(seed)
+            states = [rng.uniform(-1.0, 1.0, (8,) + d[::-1]).astype(np.float32) for d in dims]
+            list(pool.map(lambda k: b.set_state(k, states[k]), range(len(dims))))
+            got = list(pool.map(b.get_state, range(len(dims))))
+            for k in range(len(dims)):
+                assert np.array_equal(got[k], states[k]), (seed, k)
+    b.close()
+
+
 def test_batch_rejects_odd_paired_extents(F):
     with pytest.raises(F.FishError) as ei:
         F.Batch([(9, 8, 8)], [1.4], [0])
