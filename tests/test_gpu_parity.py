@@ -700,6 +700,56 @@ def test_sweep_segments(F, n, bc, precision):
 
 
 @pytest.mark.parametrize("bc", [W.BC_PERIODIC, W.BC_OUTFLOW])
+@pytest.mark.parametrize("limiter", ["vanleer", "minmod", "none", "hybrid"])
+@pytest.mark.parametrize("physics", ["plain", "unsplit", "split", "hse", "mesh", "mesh unsplit", "mesh hse"])
+def test_fp64_large_boxes_repeat_small_ones(F, physics, limiter, bc):
+    """A small FP64 box runs on a thread per cell, a large one marches its
+    columns in segments: a large box that repeats a small one (periodic: copies
+    of it side by side; open boundaries: more of the same rows across the sweep)
+    takes its values bit for bit, operator after operator.  The tests against
+    the oracle, on small boxes, so speak for the marches too."""
+    rng = np.random.RandomState(21)
+    if bc == W.BC_PERIODIC:
+        setups = [((32, 24, 20), (5, 6, 1), (0, 1, 2))]
+    else:
+        setups = [((32, 2, 20), (1, 200, 1), (0, 2)), ((2, 24, 20), (200, 1, 1), (1,))]
+    for dims, copies, axes in setups:
+        same = dims.index(2) if 2 in dims else None
+        shape = [1 if a == same else n for a, n in enumerate(dims)]
+        u = rng.random_sample((9, shape[2], shape[1], shape[0]))
+        u = np.broadcast_to(u, (9,) + dims[::-1]).copy()
+        u[0] = 1.0 + 0.25 * u[0]
+        u[1:4] = 0.5 * (u[1:4] - 0.5)
+        u[4] = 2.0 + 0.25 * u[4]
+        u[5:8] = 0.25 * (u[5:8] - 0.5)
+        width = [np.full(n, 0.1) if a == same else 0.1 + 0.05 * rng.random_sample(n) for a, n in enumerate(dims)]
+        boxes = []
+        for k in (1, 2):
+            c = copies if k == 2 else (1, 1, 1)
+            rep = lambda v: np.tile(v, (1,) * (v.ndim - 3) + c[::-1])  # noqa: E731
+            b = F.Box(*[n * m for n, m in zip(dims, c)], 5.0 / 3.0, bc=bc, precision="fp64",
+                      limiter=getattr(F, "FISH_LIM_" + limiter.upper()), hse="hse" in physics,
+                      gravity="split" if "split" in physics and "un" not in physics else "unsplit",
+                      h=(0.1, 0.11, 0.12))
+            b.set_state(rep(u[:8]))
+            if physics not in ("plain", "mesh"):
+                b.set_potential(rep(0.1 * u[8]))
+            if "mesh" in physics:
+                b.set_mesh([np.tile(w, m) for w, m in zip(width, c)])
+            boxes.append(b)
+        for d in axes:
+            for op in ("fluid", "ct"):
+                small, large = boxes
+                getattr(small, op)(d, 0.01)
+                getattr(large, op)(d, 0.01)
+                want = np.tile(small.get_state(), (1,) + copies[::-1])
+                assert np.isfinite(want).all()
+                assert np.array_equal(large.get_state(), want), (d, op)
+        for b in boxes:
+            b.close()
+
+
+@pytest.mark.parametrize("bc", [W.BC_PERIODIC, W.BC_OUTFLOW])
 @pytest.mark.parametrize("dims", [(160, 128, 1), (160, 128, 9), (31, 40, 37), (64, 62, 40)])
 def test_fp64_marches_beside_the_small_box_kernels(F, dims, bc):
     """FP64 boxes on both sides of the rule that takes a thread per cell for
