@@ -58,10 +58,21 @@ template <class T> static bool uses_pairs(const Frame &F, int lim, bool hse, boo
 
 // Output cells per tile of the FP64 thread-per-cell kernels for `groups` tiles
 // side by side and n cells along the sweep, or 0 where the column marches are
-// faster: as few cells as give at most one tile per SM, else TILE_MAX cells for
-// up to `most` tiles per SM.  L_d against the march: 12^3 (30 tiles) 29 against
-// 60 us, 32^3 (128) 49 / 78, 72 x 60 x 51 (920) 295 / 277; B_d: 12^3 16 / 31,
-// 32^3 (256) 39 / 43, 72 x 60 x 51 (1080) 122 / 85.
+// faster (the results are bitwise the same): as few cells as give at most one
+// tile per SM, else TILE_MAX cells for up to `most` tiles per SM, each SM's
+// tiles one after the other while a march fills the SMs evenly.  Tiles against
+// marches, us, boxes of 16 to 96 cells along the sweep:
+//   L_d                        100 tiles    300     400    500    600
+//     plain, Van Leer           39 /  68   90/104 131/131 174/146 174/160
+//     unsplit, split potential  42 /  81   98/121 146/151 193/168 193/185
+//                               45 /  92  103/135 152/168 202/189 203/205
+//     hydrostatic correction    60 / 111  144/164 215/203 285/229 285/250
+//     irregular mesh            53 /  95  125/149 186/190 246/216 247/240
+//   B_d                        100 tiles    300     350    450    600
+//     uniform mesh              17 /  31   35/ 41  51/ 45  51/ 47  68/ 55
+//     irregular mesh            27 /  57   57/ 78  86/ 86  86/ 94 112/113
+// so `most` is 2, and 3 where a potential alone or, for B_d, an irregular mesh
+// makes the march slower.
 static inline int tile_cells(long long groups, int n, int most)
 {
     const int sms = sm_count();
@@ -126,7 +137,7 @@ cudaError_t Launch<T>::fluid(const T *const in[8], T *const out[5], const T *phi
     A.wd = w3 ? w3[d] : nullptr;
     A.sg = split_gravity ? 1 : 0;
     if constexpr (sizeof(T) == 8) {
-        const int len = tile_cells(((long long)F.nf * F.no + 31) / 32, F.n, 4);
+        const int len = tile_cells(((long long)F.nf * F.no + 31) / 32, F.n, A.phi && !hse ? 3 : 2);
         if (len) return tile_fluid(A, hse, F.ft1, len, s);
         return col_fluid<double>(A, hse, F.ft1, s);
     } else {
@@ -182,7 +193,7 @@ cudaError_t Launch<T>::ct(const T *rho, const T *md, const T *const b[3], T *con
         A.wo = w3[F.other];
     }
     if constexpr (sizeof(T) == 8) {
-        const int len = tile_cells((long long)((F.nf + 30) / 31) * F.no, F.n, 2);
+        const int len = tile_cells((long long)((F.nf + 30) / 31) * F.no, F.n, w3 ? 3 : 2);
         if (len) return tile_ct(A, F.ft1, len, s);
         return col_ct<double>(A, F.ft1, s);
     } else {
