@@ -136,6 +136,36 @@ def test_batch_segments_of_thin_and_long_boxes(F, bc):
     b.close()
 
 
+@pytest.mark.parametrize("limiter", ["vanleer", "minmod"])
+def test_batch_is_the_single_boxes_bit_for_bit(F, limiter):
+    """Over twenty steps each box of a batch stays bitwise the single box of
+    the same cells (another segment length, another launch), and the batch,
+    stepped once more from the same states after another batch, itself."""
+    lim = getattr(F, "FISH_LIM_" + limiter.upper())
+    ws = [W.batch_box("sod", (64, 32, 36), 0), W.batch_box("brio_wu", (34, 66, 32), 1), W.blast(48, 40, 56),
+          W.random_smooth(32, 20, 9, seed=97, bc=W.BC_OUTFLOW), W.random_smooth(30, 64, 34, seed=98)]
+    b = F.Batch([w.dims for w in ws], [w.gamma for w in ws], [w.bc for w in ws], [w.h for w in ws], limiter=lim)
+    other = make_batch(F, ws[::-1])
+    runs = []
+    for _ in range(2):
+        for k, w in enumerate(ws):
+            b.set_state(k, w.state)
+        b.step(0.4, 20)
+        other.step(0.4, 1)
+        runs.append([b.get_state(k) for k in range(len(ws))])
+    dts = b.last_dt()
+    for k, w in enumerate(ws):
+        assert np.array_equal(runs[0][k], runs[1][k]), k
+        box = F.Box(*w.dims, w.gamma, bc=w.bc, precision="fp32", h=w.h, limiter=lim)
+        box.set_state(w.state)
+        box.step_cfl(0.4, 20)
+        assert box.last_dt() == dts[k], k
+        assert np.array_equal(runs[0][k], box.get_state()), k
+        box.close()
+    b.close()
+    other.close()
+
+
 def test_batch_transfers_from_several_threads(F):
     """Boxes handed over and fetched by several host threads at a time (a call
     converts on threads and staging memory that the batch has once)."""

@@ -91,6 +91,8 @@ BOX_DIGESTS = {
 
 @pytest.fixture(scope="module")
 def F():
+    from paper_0910_2854_gb300 import build
+    build.build()
     import paper_0910_2854_gb300 as F
     return F
 
