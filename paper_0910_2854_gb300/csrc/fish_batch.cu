@@ -193,8 +193,8 @@ __global__ void __launch_bounds__(32 * ROWS, FISH_CT_MINB * 4 / ROWS)
         for (int g = 0; g < groups; ++g) {
             const long long q = (long long)first / ROWS + g;
             const long long ob = (q / nseg) * ROWS + (threadIdx.x >> 5);
-            ct_columns<float, LIM, true, false, IX>(Ab, ob * nseg + q % nseg, threadIdx.x & 31, I.a, I.b,
-                                                      threadIdx.x < 32, threadIdx.x >= 32 * (ROWS - 1));
+            ct_columns<float, LIM, true, false, IX, false>(Ab, ob * nseg + q % nseg, threadIdx.x & 31, I.a, I.b,
+                                                           threadIdx.x < 32, threadIdx.x >= 32 * (ROWS - 1));
         }
     }
 }

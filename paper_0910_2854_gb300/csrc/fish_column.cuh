@@ -930,8 +930,8 @@ __device__ __forceinline__ void fluid_columns(const AR &A, long long cid, int a,
 
 // Threads of a block.  FP64 is bound by the FP64 pipe of each SM quarter,
 // which one warp nearly fills, so its blocks are single warps that spread
-// evenly (32^3, 256 warps: 136 us per L_d with one-warp blocks, 151 us with
-// four-warp blocks, 719 us with the columns uncut).
+// evenly (L_x of 72 x 60 x 51 cells: 215 us with one-warp blocks, 248 us with
+// four-warp blocks, 942 us with the columns uncut).
 template <class V> constexpr int fluid_threads() { return VT<V>::F64 ? 32 : 128; }
 // Blocks per SM the kernels are compiled for.
 template <class V, bool HSE> constexpr int fluid_resident()
@@ -1220,8 +1220,11 @@ template <class V> __device__ __forceinline__ V shfl_up1(V a)
 // - the lower other-axis pencil takes its newest product unrounded in the
 //   difference formed at cell `fin` (a cell no march reaches if there is none).
 // The loop has a copy of its steps for the cells in the middle, where only the
-// first holds: 139.1 -> 139.6 us at 256^3 and 1964 -> 1978 us at 640^3 against
+// first holds: 137.3 -> 139.2 us at 256^3 and 1954 -> 1969 us at 640^3 against
 // one form for all cells, 142.2 and 2008 us with the choice made in each step.
+// A batch, whose short marches take both copies in most work items, makes the
+// choice in each step: 808 us per double step of 12 boxes of 32 to 96 cells,
+// 817 us with the copy, 799 us with one form.
 __device__ __forceinline__ void ct_rounding(int n, int &fused, int &fin)
 {
     fused = n >= 8 ? (n - 1) / 4 * 4 : 0;
@@ -1351,7 +1354,8 @@ __device__ __forceinline__ void ctstep(const AR &A, const CTCtx<typename VT<V>::
 // own repeat a valid column and store nothing.
 // The march of warp gw (31 W columns of one row) of the box described by A
 // over the output cells a .. b-1.
-template <class V, int LIM, bool FT1, bool NU = false, class IX = long long, class AR>
+// COPY: with a copy of the steps for the cells in the middle (see ct_rounding)
+template <class V, int LIM, bool FT1, bool NU = false, class IX = long long, bool COPY = true, class AR>
 __device__ __forceinline__ void ct_columns(const AR &A, long long gw, int lane, int a, int b,
                                            bool edge_lo, bool edge_hi)
 {
@@ -1434,7 +1438,7 @@ __device__ __forceinline__ void ct_columns(const AR &A, long long gw, int lane, 
     };
 #pragma unroll 1
     for (int s = a - 4;; s += 4) {
-        if (!ct_packs<V, NU>() || (s >= 0 && s + 3 < X.fused)) {
+        if (!ct_packs<V, NU>() || (COPY && s >= 0 && s + 3 < X.fused)) {
             if (four(std::true_type{}, s)) break;
         } else {
             if (four(std::false_type{}, s)) break;
