@@ -318,7 +318,7 @@ TRAFFIC_B_PER_CELL = {"fluid": 52.2, "ct": 34.1}
 # 256^3 box.  The FP64 path
 # is bound by GB300's FP64 pipe, so its roofline is this rate against the
 # probed FMA rate of the device (fish_probe_fp64_fma).
-FP64_OPS_PER_CELL = {"fluid": 383, "ct": 110}
+FP64_OPS_PER_CELL = {"fluid": 383, "ct": 109}
 
 
 def traffic_per_cell(kernel_key):

@@ -105,8 +105,9 @@ int fish_set_option(fish_ctx *ctx, int key, double value);
 int fish_set_stream(fish_ctx *ctx, void *cuda_stream);
 
 /* Route the context's device allocations through a caller allocator (e.g.
- * PyTorch's caching allocator): alloc(size, user) returns a device pointer or
- * NULL, free(ptr, user) releases it.  Must be called before the first
+ * PyTorch's caching allocator): alloc(size, user) returns a device pointer
+ * (8-byte aligned at least: the FP32 sweeps load pairs) or NULL, free(ptr,
+ * user) releases it.  Must be called before the first
  * fish_set_state*.  NULL alloc restores cudaMalloc/cudaFree. */
 int fish_set_allocator(fish_ctx *ctx, void *(*alloc)(size_t size, void *user),
                        void (*free_fn)(void *ptr, void *user), void *user);
@@ -252,7 +253,11 @@ int fish_batch_create(int nbox, const int *dims, const double *gamma, const int 
 int fish_batch_set_option(fish_batch *b, int key, double value);
 /* queue all further work on this CUDA stream (NULL: the batch's own) */
 int fish_batch_set_stream(fish_batch *b, void *cuda_stream);
-/* upload box `box` from a host buffer of 8*nx*ny*nz doubles; synchronous */
+/* upload box `box` from a host buffer of 8*nx*ny*nz doubles; synchronous.
+ * Uploads and downloads convert on up to eight host threads and stage in 16 MB
+ * of pinned host memory (pageable where none is granted); both belong to the
+ * batch from its first transfer to its destruction.  Several host threads may
+ * transfer boxes of one batch at a time; the calls take turns. */
 int fish_batch_set_state(fish_batch *b, int box, const double *state);
 /* nsteps double steps of every box, each with dt = k * CFL of that box's
  * state at the start of the step, computed on the device.  Asynchronous. */

@@ -28,9 +28,10 @@ template <class A_> static bool fits_u32(const A_ &A)
 //   waves(blocks S) (ceil(n / S) + extra),
 // a last wave of at most `lone` blocks counting `lone_cost` of a full one.
 // Measured against every S from 1 to 64 on boxes from 32^3 to 1024^2 x 512:
-// within 3 % of the best S, e.g. L_d 95 -> 45 us at 128^3 (FP32, 4
-// segments), 666 -> 110 us at 32^3 (FP64, 16), 19.7 -> 17.6 ms at 256^3
-// (FP64, 2: less of the last wave idle), 2.95 -> 2.85 ms at 640^3 (FP32, 3).
+// within 3 % of the best S.  L_d uncut and cut: 79 -> 36 us at 128^3 (FP32, four
+// segments), 942 -> 215 us for the x sweep of 72 x 60 x 51 cells (FP64, six),
+// 13.9 -> 12.4 ms at 256^3 (FP64, two: less of the last wave idle), 2.67 ->
+// 2.52 ms at 640^3 (FP32, three).
 static inline int col_segments(int n, long long blocks, int slots, int lone, double lone_cost, int extra)
 {
     double best = 1e300;

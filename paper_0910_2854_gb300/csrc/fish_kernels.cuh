@@ -388,7 +388,6 @@ template <class T> struct TransArgs {
 #ifndef FISH_TR_ROWS
 #define FISH_TR_ROWS 64
 #endif
-// tile height: FP64 tiles stay within the 48 KB of static shared memory
 // FP32 transpose with 16-byte accesses: tiles of 64 x 64 elements, each
 // thread moves four float4 of a field per tile (source rows of 256 bytes
 // read whole, destination rows of 256 bytes written whole), the next
@@ -447,6 +446,7 @@ __global__ void __launch_bounds__(256) transpose4_kernel(TransArgs<T> A)
     }
 }
 
+// tile height: FP64 tiles stay within the 48 KB of static shared memory
 template <class T> constexpr int tr_rows() { return sizeof(T) == 8 && FISH_TR_ROWS > 64 ? 64 : FISH_TR_ROWS; }
 template <class T>
 __global__ void __launch_bounds__(256) transpose_kernel(TransArgs<T> A)

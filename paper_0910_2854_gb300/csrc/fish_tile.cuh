@@ -10,9 +10,9 @@
 // neighbours through shared memory in four rounds.  The arithmetic is the
 // marches' own (ceval, cflux1, cflux2, the kicks, cface's formulas), so results
 // are bitwise theirs.  Bound by the FP64 pipe: a tile of eight cells does 1.4
-// times the operations of eight cells.  L_d 60 -> 29 us at 12^3 and 78 -> 49 us
-// at 32^3, B_d 31 -> 16 and 43 -> 39 us; FP32 gains nothing (10.3 us either way
-// at 32^3, most of it launches).
+// times the operations of eight cells.  The times of both stand beside the rule
+// that chooses (tile_cells in fish_launch.cuh); FP32 gains nothing (10.3 us
+// either way at 32^3, most of it launches).
 #pragma once
 
 #include "fish_column.cuh"

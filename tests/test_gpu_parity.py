@@ -668,10 +668,11 @@ def test_turbulence_twin_128():
 @pytest.mark.parametrize("bc", [W.BC_PERIODIC, W.BC_OUTFLOW])
 @pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 9, 16, 33])
 def test_sweep_segments(F, n, bc, precision):
-    """A sweep over few columns is cut into segments of one or two cells,
-    whose windows reach over the boundary and over neighbouring segments:
-    every operator along the axis of n cells (thinner than the stencil, odd,
-    and longer than several segments), plain and with each potential form."""
+    """A sweep over few columns is cut into segments of one or two cells
+    (FP32), or into tiles of two cells of a thread each (FP64), whose windows
+    reach over the boundary and over their neighbours: every operator along the
+    axis of n cells (thinner than the stencil, odd, and longer than several
+    segments), plain and with each potential form."""
     for d in range(3):
         dims = [6, 5, 4]
         dims[d] = n
