@@ -463,7 +463,7 @@ struct fish_batch {
     std::unique_ptr<float[]> paged[2];
     cudaEvent_t staged[2] = {};
     HostThreads host;
-    std::mutex transfer;          // the caller's threads may move several boxes at a time; the halves serve one
+    std::mutex transfer;          // transfers from several host threads: one at a time uses tables, layout and halves
     bool tables = false;
     bool pending = false;         // minbits hold the CFL minima of the current states
     cudaGraphExec_t gexec = nullptr;
@@ -1000,10 +1000,11 @@ int fish_batch_set_stream(fish_batch *b, void *stream)
 
 int fish_batch_set_state(fish_batch *b, int box, const double *state)
 {
+    if (!b) return FISH_ERR_ARG;
+    std::lock_guard<std::mutex> lock(b->transfer);
     int r = batch_ready(b);
     if (r) return r;
     if (box < 0 || box >= b->nbox || !state) return bfail(b, FISH_ERR_ARG, "bad box or state");
-    std::lock_guard<std::mutex> lock(b->transfer);
     if ((r = batch_layout(b, 0))) return r;
     const long long N = (long long)b->dims[3 * box] * b->dims[3 * box + 1] * b->dims[3 * box + 2];
     if ((r = batch_stage(b))) return r;
@@ -1033,10 +1034,11 @@ int fish_batch_set_state(fish_batch *b, int box, const double *state)
 
 int fish_batch_get_state(fish_batch *b, int box, double *state)
 {
+    if (!b) return FISH_ERR_ARG;
+    std::lock_guard<std::mutex> lock(b->transfer);
     int r = batch_ready(b);
     if (r) return r;
     if (box < 0 || box >= b->nbox || !state) return bfail(b, FISH_ERR_ARG, "bad box or state");
-    std::lock_guard<std::mutex> lock(b->transfer);
     if ((r = batch_layout(b, 0))) return r;
     const long long N = (long long)b->dims[3 * box] * b->dims[3 * box + 1] * b->dims[3 * box + 2];
     if ((r = batch_stage(b))) return r;
